@@ -79,7 +79,7 @@ typedef struct {
     int32_t max_rounds;  /* resolve round limit, 0 = default (256)                   */
     int32_t flags;       /* SIDM_FLAG_*                                              */
     int32_t grid_ctas;   /* persistent CTAs per kernel, 0 = SM count x occupancy     */
-    int32_t use_tma;     /* 1: stage candidate tiles with bulk async copies (TMA)    */
+    int32_t use_tma;     /* 1: bulk async copies (TMA) stage candidates in the kernels that have that path */
     /* launch knobs of the hot kernels; none changes a result (0 = default) */
     int32_t knn_groups;  /* kernel-size search: lane groups of the candidate mask,   */
                          /*   2, 4 or 8 (default 2; plain-load path)                 */
@@ -88,7 +88,7 @@ typedef struct {
     int32_t knn_flush;   /*   pending keys per lane that trigger a heap merge before */
                          /*   a tree node's tests, 1..32 (default 32)                */
     float   knn_slack;   /*   warm-start bound / previous kernel size, 1..2 (1.07)   */
-    int32_t pair_per_round; /* pair kernel: pairs a lane queues per round, 1..4 (4; mixed-form draws) */
+    int32_t pair_per_round; /* pair kernel: groups of 32 pairs drawn together, 1..4 (2; plain draws) */
     int32_t knn_batch;   /* kernel-size search: 1 loops over each staged leaf's      */
                          /*   candidates, 2 over compacted batches of them, 3 as 2    */
                          /*   with warm-started searches in the fixed-bound kernel    */

@@ -1303,7 +1303,7 @@ static void free_all(sidm_ctx* c)
                     c->d_chunk_halo, c->d_chunk_begin, c->d_frame, c->d_key, c->d_key2, c->d_val, c->d_val2,
                     c->d_sort_status, c->d_sort_hist, c->d_P4, c->d_V4, c->d_ID, c->d_cell, c->d_cellb, c->d_nlo, c->d_nhi, c->d_perm, c->d_tmp_pos,
                     c->d_tmp_vel, c->d_tmp_id, c->d_claim, c->d_hits, c->d_done, c->d_ev, c->d_sump,
-                    c->d_stats_own, c->d_cnt, c->d_epart, c->d_chunk_off, c->d_group_off, c->d_gpart, c->d_lam, c->d_hprev, c->d_dacc, c->d_halo_ord,
+                    c->d_stats_own, c->d_cnt, c->d_epart, c->d_chunk_off, c->d_group_off, c->d_gpart, c->d_lam, c->d_lam4, c->d_hprev, c->d_dacc, c->d_halo_ord,
                     c->d_evg, c->d_lkey, c->d_lval, c->d_lstart, c->d_llen, c->d_lptr, c->d_lact,
                     c->d_lcnt};
     for (void* p : ptrs) if (p) cudaFree(p);
@@ -1445,6 +1445,16 @@ extern "C" int sidm_create(sidm_ctx** out, const sidm_config* cfg)
         std::vector<float> Tf(T.begin(), T.end());
         e = cudaMalloc(&c->d_lam, Tf.size() * 4); if (e != cudaSuccess) return fail("cudaMalloc lam", e);
         e = cudaMemcpy(c->d_lam, Tf.data(), Tf.size() * 4, cudaMemcpyHostToDevice);
+        if (e == cudaSuccess && (cfg->flags & (SIDM_FLAG_SUM_P | SIDM_FLAG_DRAG))) {
+            std::vector<float4> T4(Tf.size(), make_float4(0.f, 0.f, 0.f, 0.f));
+            for (int r = 0; r < kLamNR; ++r)
+                for (int x = 0; x + 3 < kLamNX; ++x) {
+                    const float* t = Tf.data() + (size_t)r * kLamNX + x;
+                    T4[(size_t)r * kLamNX + x] = make_float4(t[0], t[1], t[2], t[3]);
+                }
+            e = cudaMalloc((void**)&c->d_lam4, T4.size() * sizeof(float4)); if (e != cudaSuccess) return fail("cudaMalloc lam4", e);
+            e = cudaMemcpy(c->d_lam4, T4.data(), T4.size() * sizeof(float4), cudaMemcpyHostToDevice);
+        }
     }
     if (e != cudaSuccess) return fail("cudaMemcpy lam", e);
     e = cudaMemset(c->d_hits, 0, sizeof(uint32_t) * (size_t)N); if (e != cudaSuccess) return fail("memset", e);
@@ -1783,10 +1793,10 @@ static int scatter_impl(sidm_ctx* c, uint64_t seed, uint64_t step, const sidm_xs
     if (fp64)
         SIDM_LAUNCH(c, k_vel_refresh<double><<<grid_for(c, L.N, 256), 256, 0, s>>>(L.N, L.H, c->d_halo_off, c->d_halo_pad,
                                                                                   (const double*)vel, c->d_ID, (double4_16a*)c->d_V4));
-    else
+    else if (c->cfg.flags & (SIDM_FLAG_SUM_P | SIDM_FLAG_DRAG))   // plain draws read a few velocities only
         SIDM_LAUNCH(c, k_vel_refresh<float><<<grid_for(c, L.N, 256), 256, 0, s>>>(L.N, L.H, c->d_halo_off, c->d_halo_pad,
                                                                                 (const float*)vel, c->d_ID, (float4*)c->d_V4));
-    int rc = launch_pairs(c, seed, step, xs, dt, mass, st, s);
+    int rc = launch_pairs(c, seed, step, xs, dt, mass, vel, st, s);
     if (rc) return rc;
     const int use_sump = (c->cfg.flags & SIDM_FLAG_SUM_P) ? 1 : 0;
     if (c->cfg.flags & SIDM_FLAG_DRAG)

@@ -43,6 +43,7 @@ struct DevCounters {
     unsigned long long ev_count;     // events drawn this step
     unsigned long long de_lo;        // 128-bit fixed-point sum of pair dE (2^-80 units)
     unsigned long long de_hi;
+    unsigned int vmax[kMaxHalos];    // bits of the largest speed per halo (FP32, >= 0; halos of constant cross-section)
     unsigned int work[4];            // persistent work-queue counters; [2], [3]: grid barrier
     unsigned int status;             // sticky SIDM_DEV_* bits (cleared by sidm_status)
     unsigned int pad;
@@ -167,6 +168,7 @@ struct sidm_ctx {
 
     // Lambda table (float or double [kLamNR][kLamNX])
     void* d_lam = nullptr;
+    float4* d_lam4 = nullptr;          // mixed form with per-pair lookups: (f[x], .., f[x + 3]) per entry
 
     int knn_grid = 0, pair_grid = 0, knn_warps = 4, pair_warps = 4;
 
@@ -202,7 +204,7 @@ int occupancy(sidm_ctx* c, const void* fn, int threads, size_t smem, int* occ);
 // kernel entry points implemented in the other translation units
 int launch_knn(sidm_ctx* c, void* h_out, uint32_t* nbr, int k_stride, bool use_guess, cudaStream_t s);
 int launch_pairs(sidm_ctx* c, uint64_t seed, uint64_t step, const sidm_xs* xs, const double* dt,
-                 const double* mass, sidm_step_stats* st, cudaStream_t s);
+                 const double* mass, const void* vel, sidm_step_stats* st, cudaStream_t s);
 int launch_pairs_diag(sidm_ctx* c, const sidm_xs* xs, const double* mass, cudaStream_t s);
 
 // ---------------------------------------------------------------- device helpers
@@ -312,29 +314,56 @@ __device__ __forceinline__ R lambda_lookup(const R* __restrict__ T, R d, R hi, R
     return lambda_f<R>(T, d, hi, hj) * inv * inv * inv;
 }
 
-// FP32 interpolated f with approximate reciprocals (relative error ~1e-7,
+// Stencil of the FP32 interpolation at (d; hi, hj): first node and Lagrange
+// weights along x and rho, with approximate reciprocals (relative error ~1e-7,
 // far below the table's own 1e-6 of the peak); inv = 1/h_max from the caller.
-__device__ __forceinline__ float lambda_f_fast(const float* __restrict__ T, float d, float hi, float hj, float inv)
+// False beyond the support.
+__device__ __forceinline__ bool lambda_stencil(float d, float hi, float hj, float inv, int& ix, int& ir, float wx[4], float wr[4])
 {
     const float hmin = fminf(hi, hj);
     float x = __fdividef(d, hi + hj);
-    if (!(x < 1.f)) return 0.f;
+    if (!(x < 1.f)) return false;
     x = fmaxf(x, 0.f);
     const float rho = hmin * inv;
     const float gx = x * (float)(kLamNX - 1);
-    int ix = (int)floorf(gx) - 1;
+    ix = (int)floorf(gx) - 1;
     ix = ix < 0 ? 0 : (ix > kLamNX - 4 ? kLamNX - 4 : ix);
     const float gr = rho * (float)(kLamNR - 1);
-    int ir = (int)floorf(gr) - 1;
+    ir = (int)floorf(gr) - 1;
     ir = ir < 0 ? 0 : (ir > kLamNR - 4 ? kLamNR - 4 : ir);
-    float wx[4], wr[4];
     lagrange4<float>(gx - (float)ix, wx);
     lagrange4<float>(gr - (float)ir, wr);
+    return true;
+}
+
+// FP32 interpolated f, from the table
+__device__ __forceinline__ float lambda_f_fast(const float* __restrict__ T, float d, float hi, float hj, float inv)
+{
+    int ix, ir;
+    float wx[4], wr[4];
+    if (!lambda_stencil(d, hi, hj, inv, ix, ir, wx, wr)) return 0.f;
     float f = 0.f;
 #pragma unroll
     for (int a = 0; a < 4; ++a) {
         const float* row = T + (ir + a) * kLamNX + ix;
         f = fmaf(wr[a], wx[0] * __ldg(row) + wx[1] * __ldg(row + 1) + wx[2] * __ldg(row + 2) + wx[3] * __ldg(row + 3), f);
+    }
+    return f;
+}
+
+// The same sums from the table stored as groups of four along x: one 16-byte
+// load per row.  A warp's lanes hit different lines, so its loads cost one pass
+// per lane and load, not per byte.
+__device__ __forceinline__ float lambda_f_rows(const float4* __restrict__ T4, float d, float hi, float hj, float inv)
+{
+    int ix, ir;
+    float wx[4], wr[4];
+    if (!lambda_stencil(d, hi, hj, inv, ix, ir, wx, wr)) return 0.f;
+    float f = 0.f;
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+        const float4 r = __ldg(T4 + (ir + a) * kLamNX + ix);
+        f = fmaf(wr[a], wx[0] * r.x + wx[1] * r.y + wx[2] * r.z + wx[3] * r.w, f);
     }
     return f;
 }

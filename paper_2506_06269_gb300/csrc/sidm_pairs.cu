@@ -35,7 +35,11 @@ struct PairParams {
     const float4* nhi;
     const void* P4;
     const void* V4;
+    const uint32_t* ID;
+    const void* vel;    // the caller's velocities [3][N] (unchanged until the resolve)
+    int64_t N;
     const void* lam;
+    const float4* lam4; // the mixed form's table as groups of four along x (contexts that look up every pair)
     const sidm_xs* xs;
     const double* dt;
     const double* mass;
@@ -48,6 +52,7 @@ struct PairParams {
     unsigned long long ev_cap;
     float* sump;
     int use_sump;
+    int parts;          // warps that share a query leaf's candidate leaves (a power of two)
     double* dacc;       // local diagnostics: [5][nacc] kernel-weighted moments
     int64_t nacc;
     DevCounters* cnt;
@@ -76,7 +81,7 @@ __device__ __forceinline__ R spline_w(R d, R h)
 // pairs a lane queues per round, at most (a launch knob; swept on the GB300:
 // 1, 2, 3, 4 -> 3.76, 3.64, 3.49, 3.47 ms), and the queue entries per warp, a
 // power of two: a round adds up to 32 kPerRoundMax pairs to fewer than 32 waiting
-constexpr int kPerRoundMax = 4;
+constexpr int kPerRoundMax = 4, kPerRoundDefault = 2;
 constexpr int kQueue = 32 * (kPerRoundMax + 1) <= 64 ? 64 : 32 * (kPerRoundMax + 1) <= 128 ? 128 : 256;
 static_assert(kQueue >= 32 * (kPerRoundMax + 1), "one round must fit behind the entries still waiting");
 
@@ -122,7 +127,7 @@ constexpr size_t pair_warp_bytes()
 // that would have been formed, so a draw u >= P_up + 2e-6 decides "no event"
 // and "not within 1e-6 of P" exactly as the full evaluation would.
 template <class R, bool TMA, int MODE, int PR, bool DRAG>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_pairs(PairParams p)
+__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_pairs_queue(PairParams p)
 {
     static_assert(PR >= 1 && PR <= kPerRoundMax, "pairs per round");
     using V = typename Vec4<R>::T;
@@ -585,16 +590,629 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_pairs(PairParam
     st_pos.finish(lane, p.cnt);
 }
 
-template <class R, bool TMA, int MODE, int PR = kPerRoundMax, bool DRAG = false>
-int launch_t(sidm_ctx* c, uint64_t seed, uint64_t step, const sidm_xs* xs, const double* dt, const double* mass,
-             sidm_step_stats* st, cudaStream_t s)
+// ---------------------------------------------------------------- draws, mixed form
+// Most in-range pairs never come near an event (P ~ 1e-6 .. 1e-4), and whether
+// a draw can fire at all is decided by integers: P_ij <= T 2^-32 for every pair
+// of a query leaf, with T from the largest sigma(v) v and Lambda <= 4 / h_i^3
+// (kLamFUp), so a pair needs the two ids and Philox word 0 only; the few pairs
+// with x0 <= T take the full evaluation (velocities, P, event).  One warp per
+// query leaf, one query per lane:
+//  * the tree is walked with the box of the queries and their largest h (one box
+//    test per child, a lane each); accepted leaves are listed and loaded two at
+//    a time;
+//  * a listed leaf's candidates are kept if they come within h_j + the largest
+//    h of the queries' box (tested in the query leaf's own frame, where the gap
+//    rounded down bounds the canonical distance from below) and go to a ring;
+//  * batches of kPBatch ring entries are tested against all 32 queries, two
+//    candidates per packed FP32 operation, into one bit mask per lane;
+//  * one warp scan of the masks' bit counts per batch gives every lane its place
+//    in the warp's queue of (query lane, candidate) pairs, which is emptied 32
+//    pairs at a time, all lanes busy.
+// Issue-bound (2.8 of 4 instructions per cycle): 1.94 ms per launch for the 2^20
+// NFW halo at N_ngb = 64 (3.28 ms before), 2.65e8 in-range pairs, 1.24e9 tests.
+// Filling the queue in rounds of ballots and forming sigma(v) and
+// a bound of P for every pair, with masked tests, took 331 lane instructions
+// per in-range pair (52 % of them queueing and masks); a queue per lane, without
+// the scan, left 54 % of the lanes idle in the draws (a leaf's partners lie
+// after it in Morton order, and their number varies over its lanes).  Walk boxes
+// of 2, 4 and 8 lane groups (1.97, 2.00, 2.07 ms), batches of 8 (2.19), runs of
+// width 2, 2.5 and 4 (2.11, 1.95, 1.97), 1 and 3 groups of 32 pairs drawn together
+// (2.10, 1.99 against 1.94 for 2) and 64 registers (2.17) were slower.
+constexpr int kPBatch = 16;     // candidates per batch (batches start at multiples of it: never wrap)
+constexpr int kPRing = 128;     // candidate ring entries (x, y, z and h apart)
+constexpr int kPCand = 256;     // candidates whose ids and slots are kept for queued pairs
+constexpr int kPQueue = 32 * (kPBatch + kPerRoundMax);   // queued pairs: a batch behind less than one draw's
+constexpr int kPList = 64;      // accepted leaves listed before they are streamed
+constexpr float kPSpread = 3.0f;   // widest box of a run of queries / its largest h
+static_assert((kPRing & (kPRing - 1)) == 0 && kPRing >= kPBatch - 1 + 2 * kLeaf, "the ring holds a batch's leftover plus two leaves");
+static_assert(kPCand == 256, "a queued pair is (query lane << 8 | candidate mod 256)");
+
+constexpr size_t draw_warp_bytes()
 {
-    PairParams p;
+    return (size_t)kPRing * 16 + (size_t)kPCand * 8 + 32 * 4 + (size_t)(kPList + kStack) * 4 +
+           (size_t)4 * 16 + (size_t)kPQueue * 2 + 8 * 8;
+}
+static_assert(draw_warp_bytes() % 16 == 0 && (kPList + kStack) % 4 == 0 && kPQueue % 8 == 0, "16-byte aligned parts");
+
+// max over v of sigma(v) v / s0 for kind 1: v / (1 + (v/w)^2)^2 peaks at v = w / sqrt(3)
+constexpr float kSvMax = 0.32475953f;    // 3 sqrt(3) / 16, rounded up
+
+// packed pairs of FP32 (each half rounded to nearest like the scalar operation)
+__device__ __forceinline__ unsigned long long pack2(float a, float b)
+{
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(unsigned long long v, float& a, float& b)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b)
+{
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b)
+{
+    unsigned long long r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c)
+{
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+template <class R, int MODE, int PR, bool DRAG>
+__global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
+{
+    static_assert(PR >= 1 && PR <= kPerRoundMax, "32-pair groups drawn together");
+    using V = typename Vec4<R>::T;
+    constexpr unsigned FULL = 0xffffffffu;
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    unsigned char* base = smem + wid * draw_warp_bytes();
+    float* ring = (float*)base;                        // [4][kPRing] x, y, z, h
+    float4* wbox = (float4*)(base + kPRing * 16);      // the queries' box: lo, hi (halo frame), centre, half widths (leaf frame)
+    uint32_t* cid = (uint32_t*)(wbox + 4);             // [kPCand] candidate ids
+    uint32_t* cslot = cid + kPCand;                    // [kPCand] and slots
+    uint32_t* qid = cslot + kPCand;                    // [32] query ids
+    int* list = (int*)(qid + 32);
+    int* stack = list + kPList;
+    unsigned long long* wst = (unsigned long long*)(stack + kStack);
+    uint16_t* queue = (uint16_t*)(wst + 8);
+    if (lane < 8) wst[lane] = 0ull;
+    const R* __restrict__ T = (const R*)p.lam;
+    const V* __restrict__ P4 = (const V*)p.P4;
+    const V* __restrict__ V4 = (const V*)p.V4;
+    const uint32_t lt = (1u << lane) - 1u;
+    const int Hp = p.H + 1;
+    const int64_t items = (int64_t)p.L * p.parts;
+
+    while (true) {
+        unsigned int item = 0u;
+        if (lane == 0) item = atomicAdd(&p.cnt->work[1], 1u);
+        item = __shfl_sync(FULL, item, 0);
+        if ((int64_t)item >= items) break;
+        const int leaf = (int)(item / (unsigned)p.parts);
+        const int part = (int)(item & (unsigned)(p.parts - 1));
+        const int h = p.leaf_halo[leaf];
+        const int leaf0 = p.leaf_off[h];
+        const int A = leaf - leaf0;
+        const uint32_t nh = (uint32_t)(p.halo_off[h + 1] - p.halo_off[h]);   // n_max < 2^31
+        auto index_of = [&](uint32_t slot) {                  // padded slot -> particle index
+            return p.halo_off[h] + (int64_t)slot - (int64_t)leaf0 * kLeaf;
+        };
+        // with individual steps only particles whose step opens at this sub-step
+        // take part; a leaf without such a particle has no pair to test
+        const uint32_t slotA = (uint32_t)leaf * kLeaf + lane;
+        const bool active = (uint32_t)A * kLeaf + lane < nh &&
+                            (!p.bins || step_opens(p.bins[index_of(slotA)], p.n_bins, p.substep));
+        if (p.bins && !__any_sync(FULL, active)) continue;
+        const float4 cA = p.cell[leaf];
+        const float margin = p.frame[h].margin;
+        // forward-dominated halo: every in-range pair becomes a record (no draw);
+        // only the instantiation for contexts with SIDM_FLAG_DRAG has room for them
+        const bool drag = DRAG && p.xs[h].angular != 0;
+        if (!DRAG && p.xs[h].angular != 0) {
+            if (lane == 0) raise_status(p.cnt, SIDM_DEV_BAD_INPUT);
+            continue;
+        }
+        const float4 q = P4[slotA];
+        // the draws' integer bound: no pair's P exceeds thr 2^-32 - 2e-6 (the factor
+        // 1.001 and the 3e-6 cover every rounding and the |P - u| < 1e-6 count); a
+        // bound that is not a number below one keeps every pair
+        uint32_t thr = FULL;
+        if constexpr (MODE == kModeDraw) {
+            const sidm_xs xs = p.xs[h];
+            float sv;
+            if (xs.kind == 1) {
+                sv = kSvMax * fabsf((float)xs.w);
+            } else {
+                float vi = 0.f;
+                if (active) {
+                    const R* vel = (const R*)p.vel;
+                    const int64_t uA = index_of(slotA);
+                    const float vx = (float)vel[uA], vy = (float)vel[p.N + uA], vz = (float)vel[2 * p.N + uA];
+                    vi = sqrtf(vx * vx + vy * vy + vz * vz);
+                }
+                sv = vi + __uint_as_float(p.cnt->vmax[h]);
+            }
+            double dtl;
+            if (p.bins) {                                     // the longest step that opens now
+                const int tz = p.substep ? __ffs(p.substep) - 1 : 31;
+                dtl = ldexp(p.dt_max, -max(0, p.n_bins - 1 - tz));
+            } else {
+                dtl = p.dt[h];
+            }
+            const float inv = 1.f / q.w;
+            const float b = (float)(xs.s0 * p.mass[h] * dtl) * sv * (kLamFUp * inv * inv * inv) * 1.001f + 3e-6f;
+            uint32_t t = FULL;
+            if (b < 1.f) t = (uint32_t)(fmaxf(b, 3e-6f) * 4294967296.f) + 1u;
+            thr = __reduce_max_sync(FULL, active ? t : 0u);
+            if (drag) thr = FULL;
+        }
+        qid[lane] = active ? p.ID[slotA] : 0u;
+        uint32_t n_pairs = 0u, n_tested = 0u, n_tiles = 0u;       // the same in every lane
+
+        // the halo's factors of P in the form's precision (FP64 conversions are
+        // slow); plain draws form them for their few pairs only
+        struct Factors { R pref, inv_w, dt; bool vdep; };
+        auto factors = [&]() {
+            const sidm_xs xs = p.xs[h];
+            const R m = (R)p.mass[h], t = p.bins ? (R)p.dt_max : (R)p.dt[h];
+            return Factors{(R)xs.s0 * m * t, xs.kind == 1 ? R(1) / (R)xs.w : R(0), t, xs.kind == 1};
+        };
+        constexpr bool kEvery = MODE == kModeDrawExact || DRAG;
+        const Factors fac = kEvery ? factors() : Factors{};
+        // the full evaluation of the in-range pair (query lane li, slot sj): P (or its
+        // rate on individual steps, scaled to dt_max), decision, record
+        auto evaluate = [&](int li, uint32_t sj, uint32_t idi, uint32_t idj) -> float {
+            const Philox4 x = philox4x32_10_rk(p.step_lo, min(idi, idj), max(idi, idj), (uint32_t)h, p.rk);
+            const Factors fc = kEvery ? fac : factors();
+            const uint32_t si = (uint32_t)leaf * kLeaf + li;
+            const int64_t ui = index_of(si), uj = index_of(sj);
+            R ux, uy, uz;
+            if constexpr (MODE == kModeDraw && !DRAG) {
+                const R* vel = (const R*)p.vel;
+                ux = vel[uj] - vel[ui];
+                uy = vel[p.N + uj] - vel[p.N + ui];
+                uz = vel[2 * p.N + uj] - vel[2 * p.N + ui];
+            } else {
+                const V vi = V4[si], vj = V4[sj];
+                ux = vj.x - vi.x; uy = vj.y - vi.y; uz = vj.z - vi.z;
+            }
+            const V pi = P4[si], pj = P4[sj];
+            const R hi = pi.w, hj = pj.w;
+            const R v2 = ux * ux + uy * uy + uz * uz;
+            const uint32_t a = min(idi, idj), b = max(idi, idj);
+            // individual steps: the pair's longer step dt_max / 2^min(b_i, b_j)
+            const float up = p.bins ? __int_as_float((127 + min(p.bins[ui], p.bins[uj])) << 23) : 1.f;   // 2^min(b_i, b_j)
+            const float down = 1.f / up;                      // exact: bins are below 16
+            const R prefp = fc.pref * down;
+            // P needs ~1e-6 relative accuracy only (the event decision below is
+            // exact for the P computed here): reciprocal square roots and
+            // approximate divisions are enough.
+            const float v = v2 > 0.f ? v2 * rsqrtf(v2) : 0.f;
+            float sig = 1.f;
+            if (fc.vdep) {
+                const float qq = v * fc.inv_w, tt = 1.f + qq * qq;
+                sig = __fdividef(1.f, tt * tt);
+            }
+            const R pre = prefp * sig * v;
+            const R inv = __fdividef(1.f, fmaxf(hi, hj));
+            const R u = (R)((float)x.x[0] * 0x1p-32f);
+            bool need = true;
+            if constexpr (MODE == kModeDraw) {
+                const R P_up = pre * (R(kLamFUp) * inv * inv * inv);
+                need = drag || !(u >= P_up + R(2e-6));
+            }
+            R P = R(0), gfac = R(0);
+            bool fire = false;
+            if (need) {
+                if constexpr (MODE == kModeDraw) atomicAdd(&wst[4], 1ull);   // else every pair
+                // canonical distance: the candidate shifted into the query leaf's frame
+                const float4 cj = p.cell[sj / kLeaf];
+                const R dx = sub_rn(__fadd_rn(pj.x, __fsub_rn(cj.x, cA.x)), pi.x);
+                const R dy = sub_rn(__fadd_rn(pj.y, __fsub_rn(cj.y, cA.y)), pi.y);
+                const R dz = sub_rn(__fadd_rn(pj.z, __fsub_rn(cj.z, cA.z)), pi.z);
+                const R d2 = fma_rn(dz, dz, fma_rn(dy, dy, mul_rn(dx, dx)));
+                const float d = d2 > 0.f ? d2 * rsqrtf(d2) : 0.f;
+                const R f = kEvery ? lambda_f_rows(p.lam4, d, hi, hj, inv) : lambda_f_fast(T, d, hi, hj, inv);
+                P = pre * (f * inv * inv * inv);
+                if (drag) {
+                    // the record keeps G = m_j Lambda dt; D = P / 3 at the step start.
+                    // The turn's sine is the square root of a multiple of Lambda, so
+                    // Lambda must be accurate relative to itself where it falls to
+                    // zero, which neither the table nor an FP32 quadrature (its
+                    // integrand cancels there) is: FP64 quadrature beyond half the
+                    // support, the table inside, where Lambda > Lambda(0)/4 bounds
+                    // its relative error
+                    R lam = f * inv * inv * inv;
+                    const R dq = sqrt_rn(d2);
+                    if (dq >= R(0.5) * (hi + hj))
+                        lam = (R)lambda_quad<double>((double)dq, (double)hi, (double)hj, p.glx, p.glw);
+                    fire = true;
+                    P = pre * lam;
+                    gfac = (R)p.mass[h] * lam * (fc.dt * down);
+                    if (P > R(3)) atomicAdd(&wst[1], 1ull);
+                } else {
+                    fire = P >= R(1) || x.x[0] < (uint32_t)ceilf((float)P * 0x1p32f);
+                    if (P > R(1)) atomicAdd(&wst[1], 1ull);
+                    if (fabs(P - u) < R(1e-6)) atomicAdd(&wst[2], 1ull);
+                }
+            }
+            if (fire) {
+                // one counter update for the lanes that fire together
+                const unsigned am = __activemask();
+                const int lead = __ffs(am) - 1;
+                unsigned long long slot = 0ull;
+                if (lane == lead) slot = atomicAdd(&p.cnt->ev_count, (unsigned long long)__popc(am));
+                slot = __shfl_sync(am, slot, lead) + (unsigned long long)__popc(am & lt);
+                if (slot < p.ev_cap) {
+                    sidm_event E;
+                    E.key = ((unsigned long long)h << 54) | ((unsigned long long)a << 27) | (unsigned long long)b;
+                    E.i = (uint32_t)(idi < idj ? ui : uj);
+                    E.j = (uint32_t)(idi < idj ? uj : ui);
+                    E.x1 = x.x[1];
+                    E.x2 = x.x[2];
+                    E.P = (float)P;
+                    E.x0 = x.x[0];
+                    p.ev[slot] = E;
+                    if (drag) p.evg[slot] = (double)gfac;
+                }
+            }
+            return P * up;
+        };
+
+        // Consecutive particles of the Morton curve can lie far apart (on the sparse
+        // outer shell on opposite sides of the halo), and boxes around them would
+        // reach most of it: the queries are taken in runs of lanes whose box is at
+        // most kPSpread times their largest h wide (nearly always one run)
+        uint32_t todo = __ballot_sync(FULL, active);
+        while (todo) {
+        bool act = (todo >> lane) & 1u;
+        {
+            const float px = __fadd_rn(cA.x, q.x), py = __fadd_rn(cA.y, q.y), pz = __fadd_rn(cA.z, q.z);
+            float v[7] = {act ? px : INFINITY,  act ? py : INFINITY,  act ? pz : INFINITY,
+                          act ? -px : INFINITY, act ? -py : INFINITY, act ? -pz : INFINITY, act ? -q.w : INFINITY};
+            float w[7];
+            auto box = [&]() {                               // of the act lanes: lo, -hi, -largest h
+#pragma unroll
+                for (int i = 0; i < 7; ++i) w[i] = act ? v[i] : INFINITY;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+                    for (int i = 0; i < 7; ++i) w[i] = fminf(w[i], __shfl_xor_sync(FULL, w[i], o));
+                }
+            };
+            auto wide = [&]() {
+                return fmaxf(fmaxf(-w[3] - w[0], -w[4] - w[1]), -w[5] - w[2]) > kPSpread * -w[6];
+            };
+            box();
+            if (wide()) {                                    // the same in every lane
+                // boxes of the lanes up to this one: the run ends before the first that is too wide
+#pragma unroll
+                for (int i = 0; i < 7; ++i) w[i] = v[i];
+                for (int o = 1; o < 32; o <<= 1) {
+#pragma unroll
+                    for (int i = 0; i < 7; ++i) {
+                        const float y = __shfl_up_sync(FULL, w[i], o);
+                        if (lane >= o) w[i] = fminf(w[i], y);
+                    }
+                }
+                const uint32_t over = __ballot_sync(FULL, act && wide());
+                if (over) act = act && lane < __ffs(over) - 1;
+                box();
+            }
+            todo &= ~__ballot_sync(FULL, act);
+            float f[6] = {act ? q.x : INFINITY,  act ? q.y : INFINITY,  act ? q.z : INFINITY,
+                          act ? -q.x : INFINITY, act ? -q.y : INFINITY, act ? -q.z : INFINITY};
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+                for (int i = 0; i < 6; ++i) f[i] = fminf(f[i], __shfl_xor_sync(FULL, f[i], o));
+            }
+            __syncwarp();
+            if (lane == 0) {
+                wbox[0] = make_float4(w[0], w[1], w[2], 0.f);
+                wbox[1] = make_float4(-w[3], -w[4], -w[5], -w[6]);
+                // centre and half widths; with c = RN(x - centre) the computed gap
+                // |c| - half of a point x exceeds the true one by less than 2^-22 (gap +
+                // half), which the factors here and on the reach cover
+                const float cx = 0.5f * (f[0] - f[3]), cy = 0.5f * (f[1] - f[4]), cz = 0.5f * (f[2] - f[5]);
+                const float s = 1.0f + 0x1p-18f;
+                wbox[2] = make_float4(-cx, -cy, -cz, 0.f);
+                wbox[3] = make_float4(s * fmaxf(-f[3] - cx, cx - f[0]), s * fmaxf(-f[4] - cy, cy - f[1]),
+                                      s * fmaxf(-f[5] - cz, cz - f[2]), -w[6]);
+            }
+            __syncwarp();
+        }
+        // the query, negated, in both halves (NaN: in range of nothing)
+        const float nx = act ? -q.x : __int_as_float(0x7fffffff);
+        const unsigned long long qx2 = pack2(nx, nx), qy2 = pack2(-q.y, -q.y), qz2 = pack2(-q.z, -q.z), qw2 = pack2(q.w, q.w);
+
+        // the accepted children of a node: local leaf indices into the list (this
+        // part's share: every parts-th one), or nodes onto the stack.  A child is
+        // visited iff the queries' box comes within (h + hmax_child)(1 + 2^-20) +
+        // margin of the child's box, h the queries' largest, and its subtree holds a
+        // leaf >= A
+        int nl = 0, seen = 0, sp = 0;
+        bool failed = false;
+        auto visit = [&](int lev, int first, int base, int n) {
+            float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
+            const bool in = lane < n && ((int64_t)(first + lane + 1) << (kArityLog * lev)) > (int64_t)A;
+            if (in) { lo = p.nlo[base + first + lane]; hi = p.nhi[base + first + lane]; }
+            const float4 qhi = wbox[1];
+            const float r = __fadd_ru(__fmul_ru(__fadd_ru(qhi.w, lo.w), 1.0f + 0x1p-20f), margin);
+            const bool ok = box_gap2_rd(wbox[0], qhi, lo, hi) <= __fmul_ru(r, r);
+            uint32_t acc = __ballot_sync(FULL, in && ok);
+            if (lev == 0) {
+                const bool mine = ((acc >> lane) & 1u) && ((seen + __popc(acc & lt)) & (p.parts - 1)) == part;
+                seen += __popc(acc);
+                acc = __ballot_sync(FULL, mine);
+                if (mine) list[nl + __popc(acc & lt)] = first + lane;
+                nl += __popc(acc);
+            } else if (sp + __popc(acc) > kStack) {
+                failed = true;
+            } else {
+                // descending local index on the stack, so the lowest is visited first
+                sp += __popc(acc);
+                if ((acc >> lane) & 1u) stack[sp - 1 - __popc(acc & lt)] = (lev << 24) | (first + lane);
+            }
+            __syncwarp();
+        };
+        const int top = p.top[h];
+        {
+            const int nb = p.lvl_off[top * Hp + h];
+            visit(top, 0, nb, p.lvl_off[top * Hp + h + 1] - nb);
+        }
+        // ring entries: candidate numbers cnum .. cnum + navail - 1; queued pairs qn,
+        // the oldest candidate number they may name, entries of the query leaf
+        // itself still in the ring and this lane's rank among them
+        int navail = 0, qn = 0, nself = 0, rank = 0, li = 0;
+        uint32_t cnum = 0u, oldest = 0u;
+        const int n_act = __popc(__ballot_sync(FULL, act));
+        while (true) {
+            bool fin = false;
+            if (li < nl) {
+                // two listed leaves: shift, filter, append to the ring
+                const int Bl[2] = {list[li], list[min(li + 1, nl - 1)]};
+                float4 c[2], cB[2];
+                uint32_t id[2];
+                bool open[2];
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const uint32_t s = (uint32_t)(leaf0 + Bl[u]) * kLeaf + lane;
+                    c[u] = P4[s];
+                    cB[u] = p.cell[leaf0 + Bl[u]];
+                    id[u] = p.ID[s];
+                    open[u] = (uint32_t)Bl[u] * kLeaf + lane < nh && li + u < nl;
+                    if (p.bins) open[u] = open[u] && step_opens(p.bins[index_of(s)], p.n_bins, p.substep);
+                }
+                const float4 fc = wbox[2], fw = wbox[3];
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    c[u].x = __fadd_rn(c[u].x, __fsub_rn(cB[u].x, cA.x));     // exact shift into the query leaf's frame
+                    c[u].y = __fadd_rn(c[u].y, __fsub_rn(cB[u].y, cA.y));
+                    c[u].z = __fadd_rn(c[u].z, __fsub_rn(cB[u].z, cA.z));
+                    const float gx = fmaxf(fabsf(c[u].x + fc.x) - fw.x, 0.f), gy = fmaxf(fabsf(c[u].y + fc.y) - fw.y, 0.f),
+                                gz = fmaxf(fabsf(c[u].z + fc.z) - fw.z, 0.f);
+                    const float r = (c[u].w + fw.w) * (1.0f + 0x1p-18f);
+                    const bool keep = open[u] && gx * gx + gy * gy + gz * gz <= r * r;
+                    const uint32_t m = __ballot_sync(FULL, keep);
+                    if (u == 0 && Bl[0] == A) { nself = __popc(m); rank = __popc(m & lt); }   // A is the first of its walk
+                    if (keep) {
+                        const uint32_t e = cnum + navail + __popc(m & lt);
+                        float* at = ring + (e & (kPRing - 1));
+                        at[0] = c[u].x; at[kPRing] = c[u].y; at[2 * kPRing] = c[u].z; at[3 * kPRing] = c[u].w;
+                        uint32_t* ca = cid + (e & (kPCand - 1));
+                        ca[0] = id[u];
+                        ca[kPCand] = (uint32_t)(leaf0 + Bl[u]) * kLeaf + lane;
+                    }
+                    navail += __popc(m);
+                    n_tested += (uint32_t)(n_act * __popc(m));       // an upper bound inside the query leaf
+                }
+                n_tiles += min(2, nl - li);
+                li += 2;
+                __syncwarp();
+            } else if (sp > 0 && !failed) {
+                // walk until the list may not hold another node's leaves, or the tree is done
+                nl = li = 0;
+                do {
+                    const int e = stack[--sp];
+                    __syncwarp();
+                    const int cl = (e >> 24) - 1, first = (e & 0xFFFFFF) * kArity;
+                    const int cb = p.lvl_off[cl * Hp + h];
+                    visit(cl, first, cb, min(kArity, p.lvl_off[cl * Hp + h + 1] - cb - first));
+                } while (sp > 0 && nl <= kPList - kArity && !failed);
+            } else {
+                // at the very end fill the partial batch with infinitely far entries
+                fin = true;
+                const int fill = (kPBatch - navail % kPBatch) % kPBatch;
+                if (lane < fill) {
+                    float* at = ring + ((cnum + navail + lane) & (kPRing - 1));
+                    at[0] = INFINITY; at[kPRing] = INFINITY; at[2 * kPRing] = INFINITY; at[3 * kPRing] = 0.f;
+                }
+                navail += fill;
+                __syncwarp();
+            }
+            while (navail >= kPBatch || (fin && qn > 0)) {
+                int full = qn;                           // pairs to draw now: all of them at the very end
+                if (navail >= kPBatch) {
+                    // the ring's first kPBatch candidates against all queries
+                    uint32_t okm = 0u;
+#pragma unroll
+                    for (int t = 0; t < kPBatch; t += 4) {
+                        const float* at = ring + (cnum & (kPRing - 1)) + t;
+                        const ulonglong2 x = *(const ulonglong2*)at, y = *(const ulonglong2*)(at + kPRing),
+                                         z = *(const ulonglong2*)(at + 2 * kPRing), w = *(const ulonglong2*)(at + 3 * kPRing);
+#pragma unroll
+                        for (int u = 0; u < 2; ++u) {
+                            const unsigned long long dx = add2(u ? x.y : x.x, qx2), dy = add2(u ? y.y : y.x, qy2),
+                                                     dz = add2(u ? z.y : z.x, qz2);
+                            const unsigned long long d2 = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
+                            const unsigned long long hs = add2(qw2, u ? w.y : w.x), hs2 = mul2(hs, hs);
+                            float da, db, ha, hb;
+                            unpack2(d2, da, db);
+                            unpack2(hs2, ha, hb);
+                            if (da < ha) okm |= 1u << (t + 2 * u);
+                            if (db < hb) okm |= 2u << (t + 2 * u);
+                        }
+                    }
+                    if (nself > 0) {                     // inside the leaf each pair once: candidates after the query
+                        const int after = rank + 1;      // candidate number of the leaf, counted from the first
+                        okm &= after - (int)cnum >= 32 ? 0u : after > (int)cnum ? FULL << (after - (int)cnum) : FULL;
+                        nself -= kPBatch;
+                    }
+                    // this lane's place in the queue, then its pairs
+                    const int n = __popc(okm);
+                    int inc = n;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int y = __shfl_up_sync(FULL, inc, o);
+                        if (lane >= o) inc += y;
+                    }
+                    const int total = __shfl_sync(FULL, inc, 31);
+                    uint16_t* qp = queue + qn + inc - n;
+                    const uint32_t tag = (uint32_t)lane << 8;
+#pragma unroll
+                    for (int t = 0; t < kPBatch; ++t)
+                        if ((okm >> t) & 1u) *qp++ = (uint16_t)(tag | ((cnum + t) & (kPCand - 1)));
+                    if (qn == 0) oldest = cnum;
+                    qn += total;
+                    n_pairs += (uint32_t)total;
+                    const int rest = qn % (32 * PR);
+                    full = qn - rest;
+                    // the waiting pairs keep their candidates: draw them too before those are overwritten
+                    if (total < rest) { if (cnum + 2 * kPBatch + 2 * kLeaf - oldest > kPCand) full = qn; }
+                    else oldest = cnum;
+                    cnum += kPBatch;
+                    navail -= kPBatch;
+                    __syncwarp();
+                }
+                for (int f0 = 0; f0 < full; f0 += 32 * PR) {
+                    uint32_t ent[PR], idi[PR], idj[PR];
+                    uint32_t maybe = 0u;
+#pragma unroll
+                    for (int k = 0; k < PR; ++k) {
+                        const int at = f0 + 32 * k + lane;
+                        ent[k] = queue[at < full ? at : f0];
+                        idi[k] = qid[ent[k] >> 8];
+                        idj[k] = cid[ent[k] & (kPCand - 1)];
+                        const Philox4 x = philox4x32_10_rk(p.step_lo, min(idi[k], idj[k]), max(idi[k], idj[k]), (uint32_t)h, p.rk);
+                        maybe |= (at < full && x.x[0] <= thr ? 1u : 0u) << k;
+                    }
+                    if constexpr (MODE == kModeDrawExact) {
+                        static_assert(MODE != kModeDrawExact || PR == 1, "one group at a time");
+                        // the per-particle sums of P: the query's by one addition per run of
+                        // its pairs in the group (they stand together), the partner's each
+                        const int li = (int)(ent[0] >> 8);
+                        const uint32_t sj = cslot[ent[0] & (kPCand - 1)];
+                        float ps = maybe ? evaluate(li, sj, idi[0], idj[0]) : 0.f;
+                        if (p.use_sump) {
+                            __syncwarp();
+                            if (maybe) atomicAdd(p.sump + index_of(sj), ps);
+                            const int before = __shfl_up_sync(FULL, li, 1);
+                            const uint32_t heads = __ballot_sync(FULL, lane == 0 || before != li);
+                            const uint32_t later = heads & ~((2u << lane) - 1u);
+                            const int end = later ? __ffs(later) - 1 : 32;         // of this lane's run
+#pragma unroll
+                            for (int o = 1; o < 32; o <<= 1) {
+                                const float y = __shfl_down_sync(FULL, ps, o);
+                                if (lane + o < end) ps += y;
+                            }
+                            if (((heads >> lane) & 1u) && maybe) atomicAdd(p.sump + index_of((uint32_t)leaf * kLeaf + li), ps);
+                            __syncwarp();
+                        }
+                    } else if (maybe) {
+#pragma unroll 1
+                        for (int k = 0; k < PR; ++k) {
+                            if (!((maybe >> k) & 1u)) continue;
+                            uint32_t en = ent[0], di = idi[0], dj = idj[0];
+#pragma unroll
+                            for (int r = 1; r < PR; ++r)
+                                if (r == k) { en = ent[r]; di = idi[r]; dj = idj[r]; }
+                            evaluate((int)(en >> 8), cslot[en & (kPCand - 1)], di, dj);
+                        }
+                    }
+                }
+                // the rest moves to the queue's front
+                if (full > 0) {
+                    const int rest = qn - full;          // < 32 PR <= full: no overlap
+                    __syncwarp();
+#pragma unroll
+                    for (int k = 0; k < PR; ++k)
+                        if (32 * k + lane < rest) queue[32 * k + lane] = queue[full + 32 * k + lane];
+                    qn = rest;
+                    __syncwarp();
+                }
+            }
+            if (fin) break;
+        }
+        if (failed && lane == 0) raise_status(p.cnt, SIDM_DEV_STACK);
+        }   // runs of queries
+        // this leaf's counts into the warp's 64-bit statistics
+        {
+            __syncwarp();
+            if (lane == 0) {
+                wst[0] += n_pairs; wst[3] += n_tested; wst[5] += n_tiles;
+                if (MODE != kModeDraw) wst[4] += n_pairs;
+                wst[6] = max(wst[6], (unsigned long long)n_tiles);
+            }
+            __syncwarp();
+        }
+    }
+    // warp totals -> step statistics
+    if (lane == 0) {
+        if (wst[0]) atomicAdd(&p.st->n_pairs, wst[0]);
+        if (wst[1]) atomicAdd(&p.st->n_p_gt1, wst[1]);
+        if (wst[2]) atomicAdd(&p.st->n_near, wst[2]);
+        if (wst[3]) atomicAdd(&p.st->n_tested, wst[3]);
+        atomicAdd(&p.cnt->diag[4], wst[5]);
+        atomicMax(&p.cnt->diag[5], wst[6]);
+        if (wst[4]) atomicAdd(&p.cnt->diag[6], wst[4]);
+    }
+}
+
+// Largest speed of every halo whose cross-section does not depend on the speed
+// (kind 0), for the bound of P: kSplit CTAs per reduction chunk, one atomic each.
+// A NaN speed drops out of the maximum: its pairs have P = NaN and never fire.
+constexpr int kVmaxSplit = 4, kVmaxChunk = 16384;
+template <class R>
+__global__ void __launch_bounds__(256) k_vmax(const R* __restrict__ vel, int64_t N, const int32_t* __restrict__ chunk_halo,
+                                              const int64_t* __restrict__ chunk_begin, const int64_t* __restrict__ halo_off,
+                                              const sidm_xs* __restrict__ xs, DevCounters* __restrict__ cnt)
+{
+    const int c = blockIdx.x / kVmaxSplit, part = blockIdx.x % kVmaxSplit;
+    const int h = chunk_halo[c];
+    if (xs[h].kind == 1) return;
+    const int64_t b = chunk_begin[c] + (int64_t)part * (kVmaxChunk / kVmaxSplit);
+    const int64_t e = min(min(chunk_begin[c] + kVmaxChunk, halo_off[h + 1]), b + kVmaxChunk / kVmaxSplit);
+    float m = 0.f;
+#pragma unroll 4
+    for (int64_t s = b + threadIdx.x; s < e; s += blockDim.x) {
+        const float x = (float)vel[s], y = (float)vel[N + s], z = (float)vel[2 * N + s];
+        m = fmaxf(m, x * x + y * y + z * z);
+    }
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0 && m > 0.f) atomicMax(&cnt->vmax[h], __float_as_uint(sqrtf(m)));
+}
+
+void fill_params(sidm_ctx* c, PairParams& p, uint64_t seed, uint64_t step, const sidm_xs* xs, const double* dt,
+                 const double* mass, const void* vel, sidm_step_stats* st)
+{
     const LayoutHost& L = c->lay;
+    p = PairParams{};
     p.H = L.H; p.L = L.L;
     p.leaf_halo = c->d_leaf_halo; p.leaf_off = c->d_leaf_off; p.halo_off = c->d_halo_off;
     p.lvl_off = c->d_lvl_off; p.top = c->d_top; p.frame = c->d_frame; p.cell = c->d_cell;
-    p.nlo = c->d_nlo; p.nhi = c->d_nhi; p.P4 = c->d_P4; p.V4 = c->d_V4; p.lam = c->d_lam;
+    p.nlo = c->d_nlo; p.nhi = c->d_nhi; p.P4 = c->d_P4; p.V4 = c->d_V4; p.ID = c->d_ID; p.lam = c->d_lam; p.lam4 = c->d_lam4;
+    p.vel = vel; p.N = L.N; p.parts = 1;
     p.xs = xs; p.dt = dt; p.mass = mass;
     p.seed_lo = (uint32_t)seed; p.seed_hi = (uint32_t)(seed >> 32); p.step_lo = (uint32_t)step;
     for (int r = 0; r < 10; ++r) {
@@ -608,9 +1226,18 @@ int launch_t(sidm_ctx* c, uint64_t seed, uint64_t step, const sidm_xs* xs, const
     p.cnt = c->d_cnt; p.st = st;
     p.evg = c->d_evg;
     for (int g = 0; g < 8; ++g) { p.glx[g] = c->gl8x[g]; p.glw[g] = c->gl8w[g]; }
+}
+
+template <class R, bool TMA, int MODE, int PR = kPerRoundMax, bool DRAG = false>
+int launch_t(sidm_ctx* c, uint64_t seed, uint64_t step, const sidm_xs* xs, const double* dt, const double* mass,
+             const void* vel, sidm_step_stats* st, cudaStream_t s)
+{
+    PairParams p;
+    fill_params(c, p, seed, step, xs, dt, mass, vel, st);
+    const LayoutHost& L = c->lay;
     const int warps = c->pair_warps;
     const size_t smem = (size_t)warps * pair_warp_bytes<R, TMA>();
-    auto kern = k_pairs<R, TMA, MODE, PR, DRAG>;
+    auto kern = k_pairs_queue<R, TMA, MODE, PR, DRAG>;
     int occ = 0;
     int rc = occupancy(c, (const void*)kern, warps * 32, smem, &occ);
     if (rc) return rc;
@@ -630,37 +1257,76 @@ int launch_t(sidm_ctx* c, uint64_t seed, uint64_t step, const sidm_xs* xs, const
     return SIDM_OK;
 }
 
+// mixed-form draws.  With few query leaves each is shared by several warps (a
+// power of two, at most kPartsMax), so that every resident warp has about
+// kPartsPerWarp items: the last wave stays short, at the price of the walk that
+// the parts repeat.
+constexpr int kPartsMax = 16;
+constexpr int64_t kPartsPerWarp = 4;
+template <class R, int MODE, int PR, bool DRAG>
+int launch_draws(sidm_ctx* c, uint64_t seed, uint64_t step, const sidm_xs* xs, const double* dt, const double* mass,
+                 const void* vel, sidm_step_stats* st, cudaStream_t s)
+{
+    PairParams p;
+    fill_params(c, p, seed, step, xs, dt, mass, vel, st);
+    const LayoutHost& L = c->lay;
+    const int warps = c->pair_warps;
+    const size_t smem = (size_t)warps * draw_warp_bytes();
+    auto kern = k_pairs<R, MODE, PR, DRAG>;
+    int occ = 0;
+    if (int rc = occupancy(c, (const void*)kern, warps * 32, smem, &occ)) return rc;
+    if (occ < 1) return set_err(c, SIDM_ECAPACITY, "pair kernel does not fit on an SM");
+    int grid = c->cfg.grid_ctas > 0 ? c->cfg.grid_ctas : c->sm_count * occ;
+    while (p.parts < kPartsMax && (int64_t)L.L * p.parts < kPartsPerWarp * grid * warps) p.parts *= 2;
+    grid = (int)std::max<int64_t>(1, std::min<int64_t>(grid, ((int64_t)L.L * p.parts + warps - 1) / warps));
+    c->pair_grid = grid;
+    cudaError_t e = cudaMemsetAsync(&c->d_cnt->work[1], 0, sizeof(unsigned int), s);
+    if (e != cudaSuccess) return cuda_check(c, e, "pair work reset");
+    if (MODE == kModeDraw) {
+        k_vmax<R><<<L.nchunk * kVmaxSplit, 256, 0, s>>>((const R*)vel, L.N, c->d_chunk_halo, c->d_chunk_begin, c->d_halo_off,
+                                                        xs, c->d_cnt);
+        c->launches++;
+    }
+    const int tidx = timer_begin(c, 2, s);
+    kern<<<grid, warps * 32, smem, s>>>(p);
+    timer_end(c, tidx, s);
+    c->launches++;
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return cuda_check(c, e, "pair launch");
+    return SIDM_OK;
+}
+
 }  // namespace
 
 int launch_pairs(sidm_ctx* c, uint64_t seed, uint64_t step, const sidm_xs* xs, const double* dt, const double* mass,
-                 sidm_step_stats* st, cudaStream_t s)
+                 const void* vel, sidm_step_stats* st, cudaStream_t s)
 {
     if (c->lay.L == 0) return SIDM_OK;
     const bool tma = c->cfg.use_tma != 0;
     const bool exact = (c->cfg.flags & SIDM_FLAG_SUM_P) != 0;
     if (c->cfg.flags & SIDM_FLAG_DRAG) {                // forward-dominated halos allowed (plain loads)
         if (c->cfg.precision == SIDM_FP64)
-            return exact ? launch_t<double, false, kModeDrawExact, kPerRoundMax, true>(c, seed, step, xs, dt, mass, st, s)
-                         : launch_t<double, false, kModeDraw, kPerRoundMax, true>(c, seed, step, xs, dt, mass, st, s);
-        return exact ? launch_t<float, false, kModeDrawExact, kPerRoundMax, true>(c, seed, step, xs, dt, mass, st, s)
-                     : launch_t<float, false, kModeDraw, kPerRoundMax, true>(c, seed, step, xs, dt, mass, st, s);
+            return exact ? launch_t<double, false, kModeDrawExact, kPerRoundMax, true>(c, seed, step, xs, dt, mass, vel, st, s)
+                         : launch_t<double, false, kModeDraw, kPerRoundMax, true>(c, seed, step, xs, dt, mass, vel, st, s);
+        return exact ? launch_draws<float, kModeDrawExact, 1, true>(c, seed, step, xs, dt, mass, vel, st, s)
+                     : launch_draws<float, kModeDraw, 1, true>(c, seed, step, xs, dt, mass, vel, st, s);
     }
 #define SIDM_PAIRS_DISPATCH(R)                                                                                   \
-    if (exact) return tma ? launch_t<R, true, kModeDrawExact>(c, seed, step, xs, dt, mass, st, s)                \
-                          : launch_t<R, false, kModeDrawExact>(c, seed, step, xs, dt, mass, st, s);              \
-    if (tma) return launch_t<R, true, kModeDraw>(c, seed, step, xs, dt, mass, st, s);
+    if (exact) return tma ? launch_t<R, true, kModeDrawExact>(c, seed, step, xs, dt, mass, vel, st, s)                \
+                          : launch_t<R, false, kModeDrawExact>(c, seed, step, xs, dt, mass, vel, st, s);              \
+    if (tma) return launch_t<R, true, kModeDraw>(c, seed, step, xs, dt, mass, vel, st, s);
     if (c->cfg.precision == SIDM_FP64) {
         SIDM_PAIRS_DISPATCH(double)
-        return launch_t<double, false, kModeDraw>(c, seed, step, xs, dt, mass, st, s);
+        return launch_t<double, false, kModeDraw>(c, seed, step, xs, dt, mass, vel, st, s);
     }
-    SIDM_PAIRS_DISPATCH(float)
+    if (exact) return launch_draws<float, kModeDrawExact, 1, false>(c, seed, step, xs, dt, mass, vel, st, s);
 #undef SIDM_PAIRS_DISPATCH
     // the hot path: pairs queued per lane and round as configured (a launch knob)
-    switch (c->cfg.pair_per_round > 0 ? c->cfg.pair_per_round : kPerRoundMax) {
-    case 1: return launch_t<float, false, kModeDraw, 1>(c, seed, step, xs, dt, mass, st, s);
-    case 2: return launch_t<float, false, kModeDraw, 2>(c, seed, step, xs, dt, mass, st, s);
-    case 3: return launch_t<float, false, kModeDraw, 3>(c, seed, step, xs, dt, mass, st, s);
-    default: return launch_t<float, false, kModeDraw, 4>(c, seed, step, xs, dt, mass, st, s);
+    switch (c->cfg.pair_per_round > 0 ? c->cfg.pair_per_round : kPerRoundDefault) {
+    case 1: return launch_draws<float, kModeDraw, 1, false>(c, seed, step, xs, dt, mass, vel, st, s);
+    case 2: return launch_draws<float, kModeDraw, 2, false>(c, seed, step, xs, dt, mass, vel, st, s);
+    case 3: return launch_draws<float, kModeDraw, 3, false>(c, seed, step, xs, dt, mass, vel, st, s);
+    default: return launch_draws<float, kModeDraw, 4, false>(c, seed, step, xs, dt, mass, vel, st, s);
     }
 }
 
@@ -668,8 +1334,8 @@ int launch_pairs_diag(sidm_ctx* c, const sidm_xs* xs, const double* mass, cudaSt
 {
     if (c->lay.L == 0) return SIDM_OK;
     if (c->cfg.precision == SIDM_FP64)
-        return launch_t<double, false, kModeDiag>(c, 0, 0, xs, nullptr, mass, c->d_stats_own, s);
-    return launch_t<float, false, kModeDiag>(c, 0, 0, xs, nullptr, mass, c->d_stats_own, s);
+        return launch_t<double, false, kModeDiag>(c, 0, 0, xs, nullptr, mass, nullptr, c->d_stats_own, s);
+    return launch_t<float, false, kModeDiag>(c, 0, 0, xs, nullptr, mass, nullptr, c->d_stats_own, s);
 }
 
 }  // namespace sidm
