@@ -316,7 +316,8 @@ int sidm_kernel_times(sidm_ctx* ctx, double* ms_out, int64_t* count_out, int32_t
  * out[6] in-range pairs whose Lambda was looked up (all of them under
  * SIDM_FLAG_SUM_P; otherwise only those whose draw fell below the upper bound
  * of P), out[7] particles whose warm-started kernel-size search found fewer
- * than N_ngb candidates inside the guessed bound and was redone cold.
+ * than N_ngb candidates inside the guessed bound and was redone (with a wider
+ * bound, or cold).
  * reset != 0 clears them afterwards. */
 int sidm_diagnostics(sidm_ctx* ctx, uint64_t* out, int32_t reset);
 
@@ -415,8 +416,8 @@ int sidm_timestep_criterion(sidm_ctx* ctx, double tau, double dt_min, double dt_
  * caller's arrays must still be in the order that call left them, with the
  * same halo layout and N_ngb).  The search then only admits candidates within
  * knn_slack times that size (1.07 by default); a particle with fewer than
- * N_ngb of them is redone from scratch by a second, per-lane launch on the
- * same stream.  The result is the exact k-th distance in
+ * N_ngb of them is redone with a wider bound, or from scratch by a second,
+ * per-lane launch on the same stream.  The result is the exact k-th distance in
  * every case -- a stale or wrong guess costs time, never accuracy -- so this
  * is the usual SPH practice of starting from the previous smoothing length
  * (Sect. 2: h follows the N_ngb nearest neighbours as particles move).

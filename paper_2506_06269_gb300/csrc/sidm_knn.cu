@@ -43,6 +43,7 @@ struct KnnParams {
     const float4* nlo;
     const float4* nhi;
     void* P4;
+    const void* S4;     // FP32 offsets the warm-started search reads (mixed form: P4)
     const uint32_t* ID;
     void* h_out;
     uint32_t* nbr;
@@ -692,419 +693,489 @@ __global__ void k_knn(KnnParams p)
 // ---------------------------------------------------------------------------
 // Warm-started search.  From the second call on every particle carries its
 // previous kernel size, and only candidates inside slack x h_prev are admitted
-// (reading C14).  That bound is fixed for the whole query leaf, so:
-//  * the tree is walked level by level (the child boxes of the next frontier
-//    node load while the current one is tested); each child's box is tested
-//    against the boxes of the walk's lane groups, each grown by the largest
-//    bound of its lanes (one box test per child and group, no per-lane point
-//    tests), and the accepted leaves are listed;
-//  * the listed leaves are loaded two ahead; a candidate is kept if it lies
-//    within some filter group's largest bound of that group's box, a test made
-//    in the query leaf's own frame with directed rounding, where the box gap is
-//    a lower bound of the canonical distance (no margin needed); kept
-//    candidates go to a per-warp ring;
-//  * full batches of kWBatch ring entries are tested against all 32 queries
-//    with branch-free admission: a lane stores every key at its next free slot
-//    and advances the slot only when the key is below its bound;
-//  * the query leaf's own particles are tested first, with the exclusion of
-//    the query itself, so the batch loop needs none.
-// The keys of a lane sit in shared memory as [slot][lane]: slots 0..k-1 are a
-// 4-ary max-heap (filled unsorted, heapified once), slots k..k+2 stay zero (the
-// missing children of the last nodes), and up to kWPend further keys wait
-// there until a merge.  A leaf goes to a list that the per-lane search (k_knn,
-// warm-started, failing lanes cold) then redoes when a lane admits fewer than k
-// keys (its guess was too small), when a group box is much wider than its
-// bound (see kSpreadWalk), or when the walk's frontier overflows; so the result
-// is the same exact k-th distance as a cold search.
-constexpr int kWRing = 40;      // candidate ring entries
+// (reading C14).  One warp per query leaf (or, with few leaves, the warps of a
+// CTA share a leaf's candidate leaves and the first merges their keys); the
+// bound is fixed for the whole leaf, so:
+//  * the queries are taken in runs of lanes whose box is at most kWSpread(Team)
+//    times their largest bound wide (nearly always one run; consecutive particles of
+//    the Morton curve can lie on opposite sides of the halo);
+//  * the tree is walked with the run's box grown by its largest bound; accepted
+//    leaves are listed and loaded two at a time;
+//  * a candidate is kept if it lies within the largest bound of the box, a test
+//    made in the query leaf's own frame, and goes to a per-warp ring;
+//  * batches of kWBatch ring entries are tested against all 32 queries, two per
+//    packed FP32 operation, with branch-free admission: a lane stores every key
+//    at its next free slot and advances the slot only for a key below its bound.
+// The keys of a lane sit in shared memory as [slot][lane], the first kk of them
+// a 4-ary max-heap once it is ordered, up to kWPend further ones waiting behind.
+//
+// The mixed form's keys are the canonical distances and kk = N_ngb.  The FP64
+// form searches with FP32 offsets too (S4: offset to the leaf's cell corner, w =
+// a bound of the offset's error) and keeps kk = N_ngb + kWExtra keys with their
+// slots; distances in FP64 are formed only for the candidates whose FP32 distance
+// lies so near the N_ngb-th that rounding could change their order (one or two).
+//
+// A lane that admits fewer than N_ngb keys (its guess was too small) tries again
+// with a wider bound.  A leaf goes to a list that the per-lane search (k_knn,
+// warm-started, failing lanes cold) then redoes when its particles have no
+// previous kernel size, when kWAttempts bounds did not do, when the tree walk's
+// stack overflows, or when the FP32 order of the FP64 form does not settle it
+// (more than kWBand candidates within the error, or one that was not kept); so
+// the result is the same exact k-th distance as a cold search.
+//
+// Issue-bound and, with 10 to 15 warps per SM (their keys fill the shared memory),
+// latency-bound.  Per search, this launch and the redo's together: 2^20 NFW halo,
+// N_ngb = 64: 1.11 ms (1.60 ms with group boxes, one leaf and one candidate at a
+// time, and spread leaves and failed guesses left to the redo, which alone took
+// 0.37 ms); FP64 form 2.2 ms (11.6 ms with every distance in FP64).  Eight halos of
+// 1500 to 30000 particles, N_ngb up to 128: 0.50 ms (0.98); 2048 particles 40 us
+// (84), teams; FP64 16384 particles 0.22 ms (4.4).  kWSpread 2, 2.5, 3, 4: 1.15,
+// 1.11, 1.12, 1.20 ms at 2^20 and 0.47, 0.58, 0.60, 0.64 ms for the eight halos;
+// boxes of four lane groups in wide runs: 1.36 ms; runs of a leaf dealt out to the
+// team's warps instead of shared by them: 0.42 against 0.22 ms (FP64, 16384).
+constexpr int kWRing = 128;     // candidate ring entries
 constexpr int kWBatch = 8;      // candidates per batch (batches start at multiples of it: never wrap)
 constexpr int kWList = 64;      // accepted leaves listed before they are streamed
-constexpr int kWStack = 128;    // two frontier buffers of the walk, 64 nodes each (an overflow
-                                // hands the leaf to the redo)
-constexpr int kWPad = 3;        // zero slots after the heap
-constexpr int kWPend = 32;      // keys a lane may hold beyond k before a merge (room enough that
+constexpr int kWPend = 32;      // keys a lane may hold beyond kk before a merge (room enough that
                                 // merges are rare and most lanes order their heaps together)
-static_assert(kWRing % kWBatch == 0 && kWRing >= kWBatch - 1 + kLeaf, "the ring holds a batch's leftover plus a leaf");
+constexpr int kWExtra = 4;      // FP64 form: keys kept beyond N_ngb
+constexpr int kWBand = 4;       // FP64 form: candidates compared in FP64
+static_assert((kWRing & (kWRing - 1)) == 0 && kWRing >= kWBatch - 1 + 2 * kLeaf, "the ring holds a batch's leftover plus two leaves");
 static_assert(kWPend >= kWBatch, "one batch fits after a merge");
 constexpr int kWarmMaxWarps = 8;   // the kernel's launch bound: 256 threads, two CTAs per SM
-constexpr int kWalkGroups = 4;     // lane groups of the tree walk (8 lanes each)
-// a leaf goes to the per-lane search when the box of a walk group is wider than
-// kSpreadWalk times its largest bound, or a filter group's than kSpreadFilter times
-constexpr float kSpreadWalk = 3.0f;
-constexpr float kSpreadFilter = 4.0f;
+constexpr int kWAttempts = 6;      // bounds tried, each 1.5 times the one before, before the redo
+// widest box of a run of queries / its largest bound: a run costs a walk, a wide
+// box reaches dense regions that none of its queries does; a team shares both
+constexpr float kWSpread = 2.25f, kWSpreadTeam = 3.0f;
 
-template <class R, class K, int G>
+template <class R>
 __host__ __device__ constexpr size_t warm_warp_bytes(int kcap)
 {
-    return ((size_t)kWRing * sizeof(typename Vec4<R>::T) + (size_t)(kWList + kWStack) * 4 + (size_t)2 * kWalkGroups * 16 +
-            (size_t)(kcap + kWPad + kWPend) * 32 * sizeof(K) + 15) / 16 * 16;
+    using K = typename KeyOf<R, false>::T;
+    return (size_t)kWRing * (sizeof(R) == 8 ? 16 : 12) + 4 * 16 + (size_t)(kWList + kStack + 32) * 4 +
+           (size_t)(kcap + (sizeof(R) == 8 ? kWExtra : 0) + kWPend) * 32 * sizeof(K);
 }
 
-template <class R, int G>
+template <class R, bool TEAM>
 __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p, int32_t* redo_list, unsigned int* redo_len)
 {
-    static_assert(G == 2 || G == 4, "lane groups of 16 or 8 lanes");
-    using V = typename Vec4<R>::T;
     using K = typename KeyOf<R, false>::T;
+    using V = typename Vec4<R>::T;
     constexpr bool kF32 = sizeof(R) == 4;
-    constexpr int kGL = 32 / G;
     constexpr unsigned FULL = 0xffffffffu;
+    constexpr unsigned kRow = 32 * sizeof(K);          // bytes of one slot of all lanes
     extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ int team_leaf;
+    __shared__ unsigned int team_bad, team_fail, team_err;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    unsigned char* base = smem + wid * warm_warp_bytes<R, K, G>(p.kcap);
-    V* ring = (V*)base;
-    int* list = (int*)(base + (size_t)kWRing * sizeof(V));
-    int* fbuf = list + kWList;                         // [2][kWStack / 2] frontier buffers of the walk
-    float4* wbox = (float4*)(fbuf + kWStack);          // [kWalkGroups][2]: walk group boxes (halo frame), lo.w = bound
-    K* keys = (K*)(wbox + 2 * kWalkGroups);            // [kcap + kWPad + kWPend][32]
+    const int nw = TEAM ? (int)(blockDim.x >> 5) : 1, part = TEAM ? wid : 0;   // nw: a power of two
+    const size_t warp_bytes = warm_warp_bytes<R>(p.kcap);
+    unsigned char* base = smem + wid * warp_bytes;
+    float* ring = (float*)base;                        // [3 or 4][kWRing] x, y, z (and slot)
+    // the run's box: lo (w: squared reach of the walk), hi (halo frame), centre,
+    // half widths (leaf frame)
+    float4* wbox = (float4*)(ring + (kF32 ? 3 : 4) * kWRing);
+    int* list = (int*)(wbox + 4);
+    int* stack = list + kWList;
+    int* held = stack + kStack;                        // [32] keys of this warp's lanes (TEAM)
+    unsigned char* keys = (unsigned char*)(held + 32); // [kk + kWPend][32]
+    const float4* __restrict__ S4 = (const float4*)p.S4;
+    const V* P4 = (const V*)p.P4;
     const uint32_t lt = (1u << lane) - 1u;
     const int Hp = p.H + 1;
-    // the lanes redone cold are counted by the per-lane search that redoes them
-    unsigned long long n_cand = 0ull, n_ins = 0ull, n_tiles = 0ull, n_tiles_max = 0ull;
+    unsigned long long n_cand = 0ull, n_ins = 0ull, n_tiles = 0ull, n_tiles_max = 0ull, n_again = 0ull;
 
     while (true) {
         int leaf = 0;
-        if (lane == 0) leaf = (int)atomicAdd(p.work, 1u);
-        leaf = __shfl_sync(FULL, leaf, 0);
+        if constexpr (TEAM) {
+            __syncthreads();
+            if (threadIdx.x == 0) { team_leaf = (int)atomicAdd(p.work, 1u); team_bad = team_fail = team_err = 0u; }
+            __syncthreads();
+            leaf = team_leaf;
+        } else {
+            if (lane == 0) leaf = (int)atomicAdd(p.work, 1u);
+            leaf = __shfl_sync(FULL, leaf, 0);
+        }
         if (leaf >= p.L) break;
         const int h = p.leaf_halo[leaf];
         const int k = p.ngb[h];
+        const int kk = kF32 ? k : k + kWExtra;
         const int leaf0 = p.leaf_off[h];
-        const int64_t hb = p.halo_off[h];
-        const int64_t nh = p.halo_off[h + 1] - hb;
+        const uint32_t nh = (uint32_t)(p.halo_off[h + 1] - p.halo_off[h]);   // n_max < 2^31
         const int A = leaf - leaf0;
-        const int countA = (int)min((int64_t)kLeaf, nh - (int64_t)A * kLeaf);
-        const bool active = lane < countA;
-        const V q = ((const V*)p.P4)[(int64_t)leaf * kLeaf + lane];
+        const bool active = (uint32_t)A * kLeaf + lane < nh;
+        const uint32_t slotA = (uint32_t)leaf * kLeaf + lane;
+        const float4 q = S4[slotA];
+        const R hp = P4[slotA].w;
         const unsigned long long tiles0 = n_tiles;
         // a particle without a previous kernel size sends its leaf to the redo
-        if (__any_sync(FULL, active && !(q.w > R(0)))) {
-            if (lane == 0) { const unsigned r = atomicAdd(redo_len, 1u); redo_list[r] = leaf; }
-            continue;
-        }
-        const HaloFrame fr = p.frame[h];
+        bool bad = __any_sync(FULL, active && !(hp > R(0)));
+        const float margin = p.frame[h].margin;
         const float4 cA = p.cell[leaf];
-        // the lane's bound key: (slack h_prev)^2 rounded up; inactive lanes admit nothing
-        K root = K(0);
-        float r2walk = -1.0f;                          // the walk's bound in the halo frame (with the margin)
+        // the lane's bound: slack h_prev rounded up
+        float rad = 0.f;
         if (active) {
-            R r;
-            if constexpr (kF32) r = __fmul_ru((float)q.w, p.slack);
-            else r = __dmul_ru((double)q.w, (double)p.slack);
-            const R b2 = mul_ru(r, r);
-            root = make_key<R, false>(b2, 0u);
-            float rf = to_float_ru<R>(sqrt_ru(b2));
-            rf = __fadd_ru(__fmul_ru(rf, 1.0f + 0x1p-20f), fr.margin);
-            r2walk = __fmul_ru(rf, rf);
+            if constexpr (kF32) rad = __fmul_ru((float)hp, p.slack);
+            else rad = __double2float_ru(__dmul_ru((double)hp, (double)p.slack));
         }
-        // group boxes: the walk's in the halo frame (the frame of the node
-        // boxes), the candidate filter's in the query leaf's frame (mixed form;
-        // the FP64 form filters in the halo frame, with the walk's bounds)
-        float3 pq;
-        if constexpr (kF32) {
-            pq = make_float3(__fadd_rn(cA.x, (float)q.x), __fadd_rn(cA.y, (float)q.y), __fadd_rn(cA.z, (float)q.z));
-        } else {
-            pq = make_float3(__double2float_rn((double)q.x - fr.O[0]), __double2float_rn((double)q.y - fr.O[1]),
-                             __double2float_rn((double)q.z - fr.O[2]));
-        }
-        // walk boxes: groups of 8 lanes (a large bound of one lane grows only its
-        // own group's box); the bound of each group is stored in its lo.w.  On the
-        // halo's sparse outer shell a few consecutive particles of the Morton
-        // curve can lie on opposite sides of the halo: a group box much wider
-        // than its bound would accept most of the halo, so such a leaf is left
-        // to the per-lane search (the redo list, warm-started)
-        bool spread = false;
-        {
-            constexpr int kWL = 32 / kWalkGroups;
-            float v[7] = {active ? pq.x : INFINITY, active ? pq.y : INFINITY, active ? pq.z : INFINITY,
-                          active ? -pq.x : INFINITY, active ? -pq.y : INFINITY, active ? -pq.z : INFINITY, -r2walk};
+        uint32_t todo = bad ? 0u : __ballot_sync(FULL, active);
+        while (todo) {
+        bool act = (todo >> lane) & 1u;
+        const float px = __fadd_rn(cA.x, q.x), py = __fadd_rn(cA.y, q.y), pz = __fadd_rn(cA.z, q.z);
+        float w[7];
+        auto box = [&]() {                                   // of the act lanes: lo, -hi, -largest bound
+            w[0] = act ? px : INFINITY;  w[1] = act ? py : INFINITY;  w[2] = act ? pz : INFINITY;
+            w[3] = act ? -px : INFINITY; w[4] = act ? -py : INFINITY; w[5] = act ? -pz : INFINITY;
+            w[6] = act ? -rad : INFINITY;
+        };
+        auto widest = [&]() {
 #pragma unroll
-            for (int o = kWL / 2; o > 0; o >>= 1) {
+            for (int o = 16; o > 0; o >>= 1) {
 #pragma unroll
-                for (int i = 0; i < 7; ++i) v[i] = fminf(v[i], __shfl_xor_sync(FULL, v[i], o));
+                for (int i = 0; i < 7; ++i) w[i] = fminf(w[i], __shfl_xor_sync(FULL, w[i], o));
             }
-            if (lane % kWL == 0) {
-                wbox[2 * (lane / kWL)] = make_float4(v[0], v[1], v[2], -v[6]);
-                wbox[2 * (lane / kWL) + 1] = make_float4(-v[3], -v[4], -v[5], 0.f);
-                const float ext = fmaxf(fmaxf(-v[3] - v[0], -v[4] - v[1]), -v[5] - v[2]);
-                spread = -v[6] >= 0.f && ext * ext > kSpreadWalk * kSpreadWalk * -v[6];
+        };
+        auto wide = [&]() {
+            return fmaxf(fmaxf(-w[3] - w[0], -w[4] - w[1]), -w[5] - w[2]) > (TEAM ? kWSpreadTeam : kWSpread) * -w[6];
+        };
+        box();
+        widest();
+        if (wide()) {                                        // the same in every lane
+            // boxes of the lanes up to this one: the run ends before the first that is too wide
+            box();
+            for (int o = 1; o < 32; o <<= 1) {
+#pragma unroll
+                for (int i = 0; i < 7; ++i) {
+                    const float y = __shfl_up_sync(FULL, w[i], o);
+                    if (lane >= o) w[i] = fminf(w[i], y);
+                }
+            }
+            const uint32_t over = __ballot_sync(FULL, act && wide());
+            if (over) act = act && lane < __ffs(over) - 1;
+        }
+        todo &= ~__ballot_sync(FULL, act);
+        // a lane that admits fewer than N_ngb keys tries again with a wider bound
+        for (int attempt = 0;; ++attempt) {
+        uint32_t root = act ? __float_as_uint(__fmul_ru(rad, rad)) : 0u;   // bits of the lane's d^2 bound
+        float err = 0.f;                               // FP64 form: largest offset error of a candidate
+        // the filter's bound follows the lanes': squared, or for the FP64 form, which
+        // adds a candidate's error, plain
+        float rf = 0.f;
+        auto reach = [&]() {
+            const float r = sqrtf(__uint_as_float(__reduce_max_sync(FULL, root))) * (1.0f + 0x1p-18f);
+            rf = kF32 ? r * r : r;
+        };
+        {
+            box();
+            widest();
+            float f[6] = {act ? q.x : INFINITY,  act ? q.y : INFINITY,  act ? q.z : INFINITY,
+                          act ? -q.x : INFINITY, act ? -q.y : INFINITY, act ? -q.z : INFINITY};
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+                for (int i = 0; i < 6; ++i) f[i] = fminf(f[i], __shfl_xor_sync(FULL, f[i], o));
             }
             __syncwarp();
-        }
-        // filter boxes: groups of 32 / G lanes, in the query leaf's frame (mixed
-        // form) or the halo frame (FP64 form, with the walk's bounds)
-        float r2f[G];
-        float4 flo[G], fhi[G];
-        {
-            float v[6];
-            if constexpr (kF32) {
-                v[0] = active ? (float)q.x : INFINITY;  v[1] = active ? (float)q.y : INFINITY;  v[2] = active ? (float)q.z : INFINITY;
-                v[3] = active ? -(float)q.x : INFINITY; v[4] = active ? -(float)q.y : INFINITY; v[5] = active ? -(float)q.z : INFINITY;
-            } else {
-                v[0] = active ? pq.x : INFINITY;  v[1] = active ? pq.y : INFINITY;  v[2] = active ? pq.z : INFINITY;
-                v[3] = active ? -pq.x : INFINITY; v[4] = active ? -pq.y : INFINITY; v[5] = active ? -pq.z : INFINITY;
+            if (lane == 0) {
+                const float rw = __fadd_ru(__fmul_ru(-w[6], 1.0f + 0x1p-18f), margin);
+                wbox[0] = make_float4(w[0], w[1], w[2], __fmul_ru(rw, rw));
+                wbox[1] = make_float4(-w[3], -w[4], -w[5], 0.f);
+                // centre and half widths; with c = RN(x - centre) the computed gap
+                // |c| - half of a point x exceeds the true one by less than 2^-22 (gap +
+                // half), which the factors here and on the bound cover
+                const float cx = 0.5f * (f[0] - f[3]), cy = 0.5f * (f[1] - f[4]), cz = 0.5f * (f[2] - f[5]);
+                const float s = 1.0f + 0x1p-18f;
+                wbox[2] = make_float4(-cx, -cy, -cz, 0.f);
+                wbox[3] = make_float4(s * fmaxf(-f[3] - cx, cx - f[0]), s * fmaxf(-f[4] - cy, cy - f[1]),
+                                      s * fmaxf(-f[5] - cz, cz - f[2]), 0.f);
             }
-#pragma unroll
-            for (int o = kGL / 2; o > 0; o >>= 1) {
-#pragma unroll
-                for (int i = 0; i < 6; ++i) v[i] = fminf(v[i], __shfl_xor_sync(FULL, v[i], o));
-            }
-#pragma unroll
-            for (int g = 0; g < G; ++g) {
-                flo[g] = make_float4(__shfl_sync(FULL, v[0], g * kGL), __shfl_sync(FULL, v[1], g * kGL),
-                                     __shfl_sync(FULL, v[2], g * kGL), 0.f);
-                fhi[g] = make_float4(-__shfl_sync(FULL, v[3], g * kGL), -__shfl_sync(FULL, v[4], g * kGL),
-                                     -__shfl_sync(FULL, v[5], g * kGL), 0.f);
-            }
+            __syncwarp();
+            reach();
         }
-        // the filter's bounds: the largest bound key of each group (mixed: the
-        // exact bound; FP64: the walk's, with the margin)
-        auto filter_bounds = [&]() {
-            float b = -1.0f;
-            if constexpr (kF32) { if (active) b = key_d2<R, false>(root); }
-            else b = r2walk;
-#pragma unroll
-            for (int o = kGL / 2; o > 0; o >>= 1) b = fmaxf(b, __shfl_xor_sync(FULL, b, o));
-#pragma unroll
-            for (int g = 0; g < G; ++g) r2f[g] = __shfl_sync(FULL, b, g * kGL);
-        };
-        filter_bounds();
-#pragma unroll
-        for (int g = 0; g < G; ++g) {
-            const float ext = fmaxf(fmaxf(fhi[g].x - flo[g].x, fhi[g].y - flo[g].y), fhi[g].z - flo[g].z);
-            spread = spread || (r2f[g] >= 0.f && ext * ext > kSpreadFilter * kSpreadFilter * r2f[g]);
-        }
-        if (__any_sync(FULL, spread)) {
-            if (lane == 0) { const unsigned r = atomicAdd(redo_len, 1u); redo_list[r] = leaf; }
-            continue;
-        }
-        // zero the slots after the heap of this leaf's k
-        for (int i = 0; i < kWPad; ++i) keys[(k + i) * 32 + lane] = K(0);
-
-        int cnt = 0;                                   // keys held (slots 0..k-1, then k+3..)
-        bool heaped = false;
+        // the query, negated, in both halves; lanes outside the run admit nothing
+        const unsigned long long qx2 = pack2(-q.x, -q.x), qy2 = pack2(-q.y, -q.y), qz2 = pack2(-q.z, -q.z);
+        const unsigned off0 = (unsigned)sizeof(K) * lane;
+        unsigned off = off0;                           // end of the lane's keys (bytes)
+        const unsigned room = off0 + kRow * (unsigned)(kk + kWPend - kWBatch);
+        bool heaped = false, dropped = false;
+        auto at = [&](int t) -> K& { return *(K*)(keys + off0 + kRow * (unsigned)t); };
         auto sift = [&](int t, K key) {
             while (true) {
                 const int c0 = 4 * t + 1;
-                if (c0 >= k) break;
-                const K* cp = keys + (size_t)c0 * 32 + lane;
-                K m = cp[0];
-                int j = 0;
-                const K c1 = cp[32], c2 = cp[64], c3 = cp[96];
-                if (c1 > m) { m = c1; j = 1; }
-                if (c2 > m) { m = c2; j = 2; }
-                if (c3 > m) { m = c3; j = 3; }
+                if (c0 >= kk) break;
+                K m = at(c0);
+                int j = c0;
+#pragma unroll
+                for (int u = 1; u < 4; ++u) {
+                    const K c = c0 + u < kk ? at(c0 + u) : K(0);
+                    if (c > m) { m = c; j = c0 + u; }
+                }
                 if (!(m > key)) break;
-                keys[t * 32 + lane] = m;
-                t = c0 + j;
+                at(t) = m;
+                t = j;
             }
-            keys[t * 32 + lane] = key;
+            at(t) = key;
         };
+        auto bits = [](K key) -> uint32_t { if constexpr (kF32) return key; else return (uint32_t)(key >> 32); };
         // merge the waiting keys into the heap (each lane its own column)
         auto flush = [&]() {
-            if (active && cnt >= k) {
+            const int cnt = (int)((off - off0) / kRow);
+            if (cnt >= kk) {
                 if (!heaped) {
-                    for (int t = (k - 2) / 4; t >= 0; --t) sift(t, keys[t * 32 + lane]);
+                    for (int t = (kk - 2) / 4; t >= 0; --t) sift(t, at(t));
                     heaped = true;
-                    root = keys[lane];
                 }
-                for (int i = k; i < cnt; ++i) {
-                    const K key = keys[(i + kWPad) * 32 + lane];
-                    if (key < root) {
+                for (int i = kk; i < cnt; ++i) {
+                    const K key = at(i);
+                    if (key < at(0)) {
                         ++n_ins;
                         sift(0, key);
-                        root = keys[lane];
                     }
                 }
-                cnt = k;
+                dropped = dropped || cnt > kk;
+                root = min(root, bits(at(0)) + (kF32 ? 0u : 1u));   // FP64 form: equal FP32 distances still enter
+                off = off0 + kRow * (unsigned)kk;
             }
-            filter_bounds();
+            reach();
         };
-        // distances from every query to the kWBatch entries at src
-        auto batch = [&](const V* src, bool self) {
-            if (__any_sync(FULL, cnt > k + kWPend - kWBatch)) flush();
-            __syncwarp();
-#pragma unroll
-            for (int t = 0; t < kWBatch; t += 4) {
-                K key[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const V cj = src[t + u];
-                    const R dx = sub_rn(cj.x, q.x), dy = sub_rn(cj.y, q.y), dz = sub_rn(cj.z, q.z);
-                    key[u] = make_key<R, false>(fma_rn(dz, dz, fma_rn(dy, dy, mul_rn(dx, dx))), 0u);
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const bool adm = key[u] < root && !(self && t + u == (lane & (kWBatch - 1)));
-                    const int slot = cnt < k ? cnt : cnt + kWPad;
-                    keys[slot * 32 + lane] = key[u];
-                    cnt += adm ? 1 : 0;
-                }
-            }
-            __syncwarp();
-        };
-        V far;
-        far.x = R(INFINITY); far.y = R(INFINITY); far.z = R(INFINITY); far.w = R(0);
 
-        // 1) the query leaf's own particles, two batches of 16 (lanes past the
-        //    leaf's end read as infinitely far)
-        ring[lane] = active ? q : far;
+        // the accepted children of a node: local leaf indices into the list (this
+        // part's share), or nodes onto the stack
+        int nl = 0, seen = 0, sp = 0;
+        if (part == 0) { if (lane == 0) list[0] = A; nl = 1; }   // the query leaf first
         __syncwarp();
-        if (active) n_cand += (unsigned long long)countA;
-#pragma unroll
-        for (int b = 0; b < kLeaf; b += kWBatch) batch(ring + b, (lane & ~(kWBatch - 1)) == b);
-        __syncwarp();
-
-        // 2) stream listed leaves: filter, append to the ring, run full batches
-        int head = 0, tail = 0, navail = 0;
-        auto wrap = [](int i) { return i >= kWRing ? i - kWRing : i; };   // i < 2 kWRing
-        auto stage_leaf = [&](int Bl, V c, float4 cB) {
-            const int countB = (int)min((int64_t)kLeaf, nh - (int64_t)Bl * kLeaf);
-            bool reach = false;
-            if constexpr (kF32) {
-                c.x = __fadd_rn(c.x, __fsub_rn(cB.x, cA.x));     // exact shift into the query leaf's frame
-                c.y = __fadd_rn(c.y, __fsub_rn(cB.y, cA.y));
-                c.z = __fadd_rn(c.z, __fsub_rn(cB.z, cA.z));
-                const float3 pc = make_float3(c.x, c.y, c.z);
-#pragma unroll
-                for (int g = 0; g < G; ++g) reach = reach || point_gap2_rd(pc, flo[g], fhi[g]) <= r2f[g];
+        auto visit = [&](int lev, int first, int nb, int n) {
+            float4 lo = make_float4(INFINITY, INFINITY, INFINITY, 0.f), hi = lo;
+            const bool in = lane < n && !(lev == 0 && first + lane == A);
+            if (in) { lo = p.nlo[nb + first + lane]; hi = p.nhi[nb + first + lane]; }
+            const float4 qlo = wbox[0];
+            uint32_t acc = __ballot_sync(FULL, in && box_gap2_rd(qlo, wbox[1], lo, hi) <= qlo.w);
+            if (lev == 0) {
+                const bool mine = ((acc >> lane) & 1u) && ((seen + __popc(acc & lt)) & (nw - 1)) == part;
+                seen += __popc(acc);
+                acc = __ballot_sync(FULL, mine);
+                if (mine) list[nl + __popc(acc & lt)] = first + lane;
+                nl += __popc(acc);
+            } else if (sp + __popc(acc) > kStack) {
+                bad = true;
             } else {
-                const float3 pc = make_float3(__double2float_rn((double)c.x - fr.O[0]),
-                                              __double2float_rn((double)c.y - fr.O[1]),
-                                              __double2float_rn((double)c.z - fr.O[2]));
-#pragma unroll
-                for (int g = 0; g < G; ++g) reach = reach || point_gap2_rd(pc, flo[g], fhi[g]) <= r2f[g];
+                sp += __popc(acc);
+                if ((acc >> lane) & 1u) stack[sp - 1 - __popc(acc & lt)] = (lev << 24) | (first + lane);
             }
-            const uint32_t m = __ballot_sync(FULL, lane < countB && reach);
-            ++n_tiles;
-            if (m == 0u) return;
-            if ((m >> lane) & 1u) ring[wrap(tail + __popc(m & lt))] = c;
-            const int nm = __popc(m);
-            tail = wrap(tail + nm);
-            navail += nm;
-            __syncwarp();
-            while (navail >= kWBatch) {
-                if (active) n_cand += (unsigned long long)kWBatch;
-                batch(ring + head, false);
-                head = wrap(head + kWBatch);
-                navail -= kWBatch;
-            }
-        };
-        int nl = 0;
-        auto stream_list = [&]() {
-            using CellT = float4;
-            V c0{}, c1{};
-            CellT b0{}, b1{};
-            auto fetch = [&](int i, V& c, CellT& b) {
-                const int Bl = list[i];
-                c = ((const V*)p.P4)[(int64_t)(leaf0 + Bl) * kLeaf + lane];
-                if constexpr (kF32) b = p.cell[leaf0 + Bl];
-            };
-            if (nl > 0) fetch(0, c0, b0);
-            if (nl > 1) fetch(1, c1, b1);
-            for (int i = 0; i < nl; ++i) {
-                V c2{};
-                CellT b2{};
-                if (i + 2 < nl) fetch(i + 2, c2, b2);
-                stage_leaf(list[i], c0, b0);
-                c0 = c1; b0 = b1; c1 = c2; b1 = b2;
-            }
-            nl = 0;
             __syncwarp();
         };
-        // tree walk, level by level: the accepted nodes of a level form the
-        // frontier of the next; the child boxes of the next frontier node are
-        // loaded while the current node's children are tested (one child per
-        // lane, against every walk group's box grown by its bound)
-        auto accept = [&](int n, float4 clo, float4 chi) -> uint32_t {
-            bool ok = false;
-            if (lane < n) {
-#pragma unroll
-                for (int g = 0; g < kWalkGroups; ++g) {
-                    const float4 lo = wbox[2 * g];
-                    ok = ok || box_gap2_rd(lo, wbox[2 * g + 1], clo, chi) <= lo.w;
-                }
-            }
-            return __ballot_sync(FULL, ok);
-        };
-        auto add_leaves = [&](uint32_t acc, int first) {
-            if (nl + __popc(acc) > kWList) stream_list();
-            if ((acc >> lane) & 1u) list[nl + __popc(acc & lt)] = first + lane;
-            nl += __popc(acc);
-            __syncwarp();
-        };
-        bool overflow = false;
-        constexpr int kWFront = kWStack / 2;
-        int* front = fbuf;
-        int* nextf = fbuf + kWFront;
-        int nf = 0;
         const int top = p.top[h];
-        const int32_t* loff = p.lvl_off;
-        {
-            const int nb0 = loff[top * Hp + h];
-            const int ntop = loff[top * Hp + h + 1] - nb0;
-            float4 clo = make_float4(0.f, 0.f, 0.f, 0.f), chi = clo;
-            if (lane < ntop) { clo = p.nlo[nb0 + lane]; chi = p.nhi[nb0 + lane]; }
-            const uint32_t acc = accept(ntop, clo, chi);
-            if (top == 0) {
-                add_leaves(acc & ~(1u << A), 0);
+        bool started = false;
+        // ring entries: candidate numbers cnum .. cnum + navail - 1; entries of the
+        // query leaf still in the ring, and this lane's own number
+        int navail = 0, nself = 0, li = 0;
+        uint32_t cnum = 0u;
+        while (true) {
+            bool fin = false;
+            if (li < nl) {
+                // two listed leaves: shift, filter, append to the ring
+                const int Bl[2] = {list[li], list[min(li + 1, nl - 1)]};
+                float4 c[2], cB[2];
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    c[u] = S4[(uint32_t)(leaf0 + Bl[u]) * kLeaf + lane];
+                    cB[u] = p.cell[leaf0 + Bl[u]];
+                }
+                const float4 fc = wbox[2], fw = wbox[3];
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    c[u].x = __fadd_rn(c[u].x, __fsub_rn(cB[u].x, cA.x));     // exact shift into the query leaf's frame
+                    c[u].y = __fadd_rn(c[u].y, __fsub_rn(cB[u].y, cA.y));
+                    c[u].z = __fadd_rn(c[u].z, __fsub_rn(cB[u].z, cA.z));
+                    const float gx = fmaxf(fabsf(c[u].x + fc.x) - fw.x, 0.f), gy = fmaxf(fabsf(c[u].y + fc.y) - fw.y, 0.f),
+                                gz = fmaxf(fabsf(c[u].z + fc.z) - fw.z, 0.f);
+                    const float re = rf + c[u].w, r2 = kF32 ? rf : re * re;
+                    // the query leaf's entries all stay: their numbers are their lanes
+                    const bool self = u == 0 && Bl[0] == A;
+                    const bool keep = (uint32_t)Bl[u] * kLeaf + lane < nh && li + u < nl &&
+                                      (gx * gx + gy * gy + gz * gz <= r2 || self);
+                    const uint32_t m = __ballot_sync(FULL, keep);
+                    if (self) nself = __popc(m);
+                    if constexpr (!kF32) err = fmaxf(err, keep ? c[u].w : 0.f);
+                    if (keep) {
+                        float* e = ring + ((cnum + navail + __popc(m & lt)) & (kWRing - 1));
+                        e[0] = c[u].x; e[kWRing] = c[u].y; e[2 * kWRing] = c[u].z;
+                        if constexpr (!kF32) e[3 * kWRing] = __uint_as_float((uint32_t)(leaf0 + Bl[u]) * kLeaf + lane);
+                    }
+                    navail += __popc(m);
+                }
+                n_tiles += (unsigned long long)min(2, nl - li);
+                li += 2;
+                __syncwarp();
+            } else if (!started || sp > 0) {
+                // walk until the list may not hold another node's leaves, or the tree is done
+                nl = li = 0;
+                if (!started) {
+                    const int nb = p.lvl_off[top * Hp + h];
+                    visit(top, 0, nb, p.lvl_off[top * Hp + h + 1] - nb);
+                    started = true;
+                }
+                while (sp > 0 && nl <= kWList - kArity && !bad) {
+                    const int e = stack[--sp];
+                    __syncwarp();
+                    const int cl = (e >> 24) - 1, first = (e & 0xFFFFFF) * kArity;
+                    const int cb = p.lvl_off[cl * Hp + h];
+                    visit(cl, first, cb, min(kArity, p.lvl_off[cl * Hp + h + 1] - cb - first));
+                }
             } else {
-                if ((acc >> lane) & 1u) front[__popc(acc & lt)] = lane;
-                nf = __popc(acc);
+                // at the very end fill the partial batch with infinitely far entries
+                fin = true;
+                const int fill = (kWBatch - navail % kWBatch) % kWBatch;
+                if (lane < fill) {
+                    float* e = ring + ((cnum + navail + lane) & (kWRing - 1));
+                    e[0] = INFINITY; e[kWRing] = INFINITY; e[2 * kWRing] = INFINITY;
+                }
+                navail += fill;
                 __syncwarp();
             }
-        }
-        for (int lev = top; lev > 0 && nf > 0 && !overflow; --lev) {
-            const int cl = lev - 1;
-            const int cb = loff[cl * Hp + h];
-            const int cc = loff[cl * Hp + h + 1] - cb;
-            int nn = 0;
-            float4 lo0 = make_float4(0.f, 0.f, 0.f, 0.f), hi0 = lo0;
-            auto load = [&](int i, float4& lo, float4& hi) {
-                const int first = front[i] * kArity;
-                if (lane < min(kArity, cc - first)) { lo = p.nlo[cb + first + lane]; hi = p.nhi[cb + first + lane]; }
-            };
-            load(0, lo0, hi0);
-            for (int i = 0; i < nf; ++i) {
-                float4 lo1 = make_float4(0.f, 0.f, 0.f, 0.f), hi1 = lo1;
-                if (i + 1 < nf) load(i + 1, lo1, hi1);
-                const int first = front[i] * kArity;
-                const int nch = min(kArity, cc - first);
-                uint32_t acc = accept(nch, lo0, hi0);
-                if (cl == 0) {
-                    if (A >= first && A < first + nch) acc &= ~(1u << (A - first));
-                    add_leaves(acc, first);
-                } else {
-                    const int na = __popc(acc);
-                    if (nn + na > kWFront) { overflow = true; break; }
-                    if ((acc >> lane) & 1u) nextf[nn + __popc(acc & lt)] = first + lane;
-                    nn += na;
+            if (bad) break;
+            while (navail >= kWBatch) {
+                if (__any_sync(FULL, off > room)) flush();
+                const bool own = nself > 0;
+                const int me = own ? lane - (int)cnum : -1;   // this lane's own entry in the batch
+#pragma unroll
+                for (int t = 0; t < kWBatch; t += 4) {
+                    const float* e = ring + (cnum & (kWRing - 1)) + t;
+                    const ulonglong2 x = *(const ulonglong2*)e, y = *(const ulonglong2*)(e + kWRing),
+                                     z = *(const ulonglong2*)(e + 2 * kWRing);
+                    uint4 sl = make_uint4(0u, 0u, 0u, 0u);
+                    if constexpr (!kF32) sl = *(const uint4*)(e + 3 * kWRing);
+                    const uint32_t s4[4] = {sl.x, sl.y, sl.z, sl.w};
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        const unsigned long long dx = add2(u ? x.y : x.x, qx2), dy = add2(u ? y.y : y.x, qy2),
+                                                 dz = add2(u ? z.y : z.x, qz2);
+                        const unsigned long long d2 = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
+                        const uint32_t db[2] = {(uint32_t)d2, (uint32_t)(d2 >> 32)};
+#pragma unroll
+                        for (int r = 0; r < 2; ++r) {
+                            const int i = t + 2 * u + r;
+                            if constexpr (kF32) *(uint32_t*)(keys + off) = db[r];
+                            else *(unsigned long long*)(keys + off) = ((unsigned long long)db[r] << 32) | s4[2 * u + r];
+                            off += db[r] < root && i != me ? kRow : 0u;
+                        }
+                    }
                 }
-                lo0 = lo1; hi0 = hi1;
+                if (act) n_cand += kWBatch;
+                cnum += kWBatch;
+                navail -= kWBatch;
+                nself -= kWBatch;
+                __syncwarp();
             }
-            __syncwarp();
-            int* t = front; front = nextf; nextf = t;
-            nf = nn;
+            if (fin) break;
         }
-        stream_list();
-        // the last, partial batch: pad it with infinitely far entries
-        if (navail > 0) {
-            if (lane < kWBatch - navail) ring[wrap(tail + lane)] = far;
-            __syncwarp();
-            if (active) n_cand += (unsigned long long)navail;
-            batch(ring + head, false);
+        // the first warp takes over the other warps' keys
+        if constexpr (TEAM) {
+            flush();
+            held[lane] = (int)((off - off0) / kRow);
+            if (dropped) held[lane] |= 0x10000;
+            if (!kF32) atomicMax(&team_err, __float_as_uint(err));
+            if (bad && lane == 0) atomicOr(&team_bad, 1u);
+            __syncthreads();
+            bad = team_bad != 0u;
+            if (!kF32) err = __uint_as_float(team_err);
+            if (wid == 0 && !bad) {
+                for (int w = 1; w < nw; ++w) {
+                    const int hw = *(const int*)((const unsigned char*)(held + lane) + w * warp_bytes);
+                    dropped = dropped || (hw & 0x10000);
+                    const unsigned char* src = keys + w * warp_bytes + off0;
+                    const int most = __reduce_max_sync(FULL, hw & 0xffff);
+                    for (int i = 0; i < most; ++i) {
+                        if (__any_sync(FULL, off > room)) flush();
+                        if (i < (hw & 0xffff)) {
+                            const K key = *(const K*)(src + kRow * (unsigned)i);
+                            *(K*)(keys + off) = key;
+                            off += bits(key) < root ? kRow : 0u;
+                            dropped = dropped || bits(key) >= root;
+                        }
+                    }
+                }
+            }
         }
-        flush();
-        const bool ok = !active || heaped;
-        if (overflow || !__all_sync(FULL, ok)) {
-            if (lane == 0) { const unsigned r = atomicAdd(redo_len, 1u); redo_list[r] = leaf; }
-        } else if (active) {
-            const int64_t u = hb + (int64_t)A * kLeaf + lane;
-            const R hval = sqrt_rn(key_d2<R, false>(root));
-            ((R*)p.h_out)[u] = hval;
-            ((R*)((V*)p.P4 + (int64_t)leaf * kLeaf + lane))[3] = hval;
-            if (p.hprev) ((R*)p.hprev)[u] = hval;
+        uint32_t fail = 0u;                            // lanes that try again
+        if (!bad && part == 0) {
+            flush();
+            const int n = (int)((off - off0) / kRow);
+            bool ok = !act || n >= k, again = !ok;
+            R hval = R(0);
+            if constexpr (!kF32) {
+                // every FP32 distance is within `err` of the exact one
+                err = q.w + __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(err))) + 0x1p-19f * rad;
+            }
+            if constexpr (kF32) {
+                if (act && ok) hval = sqrt_rn(__uint_as_float(at(0)));
+            } else if (act && ok) {
+                // the k-th smallest FP32 distance: the (n - k + 1)-th largest of the n kept
+                float v[kWExtra + 1];
+#pragma unroll
+                for (int j = 0; j <= kWExtra; ++j) v[j] = -1.f;
+                for (int i = 0; i < n; ++i) {
+                    float x = __uint_as_float(bits(at(i)));
+#pragma unroll
+                    for (int j = 0; j <= kWExtra; ++j) { const float y = fmaxf(v[j], x); x = fminf(v[j], x); v[j] = y; }
+                }
+                float dk = v[0];
+#pragma unroll
+                for (int j = 1; j <= kWExtra; ++j) if (n - k == j) dk = v[j];
+                // candidates that may come before, or after, the k-th exact distance
+                dk = sqrtf(dk);
+                const float lo = dk - 2.f * err, hi = dk + 2.f * err;
+                const float lo2 = lo > 0.f ? lo * lo * (1.0f - 0x1p-20f) : -1.f, hi2 = hi * hi * (1.0f + 0x1p-20f);
+                ok = dropped ? v[0] > hi2 : hi2 < rad * rad * (1.0f - 0x1p-20f);
+                again = !ok && !dropped;
+                if (ok) {
+                    const V qd = P4[slotA];
+                    int below = 0, nb = 0;
+                    double d2[kWBand];
+                    for (int j = 0; j < kWBand; ++j) d2[j] = INFINITY;
+                    for (int i = 0; i < n; ++i) {
+                        const K key = at(i);
+                        const float x = __uint_as_float(bits(key));
+                        if (x < lo2) { ++below; continue; }
+                        if (x > hi2) continue;
+                        const V pj = P4[(uint32_t)key];
+                        const double dx = sub_rn((double)pj.x, (double)qd.x), dy = sub_rn((double)pj.y, (double)qd.y),
+                                     dz = sub_rn((double)pj.z, (double)qd.z);
+                        double e = fma_rn(dz, dz, fma_rn(dy, dy, mul_rn(dx, dx)));
+#pragma unroll
+                        for (int j = 0; j < kWBand; ++j) { const double y = fmin(d2[j], e); e = fmax(d2[j], e); d2[j] = y; }
+                        ++nb;
+                    }
+                    ok = nb <= kWBand && k - below >= 1 && k - below <= nb;
+                    double e = d2[0];
+#pragma unroll
+                    for (int j = 1; j < kWBand; ++j) if (k - below - 1 == j) e = d2[j];
+                    hval = (R)sqrt_rn(e);
+                }
+            }
+            fail = __ballot_sync(FULL, again);
+            if (__any_sync(FULL, !ok && !again) || (fail && attempt == kWAttempts - 1)) bad = true;
+            if (act && ok) {
+                const int64_t u = p.halo_off[h] + (int64_t)slotA - (int64_t)leaf0 * kLeaf;
+                ((R*)p.h_out)[u] = hval;
+                if (p.hprev) ((R*)p.hprev)[u] = hval;
+                ((R*)((V*)p.P4 + slotA))[3] = hval;
+            }
+            if (attempt == 0) n_again += (unsigned long long)__popc(fail);
         }
+        if constexpr (TEAM) {
+            if (wid == 0 && lane == 0) { team_fail = fail; if (bad) team_bad = 1u; }
+            __syncthreads();
+            fail = team_fail;
+            bad = team_bad != 0u;
+        }
+        if (bad || fail == 0u) break;
+        act = (fail >> lane) & 1u;
+        if (act) rad *= 1.5f;
+        }   // attempts
+        if (bad) break;
+        }   // runs of queries
+        if (bad && part == 0 && lane == 0) { const unsigned r = atomicAdd(redo_len, 1u); redo_list[r] = leaf; }
         n_tiles_max = n_tiles - tiles0 > n_tiles_max ? n_tiles - tiles0 : n_tiles_max;
         __syncwarp();
     }
@@ -1117,6 +1188,7 @@ __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p,
         atomicAdd(&p.cnt->diag[1], n_cand);
         atomicAdd(&p.cnt->diag[2], n_ins);
         atomicMax(&p.cnt->diag[3], n_tiles_max);
+        if (n_again) atomicAdd(&p.cnt->diag[7], n_again);
     }
 }
 
@@ -1127,6 +1199,7 @@ void fill_params(sidm_ctx* c, KnnParams& p, void* h_out, uint32_t* nbr, int k_st
     p.leaf_halo = c->d_leaf_halo; p.leaf_off = c->d_leaf_off; p.halo_off = c->d_halo_off;
     p.lvl_off = c->d_lvl_off; p.top = c->d_top; p.ngb = c->d_ngb; p.frame = c->d_frame;
     p.cell = c->d_cell; p.nlo = c->d_nlo; p.nhi = c->d_nhi; p.P4 = c->d_P4; p.ID = c->d_ID;
+    p.S4 = c->cfg.precision == SIDM_FP64 ? (const void*)c->d_S4 : c->d_P4;
     p.h_out = h_out; p.nbr = nbr; p.k_stride = k_stride; p.kcap = c->kmax_cur; p.cnt = c->d_cnt;
     p.work = &c->d_cnt->work[0];
     p.leaf_list = nullptr; p.list_len = nullptr;
@@ -1208,35 +1281,42 @@ int launch_tuned(sidm_ctx* c, void* h_out, bool use_guess, cudaStream_t s, bool 
 
 // warm-started search with the fixed-bound kernel, then the per-lane search
 // (itself warm-started: a lane whose guess fails there is redone cold) of the
-// leaves it could not finish or left to it
-template <class R, int G>
+// leaves it could not finish.  With fewer than kTeamItems leaves per resident
+// warp the warps of a CTA share a leaf.
+constexpr int64_t kTeamItems = 1;
+template <class R>
 int launch_warm(sidm_ctx* c, void* h_out, cudaStream_t s)
 {
-    using K = typename KeyOf<R, false>::T;
     KnnParams p;
     fill_params(c, p, h_out, nullptr, 0, true);
-    auto kern = k_knn_warm<R, G>;
-    const size_t per_warp = warm_warp_bytes<R, K, G>(p.kcap);
+    const size_t per_warp = warm_warp_bytes<R>(p.kcap);
     int warps = 0, grid = 0;
-    if (int rc = pick_shape(c, (const void*)kern, per_warp, &warps, &grid, kWarmMaxWarps)) return rc;
+    if (int rc = pick_shape(c, (const void*)k_knn_warm<R, false>, per_warp, &warps, &grid, kWarmMaxWarps)) return rc;
+    bool team = false;
+    if (c->lay.L < kTeamItems * grid * warps) {
+        int w = kWarmMaxWarps;
+        while (w > 1 && (w > c->knn_warps || (size_t)w * per_warp > (size_t)226 * 1024)) w /= 2;
+        int occ = 0;
+        if (int rc = occupancy(c, (const void*)k_knn_warm<R, true>, w * 32, (size_t)w * per_warp, &occ)) return rc;
+        if (occ >= 1 && w > 1) {
+            team = true;
+            warps = w;
+            grid = c->cfg.grid_ctas > 0 ? c->cfg.grid_ctas : c->sm_count * occ;
+            grid = std::max(1, std::min(grid, c->lay.L));
+        }
+    }
     c->knn_grid = grid;
     cudaError_t e = cudaMemsetAsync(&c->d_cnt->work[0], 0, sizeof(unsigned int), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(&c->d_cnt->knn_redo[0], 0, 2 * sizeof(unsigned int), s);
     if (e != cudaSuccess) return cuda_check(c, e, "knn work reset");
     const int tidx = timer_begin(c, 1, s);
-    kern<<<grid, warps * 32, (size_t)warps * per_warp, s>>>(p, c->d_knn_redo, &c->d_cnt->knn_redo[0]);
+    if (team) k_knn_warm<R, true><<<grid, warps * 32, (size_t)warps * per_warp, s>>>(p, c->d_knn_redo, &c->d_cnt->knn_redo[0]);
+    else k_knn_warm<R, false><<<grid, warps * 32, (size_t)warps * per_warp, s>>>(p, c->d_knn_redo, &c->d_cnt->knn_redo[0]);
     timer_end(c, tidx, s);
     c->launches++;
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_check(c, e, "knn launch");
     return launch_tuned<R>(c, h_out, true, s, true);
-}
-
-template <class R>
-int launch_warm_tuned(sidm_ctx* c, void* h_out, cudaStream_t s)
-{
-    const int g = c->cfg.knn_groups > 0 ? c->cfg.knn_groups : kGroupsDefault;
-    return g == 2 ? launch_warm<R, 2>(c, h_out, s) : launch_warm<R, 4>(c, h_out, s);
 }
 
 }  // namespace
@@ -1251,13 +1331,13 @@ int launch_knn(sidm_ctx* c, void* h_out, uint32_t* nbr, int k_stride, bool use_g
     const bool warm = use_guess && !tma && (c->cfg.knn_batch > 0 ? c->cfg.knn_batch : kBatchDefault) == 3;
     if (c->cfg.precision == SIDM_FP64) {
         if (nbr) return set_err(c, SIDM_EINVAL, "neighbour lists: mixed form only");
-        if (warm) return launch_warm_tuned<double>(c, h_out, s);
+        if (warm) return launch_warm<double>(c, h_out, s);
         return tma ? launch_t<double, false, true, G, CH>(c, h_out, nullptr, 0, use_guess, s)
                    : launch_tuned<double>(c, h_out, use_guess, s);
     }
     if (nbr) return tma ? launch_t<float, true, true, G, CH>(c, nullptr, nbr, k_stride, false, s)
                         : launch_t<float, true, false, G, CH>(c, nullptr, nbr, k_stride, false, s);
-    if (warm) return launch_warm_tuned<float>(c, h_out, s);
+    if (warm) return launch_warm<float>(c, h_out, s);
     return tma ? launch_t<float, false, true, G, CH>(c, h_out, nullptr, 0, use_guess, s)
                : launch_tuned<float>(c, h_out, use_guess, s);
 }

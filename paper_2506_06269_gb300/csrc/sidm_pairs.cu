@@ -637,36 +637,6 @@ static_assert(draw_warp_bytes() % 16 == 0 && (kPList + kStack) % 4 == 0 && kPQue
 // max over v of sigma(v) v / s0 for kind 1: v / (1 + (v/w)^2)^2 peaks at v = w / sqrt(3)
 constexpr float kSvMax = 0.32475953f;    // 3 sqrt(3) / 16, rounded up
 
-// packed pairs of FP32 (each half rounded to nearest like the scalar operation)
-__device__ __forceinline__ unsigned long long pack2(float a, float b)
-{
-    unsigned long long r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ void unpack2(unsigned long long v, float& a, float& b)
-{
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-}
-__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b)
-{
-    unsigned long long r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b)
-{
-    unsigned long long r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c)
-{
-    unsigned long long r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-
 template <class R, int MODE, int PR, bool DRAG>
 __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
 {
