@@ -1816,12 +1816,14 @@ static int scatter_impl(sidm_ctx* c, uint64_t seed, uint64_t step, const sidm_xs
     c->stepped = true;
     if (L.N == 0) return SIDM_OK;
     const bool fp64 = c->cfg.precision == SIDM_FP64;
-    if (fp64)
-        SIDM_LAUNCH(c, k_vel_refresh<double><<<grid_for(c, L.N, 256), 256, 0, s>>>(L.N, L.H, c->d_halo_off, c->d_halo_pad,
-                                                                                  (const double*)vel, c->d_ID, (double4_16a*)c->d_V4));
-    else if (c->cfg.flags & (SIDM_FLAG_SUM_P | SIDM_FLAG_DRAG))   // plain draws read a few velocities only
-        SIDM_LAUNCH(c, k_vel_refresh<float><<<grid_for(c, L.N, 256), 256, 0, s>>>(L.N, L.H, c->d_halo_off, c->d_halo_pad,
-                                                                                (const float*)vel, c->d_ID, (float4*)c->d_V4));
+    if (c->cfg.flags & (SIDM_FLAG_SUM_P | SIDM_FLAG_DRAG)) {         // plain draws read a few velocities only
+        if (fp64)
+            SIDM_LAUNCH(c, k_vel_refresh<double><<<grid_for(c, L.N, 256), 256, 0, s>>>(
+                L.N, L.H, c->d_halo_off, c->d_halo_pad, (const double*)vel, c->d_ID, (double4_16a*)c->d_V4));
+        else
+            SIDM_LAUNCH(c, k_vel_refresh<float><<<grid_for(c, L.N, 256), 256, 0, s>>>(
+                L.N, L.H, c->d_halo_off, c->d_halo_pad, (const float*)vel, c->d_ID, (float4*)c->d_V4));
+    }
     int rc = launch_pairs(c, seed, step, xs, dt, mass, vel, st, s);
     if (rc) return rc;
     const int use_sump = (c->cfg.flags & SIDM_FLAG_SUM_P) ? 1 : 0;

@@ -34,6 +34,7 @@ struct PairParams {
     const float4* nlo;
     const float4* nhi;
     const void* P4;
+    const void* S4;     // FP32 offsets and reach: mixed form P4, FP64 form see k_leaf_hmax
     const void* V4;
     const uint32_t* ID;
     const void* vel;    // the caller's velocities [3][N] (unchanged until the resolve)
@@ -590,7 +591,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_pairs_queue(Pai
     st_pos.finish(lane, p.cnt);
 }
 
-// ---------------------------------------------------------------- draws, mixed form
+// ---------------------------------------------------------------- draws
 // Most in-range pairs never come near an event (P ~ 1e-6 .. 1e-4), and whether
 // a draw can fire at all is decided by integers: P_ij <= T 2^-32 for every pair
 // of a query leaf, with T from the largest sigma(v) v and Lambda <= 4 / h_i^3
@@ -608,7 +609,13 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_pairs_queue(Pai
 //  * one warp scan of the masks' bit counts per batch gives every lane its place
 //    in the warp's queue of (query lane, candidate) pairs, which is emptied 32
 //    pairs at a time, all lanes busy.
-// Issue-bound (2.8 of 4 instructions per cycle): 1.94 ms per launch for the 2^20
+// The FP64 form runs the same search on FP32 offsets (S4: reach w = h and the
+// rounding errors' bound, k_leaf_hmax), where a pair is out of range, in range
+// for certain, or (about 1 in 10^3) settled by its FP64 distance before its draw;
+// only pairs whose draw can fire take FP64 arithmetic.  2^20 NFW halo: 2.8 ms
+// per launch against 39 ms with every test and P on the FP64 pipe, 16384
+// particles 0.13 against 1.30 ms.
+// Issue-bound (2.8 of 4 instructions per cycle): mixed form 1.94 ms per launch for the 2^20
 // NFW halo at N_ngb = 64 (3.28 ms before), 2.65e8 in-range pairs, 1.24e9 tests.
 // Filling the queue in rounds of ballots and forming sigma(v) and
 // a bound of P for every pair, with masked tests, took 331 lane instructions
@@ -634,6 +641,8 @@ constexpr size_t draw_warp_bytes()
 }
 static_assert(draw_warp_bytes() % 16 == 0 && (kPList + kStack) % 4 == 0 && kPQueue % 8 == 0, "16-byte aligned parts");
 
+constexpr uint32_t kUnsure = 0x80000000u;   // on a candidate's id (below 2^27): its pairs are settled in FP64
+
 // max over v of sigma(v) v / s0 for kind 1: v / (1 + (v/w)^2)^2 peaks at v = w / sqrt(3)
 constexpr float kSvMax = 0.32475953f;    // 3 sqrt(3) / 16, rounded up
 
@@ -657,7 +666,9 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
     uint16_t* queue = (uint16_t*)(wst + 8);
     if (lane < 8) wst[lane] = 0ull;
     const R* __restrict__ T = (const R*)p.lam;
+    constexpr bool kF32 = sizeof(R) == 4;
     const V* __restrict__ P4 = (const V*)p.P4;
+    const float4* __restrict__ S4 = (const float4*)p.S4;
     const V* __restrict__ V4 = (const V*)p.V4;
     const uint32_t lt = (1u << lane) - 1u;
     const int Hp = p.H + 1;
@@ -692,7 +703,10 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
             if (lane == 0) raise_status(p.cnt, SIDM_DEV_BAD_INPUT);
             continue;
         }
-        const float4 q = P4[slotA];
+        float4 q = S4[slotA];
+        // FP64 form: a pair below this share of (w_i + w_j)^2 is in range for certain
+        const float sure = kF32 ? 1.f : q.w < 0.f ? 0.f : 1.0f - 0x1p-11f;
+        if constexpr (!kF32) q.w = fabsf(q.w);
         // the draws' integer bound: no pair's P exceeds thr 2^-32 - 2e-6 (the factor
         // 1.001 and the 3e-6 cover every rounding and the |P - u| < 1e-6 count); a
         // bound that is not a number below one keeps every pair
@@ -719,7 +733,7 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
             } else {
                 dtl = p.dt[h];
             }
-            const float inv = 1.f / q.w;
+            const float inv = 1.f / (kF32 ? q.w : (1.0f - 0x1p-20f) * (float)P4[slotA].w);
             const float b = (float)(xs.s0 * p.mass[h] * dtl) * sv * (kLamFUp * inv * inv * inv) * 1.001f + 3e-6f;
             uint32_t t = FULL;
             if (b < 1.f) t = (uint32_t)(fmaxf(b, 3e-6f) * 4294967296.f) + 1u;
@@ -739,6 +753,19 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
         };
         constexpr bool kEvery = MODE == kModeDrawExact || DRAG;
         const Factors fac = kEvery ? factors() : Factors{};
+        // canonical d^2 of query pi and candidate pj (mixed form: the candidate
+        // shifted into the query leaf's frame)
+        auto pair_d2 = [&](const V& pi, const V& pj, uint32_t sj) -> R {
+            R cx = pj.x, cy = pj.y, cz = pj.z;
+            if constexpr (kF32) {
+                const float4 cj = p.cell[sj / kLeaf];
+                cx = __fadd_rn(cx, __fsub_rn(cj.x, cA.x));
+                cy = __fadd_rn(cy, __fsub_rn(cj.y, cA.y));
+                cz = __fadd_rn(cz, __fsub_rn(cj.z, cA.z));
+            }
+            const R dx = sub_rn(cx, pi.x), dy = sub_rn(cy, pi.y), dz = sub_rn(cz, pi.z);
+            return fma_rn(dz, dz, fma_rn(dy, dy, mul_rn(dx, dx)));
+        };
         // the full evaluation of the in-range pair (query lane li, slot sj): P (or its
         // rate on individual steps, scaled to dt_max), decision, record
         auto evaluate = [&](int li, uint32_t sj, uint32_t idi, uint32_t idj) -> float {
@@ -764,18 +791,25 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
             const float up = p.bins ? __int_as_float((127 + min(p.bins[ui], p.bins[uj])) << 23) : 1.f;   // 2^min(b_i, b_j)
             const float down = 1.f / up;                      // exact: bins are below 16
             const R prefp = fc.pref * down;
-            // P needs ~1e-6 relative accuracy only (the event decision below is
-            // exact for the P computed here): reciprocal square roots and
+            // mixed form: P needs ~1e-6 relative accuracy only (the event decision
+            // below is exact for the P computed here): reciprocal square roots and
             // approximate divisions are enough.
-            const float v = v2 > 0.f ? v2 * rsqrtf(v2) : 0.f;
-            float sig = 1.f;
-            if (fc.vdep) {
-                const float qq = v * fc.inv_w, tt = 1.f + qq * qq;
-                sig = __fdividef(1.f, tt * tt);
+            R v, sig = R(1), inv, u;
+            if constexpr (kF32) {
+                v = v2 > 0.f ? v2 * rsqrtf(v2) : 0.f;
+                if (fc.vdep) {
+                    const float qq = v * fc.inv_w, tt = 1.f + qq * qq;
+                    sig = __fdividef(1.f, tt * tt);
+                }
+                inv = __fdividef(1.f, fmaxf(hi, hj));
+                u = (R)((float)x.x[0] * 0x1p-32f);
+            } else {
+                v = sqrt(v2);
+                if (fc.vdep) { const R qq = v * fc.inv_w, tt = R(1) + qq * qq; sig = R(1) / (tt * tt); }
+                inv = R(1) / (hi > hj ? hi : hj);
+                u = (R)ldexp((double)x.x[0], -32);
             }
             const R pre = prefp * sig * v;
-            const R inv = __fdividef(1.f, fmaxf(hi, hj));
-            const R u = (R)((float)x.x[0] * 0x1p-32f);
             bool need = true;
             if constexpr (MODE == kModeDraw) {
                 const R P_up = pre * (R(kLamFUp) * inv * inv * inv);
@@ -785,14 +819,14 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
             bool fire = false;
             if (need) {
                 if constexpr (MODE == kModeDraw) atomicAdd(&wst[4], 1ull);   // else every pair
-                // canonical distance: the candidate shifted into the query leaf's frame
-                const float4 cj = p.cell[sj / kLeaf];
-                const R dx = sub_rn(__fadd_rn(pj.x, __fsub_rn(cj.x, cA.x)), pi.x);
-                const R dy = sub_rn(__fadd_rn(pj.y, __fsub_rn(cj.y, cA.y)), pi.y);
-                const R dz = sub_rn(__fadd_rn(pj.z, __fsub_rn(cj.z, cA.z)), pi.z);
-                const R d2 = fma_rn(dz, dz, fma_rn(dy, dy, mul_rn(dx, dx)));
-                const float d = d2 > 0.f ? d2 * rsqrtf(d2) : 0.f;
-                const R f = kEvery ? lambda_f_rows(p.lam4, d, hi, hj, inv) : lambda_f_fast(T, d, hi, hj, inv);
+                const R d2 = pair_d2(pi, pj, sj);
+                R f;
+                if constexpr (kF32) {
+                    const float d = d2 > 0.f ? d2 * rsqrtf(d2) : 0.f;
+                    f = kEvery ? lambda_f_rows(p.lam4, d, hi, hj, inv) : lambda_f_fast(T, d, hi, hj, inv);
+                } else {
+                    f = lambda_f<R>(T, sqrt_rn(d2), hi, hj);
+                }
                 P = pre * (f * inv * inv * inv);
                 if (drag) {
                     // the record keeps G = m_j Lambda dt; D = P / 3 at the step start.
@@ -800,18 +834,19 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
                     // Lambda must be accurate relative to itself where it falls to
                     // zero, which neither the table nor an FP32 quadrature (its
                     // integrand cancels there) is: FP64 quadrature beyond half the
-                    // support, the table inside, where Lambda > Lambda(0)/4 bounds
-                    // its relative error
+                    // support (everywhere in the FP64 form), the table inside, where
+                    // Lambda > Lambda(0)/4 bounds its relative error
                     R lam = f * inv * inv * inv;
                     const R dq = sqrt_rn(d2);
-                    if (dq >= R(0.5) * (hi + hj))
+                    if (!kF32 || dq >= R(0.5) * (hi + hj))
                         lam = (R)lambda_quad<double>((double)dq, (double)hi, (double)hj, p.glx, p.glw);
                     fire = true;
                     P = pre * lam;
                     gfac = (R)p.mass[h] * lam * (fc.dt * down);
                     if (P > R(3)) atomicAdd(&wst[1], 1ull);
                 } else {
-                    fire = P >= R(1) || x.x[0] < (uint32_t)ceilf((float)P * 0x1p32f);
+                    if constexpr (kF32) fire = P >= R(1) || x.x[0] < (uint32_t)ceilf((float)P * 0x1p32f);
+                    else fire = u < P;
                     if (P > R(1)) atomicAdd(&wst[1], 1ull);
                     if (fabs(P - u) < R(1e-6)) atomicAdd(&wst[2], 1ull);
                 }
@@ -836,7 +871,7 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
                     if (drag) p.evg[slot] = (double)gfac;
                 }
             }
-            return P * up;
+            return (float)(P * up);
         };
 
         // Consecutive particles of the Morton curve can lie far apart (on the sparse
@@ -958,9 +993,13 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
 #pragma unroll
                 for (int u = 0; u < 2; ++u) {
                     const uint32_t s = (uint32_t)(leaf0 + Bl[u]) * kLeaf + lane;
-                    c[u] = P4[s];
+                    c[u] = S4[s];
                     cB[u] = p.cell[leaf0 + Bl[u]];
                     id[u] = p.ID[s];
+                    if constexpr (!kF32) {
+                        if (c[u].w < 0.f) id[u] |= kUnsure;
+                        c[u].w = fabsf(c[u].w);
+                    }
                     open[u] = (uint32_t)Bl[u] * kLeaf + lane < nh && li + u < nl;
                     if (p.bins) open[u] = open[u] && step_opens(p.bins[index_of(s)], p.n_bins, p.substep);
                 }
@@ -1015,7 +1054,8 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
                 int full = qn;                           // pairs to draw now: all of them at the very end
                 if (navail >= kPBatch) {
                     // the ring's first kPBatch candidates against all queries
-                    uint32_t okm = 0u;
+                    uint32_t okm = 0u, surem = 0u;          // in range; FP64 form: for certain
+                    const unsigned long long sure2 = pack2(sure, sure);
 #pragma unroll
                     for (int t = 0; t < kPBatch; t += 4) {
                         const float* at = ring + (cnum & (kPRing - 1)) + t;
@@ -1032,6 +1072,11 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
                             unpack2(hs2, ha, hb);
                             if (da < ha) okm |= 1u << (t + 2 * u);
                             if (db < hb) okm |= 2u << (t + 2 * u);
+                            if constexpr (!kF32) {
+                                unpack2(mul2(hs2, sure2), ha, hb);
+                                if (da < ha) surem |= 1u << (t + 2 * u);
+                                if (db < hb) surem |= 2u << (t + 2 * u);
+                            }
                         }
                     }
                     if (nself > 0) {                     // inside the leaf each pair once: candidates after the query
@@ -1052,7 +1097,8 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
                     const uint32_t tag = (uint32_t)lane << 8;
 #pragma unroll
                     for (int t = 0; t < kPBatch; ++t)
-                        if ((okm >> t) & 1u) *qp++ = (uint16_t)(tag | ((cnum + t) & (kPCand - 1)));
+                        if ((okm >> t) & 1u)
+                            *qp++ = (uint16_t)(tag | ((cnum + t) & (kPCand - 1)) | (kF32 || ((surem >> t) & 1u) ? 0u : 0x8000u));
                     if (qn == 0) oldest = cnum;
                     qn += total;
                     n_pairs += (uint32_t)total;
@@ -1072,10 +1118,25 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
                     for (int k = 0; k < PR; ++k) {
                         const int at = f0 + 32 * k + lane;
                         ent[k] = queue[at < full ? at : f0];
-                        idi[k] = qid[ent[k] >> 8];
+                        idi[k] = qid[(ent[k] >> 8) & 31u];
                         idj[k] = cid[ent[k] & (kPCand - 1)];
+                        bool valid = at < full;
+                        if constexpr (!kF32) {               // settled in FP64 where FP32 is not sure
+                            const bool ask = valid && ((ent[k] & 0x8000u) || (idj[k] & kUnsure));
+                            idj[k] &= ~kUnsure;
+                            if (__any_sync(FULL, ask)) {
+                                if (ask) {
+                                    const uint32_t sj = cslot[ent[k] & (kPCand - 1)];
+                                    const V pi = P4[(uint32_t)leaf * kLeaf + ((ent[k] >> 8) & 31u)], pj = P4[sj];
+                                    const R hs = add_rn(pi.w, pj.w);
+                                    valid = pair_d2(pi, pj, sj) < mul_rn(hs, hs);
+                                }
+                                n_pairs -= (uint32_t)__popc(__ballot_sync(FULL, ask && !valid));
+                            }
+                            ent[k] &= 0x7fffu;
+                        }
                         const Philox4 x = philox4x32_10_rk(p.step_lo, min(idi[k], idj[k]), max(idi[k], idj[k]), (uint32_t)h, p.rk);
-                        maybe |= (at < full && x.x[0] <= thr ? 1u : 0u) << k;
+                        maybe |= (valid && x.x[0] <= thr ? 1u : 0u) << k;
                     }
                     if constexpr (MODE == kModeDrawExact) {
                         static_assert(MODE != kModeDrawExact || PR == 1, "one group at a time");
@@ -1181,7 +1242,7 @@ void fill_params(sidm_ctx* c, PairParams& p, uint64_t seed, uint64_t step, const
     p.H = L.H; p.L = L.L;
     p.leaf_halo = c->d_leaf_halo; p.leaf_off = c->d_leaf_off; p.halo_off = c->d_halo_off;
     p.lvl_off = c->d_lvl_off; p.top = c->d_top; p.frame = c->d_frame; p.cell = c->d_cell;
-    p.nlo = c->d_nlo; p.nhi = c->d_nhi; p.P4 = c->d_P4; p.V4 = c->d_V4; p.ID = c->d_ID; p.lam = c->d_lam; p.lam4 = c->d_lam4;
+    p.nlo = c->d_nlo; p.nhi = c->d_nhi; p.P4 = c->d_P4; p.S4 = c->cfg.precision == SIDM_FP64 ? (const void*)c->d_S4 : c->d_P4; p.V4 = c->d_V4; p.ID = c->d_ID; p.lam = c->d_lam; p.lam4 = c->d_lam4;
     p.vel = vel; p.N = L.N; p.parts = 1;
     p.xs = xs; p.dt = dt; p.mass = mass;
     p.seed_lo = (uint32_t)seed; p.seed_hi = (uint32_t)(seed >> 32); p.step_lo = (uint32_t)step;
@@ -1227,7 +1288,7 @@ int launch_t(sidm_ctx* c, uint64_t seed, uint64_t step, const sidm_xs* xs, const
     return SIDM_OK;
 }
 
-// mixed-form draws.  With few query leaves each is shared by several warps (a
+// With few query leaves each is shared by several warps (a
 // power of two, at most kPartsMax), so that every resident warp has about
 // kPartsPerWarp items: the last wave stays short, at the price of the walk that
 // the parts repeat.
@@ -1268,36 +1329,30 @@ int launch_draws(sidm_ctx* c, uint64_t seed, uint64_t step, const sidm_xs* xs, c
 
 }  // namespace
 
+template <class R>
+static int launch_form(sidm_ctx* c, uint64_t seed, uint64_t step, const sidm_xs* xs, const double* dt, const double* mass,
+                       const void* vel, sidm_step_stats* st, cudaStream_t s)
+{
+    const bool exact = (c->cfg.flags & SIDM_FLAG_SUM_P) != 0;
+    if (c->cfg.flags & SIDM_FLAG_DRAG)                  // forward-dominated halos allowed
+        return exact ? launch_draws<R, kModeDrawExact, 1, true>(c, seed, step, xs, dt, mass, vel, st, s)
+                     : launch_draws<R, kModeDraw, 1, true>(c, seed, step, xs, dt, mass, vel, st, s);
+    if (exact) return launch_draws<R, kModeDrawExact, 1, false>(c, seed, step, xs, dt, mass, vel, st, s);
+    // the hot path: groups of 32 pairs drawn together as configured (a launch knob)
+    switch (c->cfg.pair_per_round > 0 ? c->cfg.pair_per_round : kPerRoundDefault) {
+    case 1: return launch_draws<R, kModeDraw, 1, false>(c, seed, step, xs, dt, mass, vel, st, s);
+    case 2: return launch_draws<R, kModeDraw, 2, false>(c, seed, step, xs, dt, mass, vel, st, s);
+    case 3: return launch_draws<R, kModeDraw, 3, false>(c, seed, step, xs, dt, mass, vel, st, s);
+    default: return launch_draws<R, kModeDraw, 4, false>(c, seed, step, xs, dt, mass, vel, st, s);
+    }
+}
+
 int launch_pairs(sidm_ctx* c, uint64_t seed, uint64_t step, const sidm_xs* xs, const double* dt, const double* mass,
                  const void* vel, sidm_step_stats* st, cudaStream_t s)
 {
     if (c->lay.L == 0) return SIDM_OK;
-    const bool tma = c->cfg.use_tma != 0;
-    const bool exact = (c->cfg.flags & SIDM_FLAG_SUM_P) != 0;
-    if (c->cfg.flags & SIDM_FLAG_DRAG) {                // forward-dominated halos allowed (plain loads)
-        if (c->cfg.precision == SIDM_FP64)
-            return exact ? launch_t<double, false, kModeDrawExact, kPerRoundMax, true>(c, seed, step, xs, dt, mass, vel, st, s)
-                         : launch_t<double, false, kModeDraw, kPerRoundMax, true>(c, seed, step, xs, dt, mass, vel, st, s);
-        return exact ? launch_draws<float, kModeDrawExact, 1, true>(c, seed, step, xs, dt, mass, vel, st, s)
-                     : launch_draws<float, kModeDraw, 1, true>(c, seed, step, xs, dt, mass, vel, st, s);
-    }
-#define SIDM_PAIRS_DISPATCH(R)                                                                                   \
-    if (exact) return tma ? launch_t<R, true, kModeDrawExact>(c, seed, step, xs, dt, mass, vel, st, s)                \
-                          : launch_t<R, false, kModeDrawExact>(c, seed, step, xs, dt, mass, vel, st, s);              \
-    if (tma) return launch_t<R, true, kModeDraw>(c, seed, step, xs, dt, mass, vel, st, s);
-    if (c->cfg.precision == SIDM_FP64) {
-        SIDM_PAIRS_DISPATCH(double)
-        return launch_t<double, false, kModeDraw>(c, seed, step, xs, dt, mass, vel, st, s);
-    }
-    if (exact) return launch_draws<float, kModeDrawExact, 1, false>(c, seed, step, xs, dt, mass, vel, st, s);
-#undef SIDM_PAIRS_DISPATCH
-    // the hot path: pairs queued per lane and round as configured (a launch knob)
-    switch (c->cfg.pair_per_round > 0 ? c->cfg.pair_per_round : kPerRoundDefault) {
-    case 1: return launch_draws<float, kModeDraw, 1, false>(c, seed, step, xs, dt, mass, vel, st, s);
-    case 2: return launch_draws<float, kModeDraw, 2, false>(c, seed, step, xs, dt, mass, vel, st, s);
-    case 3: return launch_draws<float, kModeDraw, 3, false>(c, seed, step, xs, dt, mass, vel, st, s);
-    default: return launch_draws<float, kModeDraw, 4, false>(c, seed, step, xs, dt, mass, vel, st, s);
-    }
+    return c->cfg.precision == SIDM_FP64 ? launch_form<double>(c, seed, step, xs, dt, mass, vel, st, s)
+                                         : launch_form<float>(c, seed, step, xs, dt, mass, vel, st, s);
 }
 
 int launch_pairs_diag(sidm_ctx* c, const sidm_xs* xs, const double* mass, cudaStream_t s)

@@ -46,7 +46,7 @@ def _positions(kind, n):
                                       ("far", 3000, 32)])
 def test_warm_equals_cold_and_oracle(kind, n, k, precision):
     from paper_2506_06269_gb300 import sidm
-    x = _positions(kind, n)
+    x = np.ascontiguousarray(_positions(kind, n))
     ids = np.random.default_rng(1).permutation(n).astype(np.int64)
     out = []
     for warm in (True, False):
