@@ -63,7 +63,8 @@ extern "C" {
 #define SIDM_FLAG_TIMING  0x2  /* time hot kernels with CUDA events (sidm_kernel_times) */
 #define SIDM_FLAG_LOCAL_DIAG 0x4 /* keep scratch for sidm_local_diagnostics (40 B/particle) */
 #define SIDM_FLAG_DRAG    0x8  /* keep scratch for forward-dominated halos (sidm_xs.angular = 1):
-                                  per-particle interaction lists, 64 B per event_cap */
+                                  per-particle interaction lists, 64 B per event_cap, and
+                                  40 (FP64: 72) more up to 1024 particles per SM */
 
 typedef struct sidm_ctx sidm_ctx;
 

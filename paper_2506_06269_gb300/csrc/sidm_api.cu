@@ -576,33 +576,32 @@ __device__ __forceinline__ void fx_add(DevCounters* cnt, double v)
     atomicAdd(&cnt->de_hi, hi);
 }
 
-// Isotropic scatter of event E (Sect. 2, reading C6) on the current velocities
-// (read and written through L2); returns the change of the pair's kinetic
-// energy from the stored values, in FP64.  Equal masses within a halo.
+// Isotropic Philox direction of words 1 and 2 (reading C6).
 template <class R>
-__device__ __forceinline__ double apply_isotropic(const sidm_event& E, R* vel, int64_t N, const double* __restrict__ mass)
+__device__ __forceinline__ void philox_direction(uint32_t x1, uint32_t x2, R n[3])
 {
-    R* vx = vel; R* vy = vel + N; R* vz = vel + 2 * N;
-    const int h = (int)(E.key >> 54);
-    const double m = mass[h];
-    const R vi[3] = {__ldcg(vx + E.i), __ldcg(vy + E.i), __ldcg(vz + E.i)};
-    const R vj[3] = {__ldcg(vx + E.j), __ldcg(vy + E.j), __ldcg(vz + E.j)};
     R ct, st_, sp, cp;
     if (sizeof(R) == 4) {
-        ct = (R)fmaf((float)E.x1, 0x1p-31f, -1.0f);
+        ct = (R)fmaf((float)x1, 0x1p-31f, -1.0f);
         st_ = (R)sqrtf(fmaxf(0.f, 1.f - (float)ct * (float)ct));
         float s_, c_;
-        sincospif((float)E.x2 * 0x1p-31f, &s_, &c_);
+        sincospif((float)x2 * 0x1p-31f, &s_, &c_);
         sp = (R)s_; cp = (R)c_;
     } else {
-        ct = (R)(2.0 * ldexp((double)E.x1, -32) - 1.0);
+        ct = (R)(2.0 * ldexp((double)x1, -32) - 1.0);
         st_ = (R)sqrt(fmax(0.0, 1.0 - (double)ct * (double)ct));
         double s_, c_;
-        sincospi(ldexp((double)E.x2, -31), &s_, &c_);
+        sincospi(ldexp((double)x2, -31), &s_, &c_);
         sp = (R)s_; cp = (R)c_;
     }
-    const R nh[3] = {st_ * cp, st_ * sp, ct};
-    // equal masses within a halo: v_cm = (v_i + v_j)/2, weights 1/2
+    n[0] = st_ * cp; n[1] = st_ * sp; n[2] = ct;
+}
+
+// Isotropic scatter (Sect. 2, reading C6) of velocities vi (the smaller id), vj
+// into the direction w; equal masses within a halo: v_cm = (v_i + v_j)/2.
+template <class R>
+__device__ __forceinline__ void scatter_isotropic(const R vi[3], const R vj[3], const R w[3], R ni[3], R nj[3])
+{
     R dv2 = R(0), vc[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -611,62 +610,29 @@ __device__ __forceinline__ double apply_isotropic(const sidm_event& E, R* vel, i
         dv2 += d * d;
     }
     const R hw = R(0.5) * sqrt(dv2);
-    R ni[3], nj[3];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) { ni[a] = vc[a] + hw * nh[a]; nj[a] = vc[a] - hw * nh[a]; }
-    __stcg(vx + E.i, ni[0]); __stcg(vy + E.i, ni[1]); __stcg(vz + E.i, ni[2]);
-    __stcg(vx + E.j, nj[0]); __stcg(vy + E.j, nj[1]); __stcg(vz + E.j, nj[2]);
-    double e0 = 0.0, e1 = 0.0;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        e0 = __dadd_rn(e0, __dadd_rn(__dmul_rn((double)vi[a], (double)vi[a]), __dmul_rn((double)vj[a], (double)vj[a])));
-        e1 = __dadd_rn(e1, __dadd_rn(__dmul_rn((double)ni[a], (double)ni[a]), __dmul_rn((double)nj[a], (double)nj[a])));
-    }
-    return __dmul_rn(0.5 * m, __dsub_rn(e1, e0));
+    for (int a = 0; a < 3; ++a) { ni[a] = vc[a] + hw * w[a]; nj[a] = vc[a] - hw * w[a]; }
 }
 
-// Forward-dominated interaction of record E (Sect. 3.8 with App. A, reading
-// C20): the relative velocity u = v_i - v_j turns by alpha, cos(alpha) = 1 - D,
+// Forward-dominated interaction (Sect. 3.8 with App. A, reading C20): the
+// relative velocity u = v_i - v_j turns by alpha, cos(alpha) = 1 - D,
 // sin(alpha) = sqrt(D (2 - D)), D = (sigma_V/m)/3 |u| G, G = m_j Lambda dt of the
-// step start, towards the projection onto u's normal plane of the isotropic
-// Philox direction of words 1 and 2 (uniform in azimuth about u); |u| and v_cm
-// are kept.  D = 0 changes nothing.  Returns the pair's kinetic-energy change
-// from the stored values (FP64).
+// step start, towards the projection of the isotropic direction w onto u's normal
+// plane (uniform in azimuth about u); |u| and v_cm are kept.  D = 0 changes
+// nothing (returns false).
 template <class R>
-__device__ __forceinline__ double apply_drag(const sidm_event& E, double G, const sidm_xs& xs, R* vel, int64_t N,
-                                             const double* __restrict__ mass)
+__device__ __forceinline__ bool scatter_drag(const R vi[3], const R vj[3], const R w[3], R G, const sidm_xs& xs, R ni[3], R nj[3])
 {
-    R* vx = vel; R* vy = vel + N; R* vz = vel + 2 * N;
-    const double m = mass[(int)(E.key >> 54)];
-    const R vi[3] = {__ldcg(vx + E.i), __ldcg(vy + E.i), __ldcg(vz + E.i)};
-    const R vj[3] = {__ldcg(vx + E.j), __ldcg(vy + E.j), __ldcg(vz + E.j)};
     R u[3], vc[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) { u[a] = vi[a] - vj[a]; vc[a] = R(0.5) * (vi[a] + vj[a]); }
     const R un = sqrt(u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
     R sig = (R)xs.s0;
     if (xs.kind == 1) { const R q = un / (R)xs.w; const R t = R(1) + q * q; sig = (R)xs.s0 / (t * t); }
-    const R D = sig / R(3) * un * (R)G;
-    if (!(D > R(0))) return 0.0;
+    const R D = sig / R(3) * un * G;
+    if (!(D > R(0))) return false;
     R ca, sa;
     if (D < R(2)) { ca = R(1) - D; sa = sqrt(D * (R(2) - D)); } else { ca = R(-1); sa = R(0); }
-    // the turn's direction: the isotropic Philox direction w (words 1, 2, as an
-    // isotropic scatter draws it) projected onto the plane normal to u
-    R ct, st_, sp, cp;
-    if (sizeof(R) == 4) {
-        ct = (R)fmaf((float)E.x1, 0x1p-31f, -1.0f);
-        st_ = (R)sqrtf(fmaxf(0.f, 1.f - (float)ct * (float)ct));
-        float s_, c_;
-        sincospif((float)E.x2 * 0x1p-31f, &s_, &c_);
-        sp = (R)s_; cp = (R)c_;
-    } else {
-        ct = (R)(2.0 * ldexp((double)E.x1, -32) - 1.0);
-        st_ = (R)sqrt(fmax(0.0, 1.0 - (double)ct * (double)ct));
-        double s_, c_;
-        sincospi(ldexp((double)E.x2, -31), &s_, &c_);
-        sp = (R)s_; cp = (R)c_;
-    }
-    const R w[3] = {st_ * cp, st_ * sp, ct};
     const R nh[3] = {u[0] / un, u[1] / un, u[2] / un};
     const R wn = w[0] * nh[0] + w[1] * nh[1] + w[2] * nh[2];
     R ep[3], el = R(0);
@@ -674,13 +640,30 @@ __device__ __forceinline__ double apply_drag(const sidm_event& E, double G, cons
     for (int a = 0; a < 3; ++a) { ep[a] = w[a] - wn * nh[a]; el += ep[a] * ep[a]; }
     el = sqrt(el);
     const R sc = el > R(0) ? un * sa / el : R(0);
-    R ni[3], nj[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         const R up = ca * u[a] + sc * ep[a];
         ni[a] = vc[a] + R(0.5) * up;
         nj[a] = vc[a] - R(0.5) * up;
     }
+    return true;
+}
+
+// Event or record E on the current velocities (read and written through L2);
+// drag: the halo's cross-section if it is forward-dominated, else NULL.  Returns
+// the change of the pair's kinetic energy from the stored values, in FP64.
+template <class R>
+__device__ __forceinline__ double apply_event(const sidm_event& E, double G, const sidm_xs* drag, R* vel, int64_t N,
+                                              const double* __restrict__ mass)
+{
+    R* vx = vel; R* vy = vel + N; R* vz = vel + 2 * N;
+    const double m = mass[(int)(E.key >> 54)];
+    const R vi[3] = {__ldcg(vx + E.i), __ldcg(vy + E.i), __ldcg(vz + E.i)};
+    const R vj[3] = {__ldcg(vx + E.j), __ldcg(vy + E.j), __ldcg(vz + E.j)};
+    R w[3], ni[3], nj[3];
+    philox_direction<R>(E.x1, E.x2, w);
+    if (!drag) scatter_isotropic<R>(vi, vj, w, ni, nj);
+    else if (!scatter_drag<R>(vi, vj, w, (R)G, *drag, ni, nj)) return 0.0;
     __stcg(vx + E.i, ni[0]); __stcg(vy + E.i, ni[1]); __stcg(vz + E.i, ni[2]);
     __stcg(vx + E.j, nj[0]); __stcg(vy + E.j, nj[1]); __stcg(vz + E.j, nj[2]);
     double e0 = 0.0, e1 = 0.0;
@@ -734,7 +717,7 @@ __global__ void __launch_bounds__(1024) k_resolve(const sidm_event* __restrict__
                 if (__ldcg(done + e)) continue;
                 const sidm_event E = ev[e];
                 if (__ldcg(claim + E.i) != E.key || __ldcg(claim + E.j) != E.key) continue;
-                fx_add(cnt, apply_isotropic<R>(E, vel, N, mass));
+                fx_add(cnt, apply_event<R>(E, 0.0, nullptr, vel, N, mass));
                 done[e] = 1;
             }
             __syncthreads();
@@ -912,7 +895,7 @@ __global__ void __launch_bounds__(256) k_resolve_lists(ListResolve q)
             const uint32_t o = E.i == p ? E.j : E.i;
             if (p > o || q.lval[q.start[o] + __ldcg(q.ptr + o)] != e) continue;
             const sidm_xs xs = q.xs[(int)(E.key >> 54)];
-            acc.add(xs.angular ? apply_drag<R>(E, q.evg[e], xs, vel, q.N, q.mass) : apply_isotropic<R>(E, vel, q.N, q.mass));
+            acc.add(apply_event<R>(E, q.evg[e], xs.angular ? &xs : nullptr, vel, q.N, q.mass));
             __stcg(q.done + e, (uint8_t)1);
         }
         if (!grid_barrier(q.cnt)) { status |= SIDM_DEV_WAIT_TIMEOUT; break; }
@@ -943,6 +926,217 @@ __global__ void __launch_bounds__(256) k_resolve_lists(ListResolve q)
     }
     if (tid == 0) { q.lcnt[3] = rounds; if (status) atomicOr(&q.lcnt[4], status); }
     else if (status && threadIdx.x == 0) atomicOr(&q.lcnt[4], status);
+}
+
+// ---- the same rounds with a thread per particle -----------------------------
+// Every thread holds its particle's velocity and next interaction in registers;
+// a round is one look at the partner's (velocity, next partner) word, the
+// arithmetic of the pair by both of its threads if they name each other, and one
+// barrier.  The published words alternate between two buffers, so that a round
+// reads what the round before wrote.  An interaction's direction, strength and
+// partner are laid out per particle beforehand (k_list_entries), so a thread
+// reads its list front to back, one entry ahead, and leaves its velocity after
+// an interaction in the entry's place; the pairs' FP64 energy changes are formed
+// from those afterwards (k_list_energy), off the chain of rounds.
+//
+// Latency-bound: the number of rounds is the depth of the conflict graph (1448
+// for the in-range pairs of 16384 particles at N_ngb = 32), 2.6 us each (3.8 ms;
+// 26 us, 38.3 ms, with heads looked up in the lists, lists of active particles,
+// FP64 energies in the round and two grid barriers over 608 CTAs).  Up to 16 CTAs
+// of 1024 threads run as one cluster with its hardware barrier, more behind the
+// grid barrier; beyond one CTA per SM the lists of active particles serve.
+template <class R> struct ListEntry;
+template <> struct ListEntry<float> { float4 wg; };                 // direction, G
+template <> struct ListEntry<double> { double4_16a wg; };
+
+struct RoundsResolve {
+    const uint32_t* start;
+    const uint32_t* end;      // 0: no records
+    void* ent;                // ListEntry<R> [entries], in list order; on return the velocity after each
+    const uint32_t* part;     // partner | (this particle has the smaller id) << 31
+    const sidm_xs* xs;
+    const int64_t* halo_off;
+    int H;
+    void* vel;
+    void* pub;                // [2][N] (vx, vy, vz, next partner), then [N] the first velocities
+    int64_t N;
+    uint32_t* lcnt;           // [2] multi-hit; [3] rounds; [4] status; [5..7] CTAs with work left
+    DevCounters* cnt;         // grid barrier
+    int64_t max_rounds;
+};
+constexpr int kRoundThreads = 1024;
+constexpr int kRoundCheck = 16;       // rounds between two looks at whether anything is left
+constexpr int kRoundCluster = 16;     // CTAs of one cluster (above 8: opt-in)
+constexpr uint32_t kNoPartner = 0x7fffffffu;
+
+template <class R>
+__global__ void k_list_entries(const unsigned long long* __restrict__ key, const uint32_t* __restrict__ val, int64_t m,
+                               const sidm_event* __restrict__ ev, const double* __restrict__ evg,
+                               ListEntry<R>* __restrict__ ent, uint32_t* __restrict__ part, uint32_t* __restrict__ pos,
+                               uint32_t* __restrict__ start, uint32_t* __restrict__ end, uint32_t* __restrict__ lcnt)
+{
+    // also the bounds of each particle's list, and the number of particles in two or
+    // more records
+    uint32_t multi = 0u;
+    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < m; s += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t p = (uint32_t)(key[s] >> 27), e = val[s];
+        const sidm_event E = ev[e];
+        R w[3];
+        philox_direction<R>(E.x1, E.x2, w);
+        ListEntry<R> t;
+        t.wg.x = w[0]; t.wg.y = w[1]; t.wg.z = w[2]; t.wg.w = (R)evg[e];
+        ent[s] = t;
+        part[s] = E.i == p ? E.j | 0x80000000u : E.i;
+        pos[2 * (int64_t)e + (E.i == p ? 0 : 1)] = (uint32_t)s;
+        const bool head = s == 0 || (uint32_t)(key[s - 1] >> 27) != p, tail = s + 1 == m || (uint32_t)(key[s + 1] >> 27) != p;
+        if (head) start[p] = (uint32_t)s;
+        if (tail) end[p] = (uint32_t)(s + 1);
+        multi += head && !tail ? 1u : 0u;
+    }
+    multi = __reduce_add_sync(0xffffffffu, multi);
+    if ((threadIdx.x & 31) == 0 && multi) atomicAdd(&lcnt[2], multi);
+}
+
+template <class R, bool CLUSTER>
+__global__ void __launch_bounds__(kRoundThreads, 1) k_resolve_rounds(RoundsResolve q)
+{
+    using V = typename Vec4<R>::T;
+    const int64_t p = blockIdx.x * (int64_t)kRoundThreads + threadIdx.x;
+    const bool mine = p < q.N;
+    ListEntry<R>* ent = (ListEntry<R>*)q.ent;
+    R* vel = (R*)q.vel;
+    V* pub = (V*)q.pub;
+    auto partner_of = [](const V& v) -> uint32_t {
+        if constexpr (sizeof(R) == 4) return __float_as_uint(v.w);
+        else return (uint32_t)__double_as_longlong(v.w);
+    };
+    auto load = [](const V* a) -> V {
+        if constexpr (sizeof(R) == 4) return __ldcg(a);
+        else {
+            const double2 lo = __ldcg((const double2*)a), hi = __ldcg((const double2*)a + 1);
+            V v; v.x = lo.x; v.y = lo.y; v.z = hi.x; v.w = hi.y;
+            return v;
+        }
+    };
+    auto store = [](V* a, const R v[3], uint32_t o) {
+        if constexpr (sizeof(R) == 4) __stcg(a, make_float4(v[0], v[1], v[2], __uint_as_float(o)));
+        else {
+            __stcg((double2*)a, make_double2(v[0], v[1]));
+            __stcg((double2*)a + 1, make_double2(v[2], __longlong_as_double((long long)o)));
+        }
+    };
+    auto barrier = [&]() -> bool {
+        if constexpr (CLUSTER) {
+            asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+            asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+            return true;
+        } else {
+            return grid_barrier(q.cnt);
+        }
+    };
+    R v[3] = {R(0), R(0), R(0)};
+    uint32_t at = 0u, end = 0u, cur = kNoPartner, nxt = kNoPartner;   // this entry's partner, the next one's
+    ListEntry<R> e{}, en{};
+    sidm_xs xs{};
+    if (mine) {
+        for (int a = 0; a < 3; ++a) v[a] = vel[a * q.N + p];
+        xs = q.xs[halo_of(q.halo_off, q.H, p)];
+        end = q.end[p];
+        if (end) {
+            at = q.start[p];
+            cur = q.part[at]; e = ent[at];
+            if (at + 1 < end) { nxt = q.part[at + 1]; en = ent[at + 1]; }
+        }
+        store(pub + p, v, cur & 0x7fffffffu);
+        store(pub + 2 * q.N + p, v, 0u);
+    }
+    unsigned int last = 0u, status = 0u;
+    int slot = 0;
+    if (!barrier()) status |= SIDM_DEV_WAIT_TIMEOUT;
+    for (int64_t r = 0; status == 0u; ++r) {
+        const V* rd = pub + (r & 1 ? q.N : 0);
+        V* wr = pub + (r & 1 ? 0 : q.N);
+        if (at < end) {
+            const V o = load(rd + (cur & 0x7fffffffu));
+            if (partner_of(o) == (uint32_t)p) {
+                const R w[3] = {e.wg.x, e.wg.y, e.wg.z}, vo[3] = {o.x, o.y, o.z};
+                R ni[3], nj[3];
+                const bool first = cur >> 31;
+                const R vi[3] = {first ? v[0] : vo[0], first ? v[1] : vo[1], first ? v[2] : vo[2]};
+                const R vj[3] = {first ? vo[0] : v[0], first ? vo[1] : v[1], first ? vo[2] : v[2]};
+                bool changed = true;
+                if (xs.angular) changed = scatter_drag<R>(vi, vj, w, e.wg.w, xs, ni, nj);
+                else scatter_isotropic<R>(vi, vj, w, ni, nj);
+                if (changed)
+                    for (int a = 0; a < 3; ++a) v[a] = first ? ni[a] : nj[a];
+                store(&ent[at].wg, v, 0u);
+                ++at;
+                cur = nxt; e = en;
+                if (at >= end) cur = kNoPartner;
+                if (at + 1 < end) { nxt = q.part[at + 1]; en = ent[at + 1]; }
+                last = (unsigned int)(r + 1);
+            }
+        }
+        if (mine) store(wr + p, v, cur & 0x7fffffffu);
+        const bool look = r % kRoundCheck == kRoundCheck - 1;
+        if (look) {
+            const int left = __syncthreads_or(at < end);
+            if (left && threadIdx.x == 0) atomicAdd(&q.lcnt[5 + slot], 1u);
+        }
+        if (!barrier()) { status |= SIDM_DEV_WAIT_TIMEOUT; break; }
+        if (look) {
+            const unsigned int left = __ldcg(&q.lcnt[5 + slot]);
+            // the slot looked at before this one is free again: every CTA has read it
+            if (blockIdx.x == 0 && threadIdx.x == 0) q.lcnt[5 + (slot + 2) % 3] = 0u;
+            slot = (slot + 1) % 3;
+            if (left == 0u) break;
+            if (r >= q.max_rounds) { status |= SIDM_DEV_ROUNDS; break; }   // cannot happen: >= 1 record per round
+        }
+    }
+    if (mine)
+        for (int a = 0; a < 3; ++a) vel[a * q.N + p] = v[a];
+    last = __reduce_max_sync(0xffffffffu, last);
+    if ((threadIdx.x & 31) == 0) {
+        if (last) atomicMax(&q.lcnt[3], last);
+        if (status) atomicOr(&q.lcnt[4], status);
+    }
+}
+
+// Kinetic-energy change of every record from the stored velocities before and
+// after it (ent, and pub's first velocities), as apply_event forms it.
+template <class R>
+__global__ void k_list_energy(const sidm_event* __restrict__ ev, int64_t n, const uint32_t* __restrict__ pos,
+                              const uint32_t* __restrict__ start, const ListEntry<R>* __restrict__ ent,
+                              const typename Vec4<R>::T* __restrict__ first, const double* __restrict__ mass,
+                              DevCounters* cnt)
+{
+    Fx128 acc;
+    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x) {
+        const sidm_event E = ev[r];
+        const uint32_t si = pos[2 * r], sj = pos[2 * r + 1];
+        const typename Vec4<R>::T ni = ent[si].wg, nj = ent[sj].wg;
+        const typename Vec4<R>::T vi = si == start[E.i] ? first[E.i] : ent[si - 1].wg;
+        const typename Vec4<R>::T vj = sj == start[E.j] ? first[E.j] : ent[sj - 1].wg;
+        const double a[3] = {(double)vi.x, (double)vi.y, (double)vi.z}, b[3] = {(double)vj.x, (double)vj.y, (double)vj.z};
+        const double c[3] = {(double)ni.x, (double)ni.y, (double)ni.z}, d[3] = {(double)nj.x, (double)nj.y, (double)nj.z};
+        double e0 = 0.0, e1 = 0.0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            e0 = __dadd_rn(e0, __dadd_rn(__dmul_rn(a[k], a[k]), __dmul_rn(b[k], b[k])));
+            e1 = __dadd_rn(e1, __dadd_rn(__dmul_rn(c[k], c[k]), __dmul_rn(d[k], d[k])));
+        }
+        acc.add(__dmul_rn(0.5 * mass[(int)(E.key >> 54)], __dsub_rn(e1, e0)));
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long l = __shfl_xor_sync(0xffffffffu, acc.lo, o);
+        const unsigned long long h = __shfl_xor_sync(0xffffffffu, acc.hi, o);
+        acc.lo += l;
+        acc.hi += h + (acc.lo < l ? 1ull : 0ull);
+    }
+    if ((threadIdx.x & 31) == 0 && (acc.lo | acc.hi)) {
+        const unsigned long long old = atomicAdd(&cnt->de_lo, acc.lo);
+        atomicAdd(&cnt->de_hi, acc.hi + (old + acc.lo < old ? 1ull : 0ull));
+    }
 }
 
 // The lists' pointers back to zero (entries of the sorted lists).
@@ -1329,7 +1523,7 @@ static void free_all(sidm_ctx* c)
                     c->d_tmp_vel, c->d_tmp_id, c->d_claim, c->d_hits, c->d_done, c->d_ev, c->d_sump,
                     c->d_stats_own, c->d_cnt, c->d_epart, c->d_chunk_off, c->d_group_off, c->d_gpart, c->d_lam, c->d_lam4, c->d_hprev, c->d_dacc, c->d_halo_ord,
                     c->d_evg, c->d_lkey, c->d_lval, c->d_lstart, c->d_llen, c->d_lptr, c->d_lact,
-                    c->d_lcnt};
+                    c->d_lcnt, c->d_lent, c->d_lpart, c->d_lpub};
     for (void* p : ptrs) if (p) cudaFree(p);
     if (c->d_stage) cudaFreeHost(c->d_stage);
     for (cudaEvent_t e : c->t_ev) if (e) cudaEventDestroy(e);
@@ -1455,6 +1649,11 @@ extern "C" int sidm_create(sidm_ctx** out, const sidm_config* cfg)
         ALLOC(c->d_lptr, N);
         ALLOC(c->d_lact, 2 * N);
         ALLOC(c->d_lcnt, 8);
+        if (cdiv(N, kRoundThreads) <= c->sm_count) {                // rounds with a thread per particle
+            e = cudaMalloc(&c->d_lent, (size_t)m * 4 * rs); if (e != cudaSuccess) return fail("cudaMalloc lent", e);
+            ALLOC(c->d_lpart, m);
+            e = cudaMalloc(&c->d_lpub, (size_t)3 * N * 4 * rs); if (e != cudaSuccess) return fail("cudaMalloc lpub", e);
+        }
     }
 #undef ALLOC
     e = cudaMallocHost((void**)&c->d_stage, c->stage_bytes);
@@ -1751,6 +1950,37 @@ __global__ void k_max_sump(int64_t N, const float* __restrict__ sump, sidm_step_
     if ((threadIdx.x & 31) == 0) atomicMax((unsigned int*)&st->max_sum_p, __float_as_uint(m));
 }
 
+// Rounds with a thread per particle: one cluster if it fits, else a cooperative
+// launch behind the grid barrier.
+template <class R>
+static int launch_rounds(sidm_ctx* c, RoundsResolve q, int ctas, cudaStream_t s)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(kRoundThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)ctas; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (ctas <= kRoundCluster && c->round_clusters[ctas] < 0) {      // asked once per size
+        int n = 0;
+        cudaError_t e = cudaFuncSetAttribute(k_resolve_rounds<R, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, k_resolve_rounds<R, true>, &cfg);
+        if (e != cudaSuccess) { cudaGetLastError(); n = 0; }
+        c->round_clusters[ctas] = (int8_t)(n > 0 ? 1 : 0);
+    }
+    if (ctas <= kRoundCluster && c->round_clusters[ctas] > 0) {
+        SIDM_CUDA(c, cudaLaunchKernelEx(&cfg, k_resolve_rounds<R, true>, q));
+    } else {
+        void* args[] = {&q};
+        SIDM_CUDA(c, cudaLaunchCooperativeKernel((const void*)k_resolve_rounds<R, false>, dim3(ctas), dim3(kRoundThreads), args, 0, s));
+    }
+    c->launches++;
+    return SIDM_OK;
+}
+
 // a4 through per-particle interaction lists (contexts with SIDM_FLAG_DRAG; any
 // mix of isotropic and forward-dominated halos).  Synchronises the stream once,
 // to size the list sort from the number of records.
@@ -1781,8 +2011,28 @@ static int resolve_lists(sidm_ctx* c, const sidm_xs* xs, const double* mass, R* 
         while (ib < 31 && ((int64_t)1 << ib) < L.N) ++ib;
         const int passes = (int)cdiv(27 + ib, 8);
         if (int rc = radix_sort(c, ka, va, kb, vb, m, passes, s)) return rc;
-        SIDM_LAUNCH(c, k_list_runs<<<grid_for(c, m, 256), 256, 0, s>>>(ka, m, c->d_lstart, c->d_llen, c->d_lact, c->d_lcnt));
         SIDM_CUDA(c, cudaMemsetAsync(&c->d_cnt->work[2], 0, sizeof(unsigned int), s));
+        // a thread per particle while every CTA is resident at one per SM
+        const int64_t ctas = cdiv(L.N, kRoundThreads);
+        if (c->d_lent && ctas <= c->sm_count) {
+            SIDM_CUDA(c, cudaMemsetAsync(c->d_llen, 0, sizeof(uint32_t) * (size_t)L.N, s));
+            SIDM_LAUNCH(c, (k_list_entries<R><<<grid_for(c, m, 256), 256, 0, s>>>(
+                ka, va, m, c->d_ev, c->d_evg, (ListEntry<R>*)c->d_lent, c->d_lpart, vb, c->d_lstart, c->d_llen,
+                c->d_lcnt)));
+            RoundsResolve q;
+            q.start = c->d_lstart; q.end = c->d_llen; q.ent = c->d_lent; q.part = c->d_lpart; q.xs = xs;
+            q.halo_off = c->d_halo_off; q.H = L.H; q.vel = vel; q.pub = c->d_lpub; q.N = L.N; q.lcnt = c->d_lcnt;
+            q.cnt = c->d_cnt; q.max_rounds = (int64_t)n + kRoundCheck;
+            if (int rc = launch_rounds<R>(c, q, (int)ctas, s)) return rc;
+            using V = typename Vec4<R>::T;
+            SIDM_LAUNCH(c, (k_list_energy<R><<<grid_for(c, (int64_t)n, 256), 256, 0, s>>>(
+                c->d_ev, (int64_t)n, vb, c->d_lstart, (const ListEntry<R>*)c->d_lent, (const V*)c->d_lpub + 2 * L.N, mass, c->d_cnt)));
+            SIDM_LAUNCH(c, k_list_stats<<<1, 1, 0, s>>>((int64_t)n, c->d_lcnt, c->d_cnt, st));
+            if (use_sump) SIDM_LAUNCH(c, k_max_sump<<<1, 1024, 0, s>>>(L.N, c->d_sump, st));
+            timer_end(c, tr, s);
+            return SIDM_OK;
+        }
+        SIDM_LAUNCH(c, k_list_runs<<<grid_for(c, m, 256), 256, 0, s>>>(ka, m, c->d_lstart, c->d_llen, c->d_lact, c->d_lcnt));
         ListResolve q;
         q.ev = c->d_ev; q.evg = c->d_evg; q.xs = xs; q.mass = mass; q.lval = va; q.start = c->d_lstart;
         q.len = c->d_llen; q.ptr = c->d_lptr; q.act = c->d_lact; q.lcnt = c->d_lcnt; q.done = c->d_done;

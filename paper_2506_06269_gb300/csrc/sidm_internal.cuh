@@ -148,7 +148,11 @@ struct sidm_ctx {
     uint32_t* d_llen = nullptr;             // [N]
     uint32_t* d_lptr = nullptr;             // [N] (zero at rest)
     uint32_t* d_lact = nullptr;             // [2][N]
-    uint32_t* d_lcnt = nullptr;             // [8] active counts, multi-hit count, rounds, status
+    uint32_t* d_lcnt = nullptr;             // [8] active counts, multi-hit count, rounds, status, work left
+    void* d_lent = nullptr;                 // [2 event_cap] direction and G of each list entry (thread per particle)
+    uint32_t* d_lpart = nullptr;            // [2 event_cap] partner of each list entry
+    void* d_lpub = nullptr;                 // [2][N] velocity and next partner as published, [N] first velocities
+    int8_t round_clusters[17] = {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1};   // cluster sizes that run
     double gl8x[8] = {}, gl8w[8] = {};      // 8-point Gauss-Legendre rule (Lambda quadrature on the device)
     unsigned long long* d_halo_ord = nullptr;  // [H] per-halo minima (order-preserving bits)
 
