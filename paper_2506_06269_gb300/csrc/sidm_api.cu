@@ -393,7 +393,12 @@ __global__ void k_timestep(int64_t N, int H, const int64_t* __restrict__ halo_of
                            double* __restrict__ dt_out, int32_t* __restrict__ bin_out,
                            unsigned long long* __restrict__ halo_min)
 {
-    for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < N; u += (int64_t)gridDim.x * blockDim.x) {
+    // whole warps stay in the loop: the halo minimum is taken over the warp first
+    // (one atomic per warp inside a halo instead of one per particle)
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t u0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); u0 < N; u0 += step) {
+        const int64_t u = min(u0 + (threadIdx.x & 31), N - 1);
+        const bool own = u0 + (threadIdx.x & 31) < N;
         int lo = 0, hi = H - 1;                    // halo of particle u: last h with halo_off[h] <= u
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
@@ -404,9 +409,17 @@ __global__ void k_timestep(int64_t N, int H, const int64_t* __restrict__ halo_of
         di = fmin(fmax(di, dt_min), dt_max);
         int b = 0;
         while (b < n_bins - 1 && ldexp(dt_max, -b) > di) ++b;
-        if (dt_out) dt_out[u] = di;
-        if (bin_out) bin_out[u] = b;
-        if (halo_min) atomicMin(halo_min + lo, dbl_to_ord(di));
+        if (own && dt_out) dt_out[u] = di;
+        if (own && bin_out) bin_out[u] = b;
+        if (halo_min) {
+            unsigned long long v = dbl_to_ord(di);
+            if (__all_sync(0xffffffffu, lo == __shfl_sync(0xffffffffu, lo, 0))) {
+                for (int o = 16; o > 0; o >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, o));
+                if ((threadIdx.x & 31) == 0) atomicMin(halo_min + lo, v);
+            } else {
+                atomicMin(halo_min + lo, v);
+            }
+        }
     }
 }
 
@@ -683,7 +696,7 @@ template <class R>
 __global__ void __launch_bounds__(1024) k_resolve(const sidm_event* __restrict__ ev, int64_t cap, R* vel, int64_t N,
                                                   const double* __restrict__ mass, unsigned long long* claim,
                                                   uint32_t* hits, uint8_t* done, DevCounters* cnt,
-                                                  sidm_step_stats* st, int max_rounds, const float* sump, int use_sump)
+                                                  sidm_step_stats* st, int max_rounds)
 {
     __shared__ unsigned int s_rem;
     __shared__ unsigned long long s_multi;
@@ -749,12 +762,6 @@ __global__ void __launch_bounds__(1024) k_resolve(const sidm_event* __restrict__
         st->status = status;
         const unsigned long long hi = cnt->de_hi, lo = cnt->de_lo;
         st->d_energy = ldexp((double)(long long)hi, -16) + ldexp((double)lo, -80);
-    }
-    if (use_sump) {   // max_i sum_j P_ij
-        float m = 0.f;
-        for (int64_t s = threadIdx.x; s < N; s += blockDim.x) m = fmaxf(m, sump[s]);
-        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        if ((threadIdx.x & 31) == 0) atomicMax((unsigned int*)&st->max_sum_p, __float_as_uint(m));
     }
 }
 
@@ -1208,6 +1215,22 @@ __global__ void k_energy_final(int H, const int32_t* __restrict__ group_off, con
     const int h = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     if (h >= H) return;                                  // whole warps
     sidm_sum::halo_result(gpart, group_off[h], group_off[h + 1], mass[h], out + 4 * h, comp ? comp + 4 * h : nullptr);
+}
+
+// Both levels in one launch while no halo has more than one group (a small halo's
+// step is a chain of launches of a few us each): one warp per halo.
+__global__ void k_energy_small(int H, const int32_t* __restrict__ group_off, const int32_t* __restrict__ chunk_off,
+                               const double* __restrict__ mass, const double* __restrict__ part,
+                               double* __restrict__ out, double* __restrict__ comp)
+{
+    __shared__ double group[4][8];
+    double* g = group[threadIdx.x >> 5];
+    const int h = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    if (h >= H) return;                                  // whole warps
+    const int n = group_off[h + 1] - group_off[h];
+    if (n > 0) sidm_sum::group_sums(part, chunk_off[h], chunk_off[h + 1], g);
+    __syncwarp();
+    sidm_sum::halo_result(g, 0, n, mass[h], out + 4 * h, comp ? comp + 4 * h : nullptr);
 }
 
 // ------------------------------------------------------------------ harness
@@ -1945,7 +1968,7 @@ extern "C" int sidm_neighbours(sidm_ctx* c, const int32_t* n_ngb, int32_t k_stri
 __global__ void k_max_sump(int64_t N, const float* __restrict__ sump, sidm_step_stats* st)
 {
     float m = 0.f;
-    for (int64_t s = threadIdx.x; s < N; s += blockDim.x) m = fmaxf(m, sump[s]);
+    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < N; s += (int64_t)gridDim.x * blockDim.x) m = fmaxf(m, sump[s]);
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     if ((threadIdx.x & 31) == 0) atomicMax((unsigned int*)&st->max_sum_p, __float_as_uint(m));
 }
@@ -2028,7 +2051,7 @@ static int resolve_lists(sidm_ctx* c, const sidm_xs* xs, const double* mass, R* 
             SIDM_LAUNCH(c, (k_list_energy<R><<<grid_for(c, (int64_t)n, 256), 256, 0, s>>>(
                 c->d_ev, (int64_t)n, vb, c->d_lstart, (const ListEntry<R>*)c->d_lent, (const V*)c->d_lpub + 2 * L.N, mass, c->d_cnt)));
             SIDM_LAUNCH(c, k_list_stats<<<1, 1, 0, s>>>((int64_t)n, c->d_lcnt, c->d_cnt, st));
-            if (use_sump) SIDM_LAUNCH(c, k_max_sump<<<1, 1024, 0, s>>>(L.N, c->d_sump, st));
+            if (use_sump) SIDM_LAUNCH(c, k_max_sump<<<grid_for(c, L.N, 1024), 256, 0, s>>>(L.N, c->d_sump, st));
             timer_end(c, tr, s);
             return SIDM_OK;
         }
@@ -2049,7 +2072,7 @@ static int resolve_lists(sidm_ctx* c, const sidm_xs* xs, const double* mass, R* 
         SIDM_LAUNCH(c, k_list_reset<<<grid_for(c, m, 256), 256, 0, s>>>(ka, m, c->d_lptr));
     }
     SIDM_LAUNCH(c, k_list_stats<<<1, 1, 0, s>>>((int64_t)n, c->d_lcnt, c->d_cnt, st));
-    if (use_sump) SIDM_LAUNCH(c, k_max_sump<<<1, 1024, 0, s>>>(L.N, c->d_sump, st));
+    if (use_sump) SIDM_LAUNCH(c, k_max_sump<<<grid_for(c, L.N, 1024), 256, 0, s>>>(L.N, c->d_sump, st));
     timer_end(c, tr, s);
     return SIDM_OK;
 }
@@ -2083,10 +2106,11 @@ static int scatter_impl(sidm_ctx* c, uint64_t seed, uint64_t step, const sidm_xs
     const int tr = timer_begin(c, 3, s);
     if (fp64)
         SIDM_LAUNCH(c, k_resolve<double><<<1, 1024, 0, s>>>(c->d_ev, c->cfg.event_cap, (double*)vel, L.N, mass, c->d_claim,
-                                                          c->d_hits, c->d_done, c->d_cnt, st, c->cfg.max_rounds, c->d_sump, use_sump));
+                                                          c->d_hits, c->d_done, c->d_cnt, st, c->cfg.max_rounds));
     else
         SIDM_LAUNCH(c, k_resolve<float><<<1, 1024, 0, s>>>(c->d_ev, c->cfg.event_cap, (float*)vel, L.N, mass, c->d_claim,
-                                                         c->d_hits, c->d_done, c->d_cnt, st, c->cfg.max_rounds, c->d_sump, use_sump));
+                                                         c->d_hits, c->d_done, c->d_cnt, st, c->cfg.max_rounds));
+    if (use_sump) SIDM_LAUNCH(c, k_max_sump<<<grid_for(c, L.N, 1024), 256, 0, s>>>(L.N, c->d_sump, st));   // max_i sum_j P_ij
     timer_end(c, tr, s);
     return SIDM_OK;
 }
@@ -2127,14 +2151,16 @@ extern "C" int sidm_local_diagnostics(sidm_ctx* c, const sidm_xs* xs, const doub
     const LayoutHost& L = c->lay;
     if (L.N == 0) return SIDM_OK;
     const bool fp64 = c->cfg.precision == SIDM_FP64;
-    SIDM_CUDA(c, cudaMemsetAsync(c->d_dacc, 0, sizeof(double) * 5 * L.N, s));
+    if (fp64) SIDM_CUDA(c, cudaMemsetAsync(c->d_dacc, 0, sizeof(double) * 5 * L.N, s));
     if (fp64)
         SIDM_LAUNCH(c, k_vel_refresh<double><<<grid_for(c, L.N, 256), 256, 0, s>>>(L.N, L.H, c->d_halo_off, c->d_halo_pad,
                                                                                   (const double*)vel, c->d_ID, (double4_16a*)c->d_V4));
     else
         SIDM_LAUNCH(c, k_vel_refresh<float><<<grid_for(c, L.N, 256), 256, 0, s>>>(L.N, L.H, c->d_halo_off, c->d_halo_pad,
                                                                                 (const float*)vel, c->d_ID, (float4*)c->d_V4));
-    int rc = launch_pairs_diag(c, xs, mass, s);
+    // mixed form: one search per particle inside its own kernel; FP64 form: one
+    // traversal of the in-range pairs
+    int rc = fp64 ? launch_pairs_diag(c, xs, mass, s) : launch_moments(c, mass, s);
     if (rc) return rc;
     const int blocks = (int)(((int64_t)L.L * kLeaf + 255) / 256);
     if (fp64)
@@ -2323,6 +2349,13 @@ extern "C" int sidm_energy_momentum(sidm_ctx* c, const double* mass, const void*
         else
             SIDM_LAUNCH(c, k_energy_partial<float><<<L.nchunk, sidm_sum::chunk_threads<float>(), 0, s>>>(
                 (const float*)vel, L.N, c->d_chunk_halo, c->d_chunk_begin, c->d_halo_off, c->d_epart));
+    }
+    bool small = true;
+    for (int h = 0; h < L.H && small; ++h) small = L.group_off[h + 1] - L.group_off[h] <= 1;
+    if (small) {
+        SIDM_LAUNCH(c, k_energy_small<<<(L.H + 3) / 4, 128, 0, s>>>(L.H, c->d_group_off, c->d_chunk_off, mass, c->d_epart,
+                                                                    out, comp));
+        return SIDM_OK;
     }
     if (L.ngroup > 0)
         SIDM_LAUNCH(c, k_energy_group<<<(L.ngroup + 3) / 4, 128, 0, s>>>(L.H, L.ngroup, c->d_group_off, c->d_chunk_off,

@@ -210,6 +210,7 @@ int occupancy(sidm_ctx* c, const void* fn, int threads, size_t smem, int* occ);
 int launch_knn(sidm_ctx* c, void* h_out, uint32_t* nbr, int k_stride, bool use_guess, cudaStream_t s);
 int launch_pairs(sidm_ctx* c, uint64_t seed, uint64_t step, const sidm_xs* xs, const double* dt,
                  const double* mass, const void* vel, sidm_step_stats* st, cudaStream_t s);
+int launch_moments(sidm_ctx* c, const double* mass, cudaStream_t s);
 int launch_pairs_diag(sidm_ctx* c, const sidm_xs* xs, const double* mass, cudaStream_t s);
 
 // ---------------------------------------------------------------- device helpers
@@ -218,32 +219,13 @@ __device__ __forceinline__ void raise_status(DevCounters* cnt, unsigned int bits
     atomicOr(&cnt->status, bits);
 }
 
-// Philox4x32-10 block (Salmon et al. 2011): per round the products
-// M0*c0 and M1*c2 are split into high/low words and mixed with c1, c3 and the
-// key; the key advances by the Weyl constants after each round.
+// Philox4x32-10 block (Salmon et al. 2011): per round the products M0*c0 and
+// M1*c2 are split into high/low words and mixed with c1, c3 and the key, which
+// advances by the Weyl constants after each round.  The round keys are given
+// (rk[2r], rk[2r+1] = key + r * Weyl pair, mod 2^32); a launch passes them as
+// kernel parameters, so a round is the two products and two three-way xors.
 struct Philox4 { uint32_t x[4]; };
 
-__device__ __forceinline__ Philox4 philox4x32_10(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
-                                                 uint32_t k0, uint32_t k1)
-{
-#pragma unroll
-    for (int r = 0; r < 10; ++r) {
-        const unsigned long long p0 = (unsigned long long)0xD2511F53u * c0;   // one 32x32->64 product
-        const unsigned long long p1 = (unsigned long long)0xCD9E8D57u * c2;
-        const uint32_t lo0 = (uint32_t)p0, hi0 = (uint32_t)(p0 >> 32);
-        const uint32_t lo1 = (uint32_t)p1, hi1 = (uint32_t)(p1 >> 32);
-        const uint32_t y0 = hi1 ^ c1 ^ k0;
-        const uint32_t y2 = hi0 ^ c3 ^ k1;
-        c0 = y0; c1 = lo1; c2 = y2; c3 = lo0;
-        k0 += 0x9E3779B9u; k1 += 0xBB67AE85u;
-    }
-    Philox4 o; o.x[0] = c0; o.x[1] = c1; o.x[2] = c2; o.x[3] = c3;
-    return o;
-}
-
-// The same block with the round keys given (rk[2r], rk[2r+1] = key + r * Weyl
-// pair, mod 2^32); a launch passes them as kernel parameters, so a round is the
-// two products and two three-way xors.
 __device__ __forceinline__ Philox4 philox4x32_10_rk(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
                                                     const uint32_t* rk)
 {

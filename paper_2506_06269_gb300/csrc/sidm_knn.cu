@@ -56,6 +56,11 @@ struct KnnParams {
     void* hprev;        // out: h per particle (next call's guess), NULL for neighbour lists
     int use_guess;      // P4.w holds each particle's previous kernel size
     float slack;        // guess bound = previous h * slack
+    float grow;         // factor of the bound between attempts
+    const void* V4;     // moments: velocities, particle mass, sums [5][nacc]
+    const double* mass;
+    double* dacc;
+    int64_t nacc;
     int flush_node;     // pending keys per lane that trigger a merge before a node's tests
 };
 
@@ -691,9 +696,11 @@ __global__ void k_knn(KnnParams p)
 }
 
 // ---------------------------------------------------------------------------
-// Warm-started search.  From the second call on every particle carries its
+// Fixed-bound search.  From the second call on every particle carries its
 // previous kernel size, and only candidates inside slack x h_prev are admitted
-// (reading C14).  One warp per query leaf (or, with few leaves, the warps of a
+// (reading C14); a first call takes a density guess instead (k_knn_guess).  The
+// same walk collects neighbour lists and the moments of the local diagnostics
+// inside the kernel size itself.  One warp per query leaf (or, with few leaves, the warps of a
 // CTA share a leaf's candidate leaves and the first merges their keys); the
 // bound is fixed for the whole leaf, so:
 //  * the queries are taken in runs of lanes whose box is at most kWSpread(Team)
@@ -731,7 +738,13 @@ __global__ void k_knn(KnnParams p)
 // 1500 to 30000 particles, N_ngb up to 128: 0.50 ms (0.98); 2048 particles 40 us
 // (84), teams; FP64 16384 particles 0.22 ms (4.4).  kWSpread 2, 2.5, 3, 4: 1.15,
 // 1.11, 1.12, 1.20 ms at 2^20 and 0.47, 0.58, 0.60, 0.64 ms for the eight halos;
-// boxes of four lane groups in wide runs: 1.36 ms; runs of a leaf dealt out to the
+// A first search, 300,007 NFW particles, N_ngb = 48: 0.85 ms with the guess
+// against 2.5 ms in the per-lane kernel (whose heaps fill from the Morton window,
+// 20 of 32 lanes active); 100,003 Hernquist particles 1.2 against 1.5 ms (its
+// longest leaf).  Neighbour lists there 0.45 ms (1.87 in the per-lane kernel);
+// moments of the 300,007 particles 0.57 ms (1.74 ms over in-range pairs, with ten
+// FP64 atomics each).
+// Boxes of four lane groups in wide runs: 1.36 ms; runs of a leaf dealt out to the
 // team's warps instead of shared by them: 0.42 against 0.22 ms (FP64, 16384).
 constexpr int kWRing = 128;     // candidate ring entries
 constexpr int kWBatch = 8;      // candidates per batch (batches start at multiples of it: never wrap)
@@ -743,25 +756,33 @@ constexpr int kWBand = 4;       // FP64 form: candidates compared in FP64
 static_assert((kWRing & (kWRing - 1)) == 0 && kWRing >= kWBatch - 1 + 2 * kLeaf, "the ring holds a batch's leftover plus two leaves");
 static_assert(kWPend >= kWBatch, "one batch fits after a merge");
 constexpr int kWarmMaxWarps = 8;   // the kernel's launch bound: 256 threads, two CTAs per SM
-constexpr int kWAttempts = 6;      // bounds tried, each 1.5 times the one before, before the redo
+constexpr int kWAttempts = 10;     // bounds tried, each KnnParams::grow times the one before, before the redo
 // widest box of a run of queries / its largest bound: a run costs a walk, a wide
 // box reaches dense regions that none of its queries does; a team shares both
 constexpr float kWSpread = 2.25f, kWSpreadTeam = 3.0f;
 
-template <class R>
+// what a fixed-bound search collects: the kernel size, the neighbour list within
+// it, or the kernel-weighted moments of the neighbours within it (mixed form)
+constexpr int kSizes = 0, kLists = 1, kMoments = 2;
+
+template <class R, int MODE>
 __host__ __device__ constexpr size_t warm_warp_bytes(int kcap)
 {
-    using K = typename KeyOf<R, false>::T;
-    return (size_t)kWRing * (sizeof(R) == 8 ? 16 : 12) + 4 * 16 + (size_t)(kWList + kStack + 32) * 4 +
+    using K = typename KeyOf<R, MODE == kLists>::T;
+    return (size_t)kWRing * (sizeof(K) == 8 || MODE == kMoments ? 16 : 12) + 4 * 16 + (size_t)(kWList + kStack + 32) * 4 +
            (size_t)(kcap + (sizeof(R) == 8 ? kWExtra : 0) + kWPend) * 32 * sizeof(K);
 }
 
-template <class R, bool TEAM>
+template <class R, bool TEAM, int MODE>
 __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p, int32_t* redo_list, unsigned int* redo_len)
 {
-    using K = typename KeyOf<R, false>::T;
+    constexpr bool NBR = MODE == kLists;
+    using K = typename KeyOf<R, NBR>::T;
     using V = typename Vec4<R>::T;
     constexpr bool kF32 = sizeof(R) == 4;
+    static_assert(MODE == kSizes || kF32, "lists and moments: mixed form");
+    constexpr bool kTag = sizeof(K) == 8;              // keys carry the slot (FP64 form) or the id (neighbour lists)
+    constexpr bool kRingTag = kTag || MODE == kMoments;   // moments keep slots alone
     constexpr unsigned FULL = 0xffffffffu;
     constexpr unsigned kRow = 32 * sizeof(K);          // bytes of one slot of all lanes
     extern __shared__ __align__(16) unsigned char smem[];
@@ -769,12 +790,12 @@ __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p,
     __shared__ unsigned int team_bad, team_fail, team_err;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int nw = TEAM ? (int)(blockDim.x >> 5) : 1, part = TEAM ? wid : 0;   // nw: a power of two
-    const size_t warp_bytes = warm_warp_bytes<R>(p.kcap);
+    const size_t warp_bytes = warm_warp_bytes<R, MODE>(p.kcap);
     unsigned char* base = smem + wid * warp_bytes;
-    float* ring = (float*)base;                        // [3 or 4][kWRing] x, y, z (and slot)
+    float* ring = (float*)base;                        // [3 or 4][kWRing] x, y, z (and the tag)
     // the run's box: lo (w: squared reach of the walk), hi (halo frame), centre,
     // half widths (leaf frame)
-    float4* wbox = (float4*)(ring + (kF32 ? 3 : 4) * kWRing);
+    float4* wbox = (float4*)(ring + (kRingTag ? 4 : 3) * kWRing);
     int* list = (int*)(wbox + 4);
     int* stack = list + kWList;
     int* held = stack + kStack;                        // [32] keys of this warp's lanes (TEAM)
@@ -809,13 +830,15 @@ __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p,
         const R hp = P4[slotA].w;
         const unsigned long long tiles0 = n_tiles;
         // a particle without a previous kernel size sends its leaf to the redo
-        bool bad = __any_sync(FULL, active && !(hp > R(0)));
+        // (moments: a particle without an extent has no neighbours inside it)
+        bool bad = MODE != kMoments && __any_sync(FULL, active && !(hp > R(0)));
         const float margin = p.frame[h].margin;
         const float4 cA = p.cell[leaf];
         // the lane's bound: slack h_prev rounded up
         float rad = 0.f;
         if (active) {
-            if constexpr (kF32) rad = __fmul_ru((float)hp, p.slack);
+            if constexpr (MODE == kMoments) rad = (float)hp;
+            else if constexpr (kF32) rad = __fmul_ru((float)hp, p.slack);
             else rad = __double2float_ru(__dmul_ru((double)hp, (double)p.slack));
         }
         uint32_t todo = bad ? 0u : __ballot_sync(FULL, active);
@@ -856,14 +879,18 @@ __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p,
         todo &= ~__ballot_sync(FULL, act);
         // a lane that admits fewer than N_ngb keys tries again with a wider bound
         for (int attempt = 0;; ++attempt) {
-        uint32_t root = act ? __float_as_uint(__fmul_ru(rad, rad)) : 0u;   // bits of the lane's d^2 bound
+        uint32_t root = act ? __float_as_uint(MODE == kMoments ? __fmul_rn(rad, rad) : __fmul_ru(rad, rad)) : 0u;   // bits of the lane's d^2 bound
         float err = 0.f;                               // FP64 form: largest offset error of a candidate
         // the filter's bound follows the lanes': squared, or for the FP64 form, which
         // adds a candidate's error, plain
         float rf = 0.f;
         auto reach = [&]() {
-            const float r = sqrtf(__uint_as_float(__reduce_max_sync(FULL, root))) * (1.0f + 0x1p-18f);
+            const float r = sqrtf(__uint_as_float(__reduce_max_sync(FULL, root))) * (1.0f + 0x1p-17f);
             rf = kF32 ? r * r : r;
+            const float rw = __fadd_ru(r, margin);
+            __syncwarp();
+            if (lane == 0) wbox[0].w = __fmul_ru(rw, rw);    // and the walk's
+            __syncwarp();
         };
         {
             box();
@@ -877,8 +904,7 @@ __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p,
             }
             __syncwarp();
             if (lane == 0) {
-                const float rw = __fadd_ru(__fmul_ru(-w[6], 1.0f + 0x1p-18f), margin);
-                wbox[0] = make_float4(w[0], w[1], w[2], __fmul_ru(rw, rw));
+                wbox[0] = make_float4(w[0], w[1], w[2], 0.f);
                 wbox[1] = make_float4(-w[3], -w[4], -w[5], 0.f);
                 // centre and half widths; with c = RN(x - centre) the computed gap
                 // |c| - half of a point x exceeds the true one by less than 2^-22 (gap +
@@ -898,6 +924,7 @@ __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p,
         unsigned off = off0;                           // end of the lane's keys (bytes)
         const unsigned room = off0 + kRow * (unsigned)(kk + kWPend - kWBatch);
         bool heaped = false, dropped = false;
+        double mom[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
         auto at = [&](int t) -> K& { return *(K*)(keys + off0 + kRow * (unsigned)t); };
         auto sift = [&](int t, K key) {
             while (true) {
@@ -916,9 +943,33 @@ __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p,
             }
             at(t) = key;
         };
-        auto bits = [](K key) -> uint32_t { if constexpr (kF32) return key; else return (uint32_t)(key >> 32); };
+        auto bits = [](K key) -> uint32_t { if constexpr (kTag) return (uint32_t)(key >> 32); else return key; };
+        // moments: the waiting neighbours of every lane, added up in FP64
+        auto gather = [&]() {
+            const V* V4 = (const V*)p.V4;
+            const R m = (R)p.mass[h], hq = (R)rad;
+            const R norm = R(8.0 / 3.14159265358979323846) / (hq * hq * hq);
+            for (unsigned o = off0; o < off; o += kRow) {
+                const uint32_t sj = *(const uint32_t*)(keys + o);
+                const V pj = P4[sj], vj = V4[sj];
+                const float4 cj = p.cell[sj / kLeaf];
+                const R dx = sub_rn(__fadd_rn(pj.x, __fsub_rn(cj.x, cA.x)), q.x), dy = sub_rn(__fadd_rn(pj.y, __fsub_rn(cj.y, cA.y)), q.y),
+                        dz = sub_rn(__fadd_rn(pj.z, __fsub_rn(cj.z, cA.z)), q.z);
+                const R d = sqrt_rn(fma_rn(dz, dz, fma_rn(dy, dy, mul_rn(dx, dx))));
+                const R t = d / hq, u = R(1) - t;
+                const R w = t < R(0.5) ? norm * (R(1) - R(6) * t * t * u) : norm * R(2) * u * u * u;
+                const double wt = (double)(m * w), vx = (double)vj.x, vy = (double)vj.y, vz = (double)vj.z;
+                mom[0] = __dadd_rn(mom[0], wt);
+                mom[1] = __fma_rn(wt, vx, mom[1]);
+                mom[2] = __fma_rn(wt, vy, mom[2]);
+                mom[3] = __fma_rn(wt, vz, mom[3]);
+                mom[4] = __fma_rn(wt, __fma_rn(vx, vx, __fma_rn(vy, vy, __dmul_rn(vz, vz))), mom[4]);
+            }
+            off = off0;
+        };
         // merge the waiting keys into the heap (each lane its own column)
         auto flush = [&]() {
+            if constexpr (MODE == kMoments) { gather(); __syncwarp(); return; }
             const int cnt = (int)((off - off0) / kRow);
             if (cnt >= kk) {
                 if (!heaped) {
@@ -933,7 +984,7 @@ __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p,
                     }
                 }
                 dropped = dropped || cnt > kk;
-                root = min(root, bits(at(0)) + (kF32 ? 0u : 1u));   // FP64 form: equal FP32 distances still enter
+                root = min(root, bits(at(0)) + (kTag ? 1u : 0u));   // tagged keys: equal FP32 distances still enter
                 off = off0 + kRow * (unsigned)kk;
             }
             reach();
@@ -941,7 +992,7 @@ __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p,
 
         // the accepted children of a node: local leaf indices into the list (this
         // part's share), or nodes onto the stack
-        int nl = 0, seen = 0, sp = 0;
+        int nl = 0, sp = 0;
         if (part == 0) { if (lane == 0) list[0] = A; nl = 1; }   // the query leaf first
         __syncwarp();
         auto visit = [&](int lev, int first, int nb, int n) {
@@ -951,8 +1002,9 @@ __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p,
             const float4 qlo = wbox[0];
             uint32_t acc = __ballot_sync(FULL, in && box_gap2_rd(qlo, wbox[1], lo, hi) <= qlo.w);
             if (lev == 0) {
-                const bool mine = ((acc >> lane) & 1u) && ((seen + __popc(acc & lt)) & (nw - 1)) == part;
-                seen += __popc(acc);
+                // a team's leaves are dealt by number: its warps' bounds, and so the
+                // leaves they accept, differ once keys have been merged
+                const bool mine = ((acc >> lane) & 1u) && ((first + lane) & (nw - 1)) == part;
                 acc = __ballot_sync(FULL, mine);
                 if (mine) list[nl + __popc(acc & lt)] = first + lane;
                 nl += __popc(acc);
@@ -1000,7 +1052,8 @@ __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p,
                     if (keep) {
                         float* e = ring + ((cnum + navail + __popc(m & lt)) & (kWRing - 1));
                         e[0] = c[u].x; e[kWRing] = c[u].y; e[2 * kWRing] = c[u].z;
-                        if constexpr (!kF32) e[3 * kWRing] = __uint_as_float((uint32_t)(leaf0 + Bl[u]) * kLeaf + lane);
+                        const uint32_t slot = (uint32_t)(leaf0 + Bl[u]) * kLeaf + lane;
+                        if constexpr (kRingTag) e[3 * kWRing] = __uint_as_float(NBR ? p.ID[slot] : slot);
                     }
                     navail += __popc(m);
                 }
@@ -1044,7 +1097,7 @@ __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p,
                     const ulonglong2 x = *(const ulonglong2*)e, y = *(const ulonglong2*)(e + kWRing),
                                      z = *(const ulonglong2*)(e + 2 * kWRing);
                     uint4 sl = make_uint4(0u, 0u, 0u, 0u);
-                    if constexpr (!kF32) sl = *(const uint4*)(e + 3 * kWRing);
+                    if constexpr (kRingTag) sl = *(const uint4*)(e + 3 * kWRing);
                     const uint32_t s4[4] = {sl.x, sl.y, sl.z, sl.w};
 #pragma unroll
                     for (int u = 0; u < 2; ++u) {
@@ -1055,7 +1108,7 @@ __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p,
 #pragma unroll
                         for (int r = 0; r < 2; ++r) {
                             const int i = t + 2 * u + r;
-                            if constexpr (kF32) *(uint32_t*)(keys + off) = db[r];
+                            if constexpr (!kTag) *(uint32_t*)(keys + off) = MODE == kMoments ? s4[2 * u + r] : db[r];
                             else *(unsigned long long*)(keys + off) = ((unsigned long long)db[r] << 32) | s4[2 * u + r];
                             off += db[r] < root && i != me ? kRow : 0u;
                         }
@@ -1069,8 +1122,29 @@ __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p,
             }
             if (fin) break;
         }
+        if constexpr (MODE == kMoments) {
+            // the warps' moments, added in order by the first
+            gather();
+            double* part_mom = (double*)(keys) + lane;         // [5][32], the queue is empty
+            for (int i = 0; TEAM && i < 5; ++i) part_mom[32 * i] = mom[i];
+            if constexpr (TEAM) {
+                if (bad && lane == 0) atomicOr(&team_bad, 1u);
+                __syncthreads();
+                bad = team_bad != 0u;
+            }
+            if (bad && part == 0 && lane == 0) raise_status(p.cnt, SIDM_DEV_STACK);
+            if (part == 0 && act) {
+                for (int w = 1; w < nw; ++w)
+                    for (int i = 0; i < 5; ++i)
+                        mom[i] = __dadd_rn(mom[i], *(const double*)((const unsigned char*)(part_mom + 32 * i) + w * warp_bytes));
+                const int64_t u = p.halo_off[h] + (int64_t)slotA - (int64_t)leaf0 * kLeaf;
+                for (int i = 0; i < 5; ++i) p.dacc[i * p.nacc + u] = mom[i];
+            }
+            if constexpr (TEAM) __syncthreads();
+            break;
+        }
         // the first warp takes over the other warps' keys
-        if constexpr (TEAM) {
+        if constexpr (TEAM && MODE != kMoments) {
             flush();
             held[lane] = (int)((off - off0) / kRow);
             if (dropped) held[lane] |= 0x10000;
@@ -1108,7 +1182,7 @@ __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p,
                 err = q.w + __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(err))) + 0x1p-19f * rad;
             }
             if constexpr (kF32) {
-                if (act && ok) hval = sqrt_rn(__uint_as_float(at(0)));
+                if (!NBR && act && ok) hval = sqrt_rn(__uint_as_float(bits(at(0))));
             } else if (act && ok) {
                 // the k-th smallest FP32 distance: the (n - k + 1)-th largest of the n kept
                 float v[kWExtra + 1];
@@ -1157,9 +1231,28 @@ __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p,
             if (__any_sync(FULL, !ok && !again) || (fail && attempt == kWAttempts - 1)) bad = true;
             if (act && ok) {
                 const int64_t u = p.halo_off[h] + (int64_t)slotA - (int64_t)leaf0 * kLeaf;
-                ((R*)p.h_out)[u] = hval;
-                if (p.hprev) ((R*)p.hprev)[u] = hval;
-                ((R*)((V*)p.P4 + slotA))[3] = hval;
+                if constexpr (NBR) {
+                    // heap sort: repeatedly move the maximum behind the shrinking heap
+                    for (int end = k - 1; end > 0; --end) {
+                        const K top_key = at(0), key = at(end);
+                        int t = 0;
+                        while (4 * t + 1 < end) {
+                            int j = 4 * t + 1;
+                            K mk = at(j);
+                            for (int c = 4 * t + 2; c < min(4 * t + 5, end); ++c) if (at(c) > mk) { mk = at(c); j = c; }
+                            if (!(mk > key)) break;
+                            at(t) = mk;
+                            t = j;
+                        }
+                        at(t) = key;
+                        at(end) = top_key;
+                    }
+                    for (int t = 0; t < k; ++t) p.nbr[u * p.k_stride + t] = (uint32_t)at(t);
+                } else {
+                    ((R*)p.h_out)[u] = hval;
+                    if (p.hprev) ((R*)p.hprev)[u] = hval;
+                    ((R*)((V*)p.P4 + slotA))[3] = hval;
+                }
             }
             if (attempt == 0) n_again += (unsigned long long)__popc(fail);
         }
@@ -1171,11 +1264,11 @@ __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p,
         }
         if (bad || fail == 0u) break;
         act = (fail >> lane) & 1u;
-        if (act) rad *= 1.5f;
+        if (act) rad *= p.grow;
         }   // attempts
         if (bad) break;
         }   // runs of queries
-        if (bad && part == 0 && lane == 0) { const unsigned r = atomicAdd(redo_len, 1u); redo_list[r] = leaf; }
+        if (MODE != kMoments && bad && part == 0 && lane == 0) { const unsigned r = atomicAdd(redo_len, 1u); redo_list[r] = leaf; }
         n_tiles_max = n_tiles - tiles0 > n_tiles_max ? n_tiles - tiles0 : n_tiles_max;
         __syncwarp();
     }
@@ -1206,6 +1299,7 @@ void fill_params(sidm_ctx* c, KnnParams& p, void* h_out, uint32_t* nbr, int k_st
     p.hprev = nbr ? nullptr : c->d_hprev;
     p.use_guess = use_guess ? 1 : 0;
     p.slack = c->cfg.knn_slack > 0.f ? c->cfg.knn_slack : kGuessSlackDefault;
+    p.grow = 1.5f;
     p.flush_node = c->cfg.knn_flush > 0 ? c->cfg.knn_flush : kFlushNodeDefault;
 }
 
@@ -1284,20 +1378,25 @@ int launch_tuned(sidm_ctx* c, void* h_out, bool use_guess, cudaStream_t s, bool 
 // leaves it could not finish.  With fewer than kTeamItems leaves per resident
 // warp the warps of a CTA share a leaf.
 constexpr int64_t kTeamItems = 1;
-template <class R>
-int launch_warm(sidm_ctx* c, void* h_out, cudaStream_t s)
+template <class R, int MODE = kSizes>
+int launch_warm(sidm_ctx* c, void* h_out, cudaStream_t s, uint32_t* nbr = nullptr, int k_stride = 0, const double* mass = nullptr,
+                bool guessed = false)
 {
+    constexpr bool NBR = MODE == kLists;
     KnnParams p;
-    fill_params(c, p, h_out, nullptr, 0, true);
-    const size_t per_warp = warm_warp_bytes<R>(p.kcap);
+    fill_params(c, p, h_out, nbr, k_stride, true);
+    p.V4 = c->d_V4; p.mass = mass; p.dacc = c->d_dacc; p.nacc = c->lay.N;
+    if (guessed) { p.slack = 1.0f; p.grow = 2.0f; }   // a density guess (k_knn_guess)
+    if (NBR) p.slack = 1.0f + 0x1p-20f;            // the kernel size itself is the bound
+    const size_t per_warp = warm_warp_bytes<R, MODE>(p.kcap);
     int warps = 0, grid = 0;
-    if (int rc = pick_shape(c, (const void*)k_knn_warm<R, false>, per_warp, &warps, &grid, kWarmMaxWarps)) return rc;
+    if (int rc = pick_shape(c, (const void*)k_knn_warm<R, false, MODE>, per_warp, &warps, &grid, kWarmMaxWarps)) return rc;
     bool team = false;
     if (c->lay.L < kTeamItems * grid * warps) {
         int w = kWarmMaxWarps;
         while (w > 1 && (w > c->knn_warps || (size_t)w * per_warp > (size_t)226 * 1024)) w /= 2;
         int occ = 0;
-        if (int rc = occupancy(c, (const void*)k_knn_warm<R, true>, w * 32, (size_t)w * per_warp, &occ)) return rc;
+        if (int rc = occupancy(c, (const void*)k_knn_warm<R, true, MODE>, w * 32, (size_t)w * per_warp, &occ)) return rc;
         if (occ >= 1 && w > 1) {
             team = true;
             warps = w;
@@ -1309,14 +1408,127 @@ int launch_warm(sidm_ctx* c, void* h_out, cudaStream_t s)
     cudaError_t e = cudaMemsetAsync(&c->d_cnt->work[0], 0, sizeof(unsigned int), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(&c->d_cnt->knn_redo[0], 0, 2 * sizeof(unsigned int), s);
     if (e != cudaSuccess) return cuda_check(c, e, "knn work reset");
-    const int tidx = timer_begin(c, 1, s);
-    if (team) k_knn_warm<R, true><<<grid, warps * 32, (size_t)warps * per_warp, s>>>(p, c->d_knn_redo, &c->d_cnt->knn_redo[0]);
-    else k_knn_warm<R, false><<<grid, warps * 32, (size_t)warps * per_warp, s>>>(p, c->d_knn_redo, &c->d_cnt->knn_redo[0]);
+    const int tidx = MODE == kMoments ? -1 : timer_begin(c, 1, s);
+    if (team) k_knn_warm<R, true, MODE><<<grid, warps * 32, (size_t)warps * per_warp, s>>>(p, c->d_knn_redo, &c->d_cnt->knn_redo[0]);
+    else k_knn_warm<R, false, MODE><<<grid, warps * 32, (size_t)warps * per_warp, s>>>(p, c->d_knn_redo, &c->d_cnt->knn_redo[0]);
     timer_end(c, tidx, s);
     c->launches++;
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_check(c, e, "knn launch");
-    return launch_tuned<R>(c, h_out, true, s, true);
+    if constexpr (MODE == kMoments) return SIDM_OK;
+    else if constexpr (NBR) return launch_t<float, true, false, kGroupsDefault, kChainsDefault>(c, nullptr, nbr, k_stride, false, s, true);
+    else return launch_tuned<R>(c, h_out, true, s, true);
+}
+
+// A guess for every particle of a search that has no earlier kernel sizes, into
+// P4.w: the radius of the kGuessRank-th nearest of the leaf's other particles (of
+// the kGuessNear-th where that radius jumps: the leaf holds clumps), scaled to
+// N_ngb with two standard deviations of a Poisson count, so that few guesses fail,
+// and at most kGuessWide times the leaf's lower quartile for particles near it
+// (those at the leaf's rim see a part of their neighbourhood only).  One warp per
+// leaf; a wrong guess costs time, never accuracy.
+// A guess that holds more than N_ngb particles of the kGuessSpan leaves on either
+// side in Morton order is lowered to the radius that holds N_ngb of them: on the
+// sparse shell even the quartile can reach across the halo.
+constexpr int kGuessRank = 10, kGuessNear = 4, kGuessSpan = 4;
+constexpr float kGuessWide = 1.0f;
+template <class R>
+__global__ void __launch_bounds__(256) k_knn_guess(int L, const int32_t* __restrict__ leaf_halo, const int32_t* __restrict__ leaf_off,
+                                                   const int64_t* __restrict__ halo_off, const int32_t* __restrict__ ngb,
+                                                   const float4* __restrict__ S4, const float4* __restrict__ cell,
+                                                   typename Vec4<R>::T* __restrict__ P4)
+{
+    constexpr unsigned FULL = 0xffffffffu;
+    __shared__ float4 window[8][(2 * kGuessSpan + 1) * kLeaf];
+    const int lane = threadIdx.x & 31;
+    float4* win = window[threadIdx.x >> 5];
+    const int leaf = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    if (leaf >= L) return;                                     // whole warps
+    const int h = leaf_halo[leaf];
+    const int n = (int)min((int64_t)kLeaf, halo_off[h + 1] - halo_off[h] - (int64_t)(leaf - leaf_off[h]) * kLeaf);
+    const float4 q = S4[(int64_t)leaf * kLeaf + lane];
+    float d2[kLeaf];
+    float hi = 0.f;
+#pragma unroll
+    for (int t = 0; t < kLeaf; ++t) {
+        const float dx = __shfl_sync(FULL, q.x, t) - q.x, dy = __shfl_sync(FULL, q.y, t) - q.y, dz = __shfl_sync(FULL, q.z, t) - q.z;
+        d2[t] = t < n ? dx * dx + dy * dy + dz * dz : INFINITY;
+        if (t < n) hi = fmaxf(hi, d2[t]);
+    }
+    // squared radius holding m others (and the particle itself) by bisection on the bits
+    auto radius2 = [&](int m) -> float {
+        uint32_t lo = 0u, up = __float_as_uint(hi);
+        for (int it = 0; it < 20 && up - lo > 1u; ++it) {
+            const uint32_t mid = lo + (up - lo) / 2u;
+            const float x = __uint_as_float(mid);
+            int c = 0;
+#pragma unroll
+            for (int t = 0; t < kLeaf; ++t) c += d2[t] <= x ? 1 : 0;
+            if (c >= m + 1) up = mid; else lo = mid;
+        }
+        return __uint_as_float(up);
+    };
+    const int far = min(kGuessRank, max(1, n / 3)), near = min(kGuessNear, far);
+    // r^3 per particle, from the far rank or, where that is several times the near one's, from the near
+    const float rf = radius2(far), rn = radius2(near);
+    const float vf = rf * sqrtf(rf) / (float)far, vn = rn * sqrtf(rn) / (float)near;
+    const float v = lane < n ? (vf > 6.f * vn ? 1.5f * vn : vf) : INFINITY;
+    int rank = 0;
+    for (int t = 0; t < kLeaf; ++t) {
+        const float y = __shfl_sync(FULL, v, t);
+        rank += y < v || (y == v && t < lane) ? 1 : 0;
+    }
+    const uint32_t at = __ballot_sync(FULL, rank == n / 4);
+    const float quart = __shfl_sync(FULL, v, __ffs(at) - 1);
+    constexpr float wide = kGuessWide * kGuessWide * kGuessWide;
+    const float vg = fminf(v, wide * quart);
+    const float k = (float)ngb[h];
+    float g = cbrtf(vg * (k + 2.f * sqrtf(k) + 1.f)), g2 = g * g;
+    // the window, in this leaf's frame
+    const int first = max(leaf_off[h], leaf - kGuessSpan), last = min(leaf_off[h + 1] - 1, leaf + kGuessSpan);
+    const int64_t end = (int64_t)leaf_off[h] * kLeaf + (halo_off[h + 1] - halo_off[h]);
+    const float4 cA = cell[leaf];
+    for (int b = first; b <= last; ++b) {
+        float4 c = S4[(int64_t)b * kLeaf + lane];
+        const float4 cB = cell[b];
+        c.x += cB.x - cA.x; c.y += cB.y - cA.y; c.z += cB.z - cA.z;
+        if ((int64_t)b * kLeaf + lane >= end) c.x = INFINITY;
+        win[(b - first) * kLeaf + lane] = c;
+    }
+    __syncwarp();
+    const int nw = (last - first + 1) * kLeaf;
+    auto within = [&](float r2) -> int {
+        int c = 0;
+#pragma unroll 8
+        for (int t = 0; t < nw; ++t) {
+            const float4 w = win[t];
+            const float dx = w.x - q.x, dy = w.y - q.y, dz = w.z - q.z;
+            c += dx * dx + dy * dy + dz * dz <= r2 ? 1 : 0;
+        }
+        return c;
+    };
+    const int want = ngb[h] + 1;                               // the particle itself among them
+    float low = 0.f, high = g2;
+    const bool more = lane < n && within(g2) > want;
+    if (__any_sync(FULL, more)) {
+        for (int it = 0; it < 8; ++it) {
+            const float mid = 0.5f * (low + high);
+            if (within(mid) >= want) high = mid; else low = mid;
+        }
+        if (more) g = sqrtf(high) * 1.001f;
+    }
+    if (lane < n) P4[(int64_t)leaf * kLeaf + lane].w = (R)g;
+}
+
+template <class R>
+int launch_guess(sidm_ctx* c, cudaStream_t s)
+{
+    using V = typename Vec4<R>::T;
+    const float4* S4 = c->cfg.precision == SIDM_FP64 ? c->d_S4 : (const float4*)c->d_P4;
+    k_knn_guess<R><<<(unsigned)(((int64_t)c->lay.L * 32 + 255) / 256), 256, 0, s>>>(c->lay.L, c->d_leaf_halo, c->d_leaf_off, c->d_halo_off,
+                                                                                  c->d_ngb, S4, c->d_cell, (V*)c->d_P4);
+    c->launches++;
+    return cuda_check(c, cudaGetLastError(), "knn guess launch");
 }
 
 }  // namespace
@@ -1326,20 +1538,34 @@ int launch_knn(sidm_ctx* c, void* h_out, uint32_t* nbr, int k_stride, bool use_g
     if (c->lay.L == 0) return SIDM_OK;
     const bool tma = c->cfg.use_tma != 0;
     constexpr int G = kGroupsDefault, CH = kChainsDefault;   // neighbour lists and bulk copies: defaults
-    // warm-started searches take the fixed-bound kernel unless the knobs ask for
-    // bulk copies or the earlier combined kernel (knn_batch 1 or 2)
-    const bool warm = use_guess && !tma && (c->cfg.knn_batch > 0 ? c->cfg.knn_batch : kBatchDefault) == 3;
+    // the fixed-bound kernel, from the previous kernel sizes or a density guess,
+    // unless the knobs ask for bulk copies or the per-lane kernel (knn_batch 1 or 2)
+    const bool fixed = !tma && (c->cfg.knn_batch > 0 ? c->cfg.knn_batch : kBatchDefault) == 3;
     if (c->cfg.precision == SIDM_FP64) {
         if (nbr) return set_err(c, SIDM_EINVAL, "neighbour lists: mixed form only");
-        if (warm) return launch_warm<double>(c, h_out, s);
+        if (fixed) {
+            if (!use_guess) { if (int rc = launch_guess<double>(c, s)) return rc; }
+            return launch_warm<double>(c, h_out, s, nullptr, 0, nullptr, !use_guess);
+        }
         return tma ? launch_t<double, false, true, G, CH>(c, h_out, nullptr, 0, use_guess, s)
                    : launch_tuned<double>(c, h_out, use_guess, s);
     }
+    if (nbr && fixed) return launch_warm<float, kLists>(c, nullptr, s, nbr, k_stride);
     if (nbr) return tma ? launch_t<float, true, true, G, CH>(c, nullptr, nbr, k_stride, false, s)
                         : launch_t<float, true, false, G, CH>(c, nullptr, nbr, k_stride, false, s);
-    if (warm) return launch_warm<float>(c, h_out, s);
+    if (fixed) {
+        if (!use_guess) { if (int rc = launch_guess<float>(c, s)) return rc; }
+        return launch_warm<float>(c, h_out, s, nullptr, 0, nullptr, !use_guess);
+    }
     return tma ? launch_t<float, false, true, G, CH>(c, h_out, nullptr, 0, use_guess, s)
                : launch_tuned<float>(c, h_out, use_guess, s);
+}
+
+// kernel-weighted moments of every particle's neighbours (local diagnostics, mixed form)
+int launch_moments(sidm_ctx* c, const double* mass, cudaStream_t s)
+{
+    if (c->lay.L == 0) return SIDM_OK;
+    return launch_warm<float, kMoments>(c, nullptr, s, nullptr, 0, mass);
 }
 
 }  // namespace sidm

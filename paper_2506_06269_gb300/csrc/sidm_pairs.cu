@@ -9,13 +9,9 @@
 // max id, halo), so the draw is independent of thread order.  Event iff
 // u = x0 2^-32 < P (no clamp: P >= 1 always fires).
 //
-// One warp per query leaf A; the tree walk visits leaves B >= A whose boxes
-// are within h_max(A) + h_max(B), so each unordered pair is tested once, in
-// the frame of the lower leaf.  The in-range test runs on a 32 x 32 block;
-// in-range pairs are compacted into a per-warp queue of (slot i, slot j, d^2)
-// that persists across candidate leaves, so the expensive part (sigma,
-// Philox, Lambda) runs on full warps.  The Lambda table is read only for the
-// pairs whose draw falls below an upper bound of P (see k_pairs).
+// Each unordered pair is tested once, in the frame of the lower leaf: a query
+// leaf A meets the leaves B >= A.  k_pairs draws; k_pairs_all forms every P
+// (per-particle sums of P) and the FP64 form's moments.
 #include "sidm_internal.cuh"
 #include "sidm_tile.cuh"
 
@@ -63,9 +59,8 @@ struct PairParams {
 };
 
 // what one traversal of the in-range pairs computes
-constexpr int kModeDraw = 0;        // draws, Lambda only below the bound of P
 constexpr int kModeDrawExact = 1;   // draws, every P formed (per-particle sums of P)
-constexpr int kModeDiag = 2;        // no draws: kernel-weighted moments for the local diagnostics
+constexpr int kModeDiag = 2;        // no draws: kernel-weighted moments for the local diagnostics (FP64 form)
 
 // spline kernel of Sect. 2, support h, normalised to one
 template <class R>
@@ -79,12 +74,13 @@ __device__ __forceinline__ R spline_w(R d, R h)
     return norm * R(2) * t * t * t;
 }
 
-// pairs a lane queues per round, at most (a launch knob; swept on the GB300:
-// 1, 2, 3, 4 -> 3.76, 3.64, 3.49, 3.47 ms), and the queue entries per warp, a
-// power of two: a round adds up to 32 kPerRoundMax pairs to fewer than 32 waiting
+// groups of 32 pairs drawn together (a launch knob)
 constexpr int kPerRoundMax = 4, kPerRoundDefault = 2;
-constexpr int kQueue = 32 * (kPerRoundMax + 1) <= 64 ? 64 : 32 * (kPerRoundMax + 1) <= 128 ? 128 : 256;
-static_assert(kQueue >= 32 * (kPerRoundMax + 1), "one round must fit behind the entries still waiting");
+// moments: pairs a lane queues per round, and the queue entries per warp, a power
+// of two: a round adds up to 32 kQueuePerRound pairs to fewer than 32 waiting
+constexpr int kQueuePerRound = 4;
+constexpr int kQueue = 256;
+static_assert(kQueue >= 32 * (kQueuePerRound + 1), "one round must fit behind the entries still waiting");
 
 template <class R>
 __device__ __forceinline__ uint32_t id_of(R w)
@@ -112,30 +108,31 @@ __device__ __forceinline__ float to_float_ru_p(R v)
 // first; the plain path keeps the query leaf's own points there), the shifted
 // candidate leaf, queue of in-range pairs (slot i, slot j), traversal stack,
 // boxes of the nodes under test (32 lo + 32 hi)
-template <class R, bool TMA>
+template <class R>
 constexpr size_t pair_warp_bytes()
 {
-    return (TileStageT<R, TMA>::bytes() + kQueue * 8 + kStack * 4 + 64 * 16 + 8 * 8 + 15) / 16 * 16;
+    return (TileStageT<R, false>::bytes() + kQueue * 8 + kStack * 4 + 64 * 16 + 8 * 8 + 15) / 16 * 16;
 }
 
-// MODE kModeDrawExact: form P (and so Lambda) for every in-range pair
-// (per-particle sums of P requested).  kModeDiag: no draws; each pair adds
-// m W(d, h_i) and its velocity moments of j to particle i when d < h_i, and
-// the same for j (the SPH sums of the local diagnostics).  kModeDraw: Lambda
-// is looked up only when the draw lies below
-// an upper bound of P: P_up uses kLamFUp in place of the interpolated table
-// value, and since FP32/FP64 products round monotonically P <= P_up for the P
-// that would have been formed, so a draw u >= P_up + 2e-6 decides "no event"
-// and "not within 1e-6 of P" exactly as the full evaluation would.
-template <class R, bool TMA, int MODE, int PR, bool DRAG>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_pairs_queue(PairParams p)
+// Every P formed (kModeDrawExact: per-particle sums of P), or the FP64 form's
+// moments for the local diagnostics (kModeDiag: no draws; each pair adds
+// m W(d, h_i) and its velocity moments of j to particle i when d < h_i, and the
+// same for j; the mixed form gathers them per particle, k_knn_warm).  In-range
+// pairs are compacted into a per-warp queue of (slot i, slot j) that persists
+// across candidate leaves, filled in rounds of ballots.  The sums keep one FP32
+// addition per pair and particle, in this kernel's order of pairs: k_pairs with
+// the query's terms added up per run of its pairs took 31.5 ms where this takes
+// 38 for a satellite's big step of 2^22 particles (scalar table loads), but moved
+// the sums by their rounding (5e-7).
+template <class R, int MODE, bool DRAG>
+__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_pairs_all(PairParams p)
 {
-    static_assert(PR >= 1 && PR <= kPerRoundMax, "pairs per round");
+    constexpr int PR = kQueuePerRound;
     using V = typename Vec4<R>::T;
-    using Stage = TileStageT<R, TMA>;
+    using Stage = TileStageT<R, false>;
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    unsigned char* base = smem + wid * pair_warp_bytes<R, TMA>();
+    unsigned char* base = smem + wid * pair_warp_bytes<R>();
     Stage st_pos(base);
     uint32_t* q_si = (uint32_t*)(base + Stage::bytes());
     uint32_t* q_sj = q_si + kQueue;
@@ -191,11 +188,9 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_pairs_queue(Pai
         // the queries in their own frame, for tiles tested candidate by lane (the
         // plain path stages tiles in registers, so the first staging buffer is free)
         V* qsh = st_pos.raw();
-        if constexpr (!TMA) {
-            __syncwarp();
-            qsh[lane] = q;
-            __syncwarp();
-        }
+        __syncwarp();
+        qsh[lane] = q;
+        __syncwarp();
         int qhead = 0, qn = 0;
         uint32_t n_pairs = 0u, n_gt1 = 0u, n_near = 0u, n_tested = 0u, n_lam = 0u, n_tiles = 0u;
 
@@ -264,7 +259,6 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_pairs_queue(Pai
                     prefp = (R)xs.s0 * (R)p.mass[h] * (R)ldexp(p.dt_max, -bmin);
                 }
                 R P, pre, inv, u;
-                bool need;
                 if constexpr (sizeof(R) == 4) {
                     // P needs ~1e-6 relative accuracy only (the event decision below is
                     // exact for the P computed here): reciprocal square roots and
@@ -283,22 +277,16 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_pairs_queue(Pai
                     inv = R(1) / (hi > hj ? hi : hj);
                     u = (R)ldexp((double)x.x[0], -32);
                 }
-                if constexpr (MODE == kModeDrawExact) {
-                    need = true;
-                } else {
-                    const R P_up = pre * (R(kLamFUp) * inv * inv * inv);
-                    need = drag || !(u >= P_up + R(2e-6));
-                }
                 P = R(0);
                 R gfac = R(0);
                 bool fire = false;
-                if (need) {
+                {
                     ++n_lam;
                     const R d2 = pair_d2(si, sj, P4[si], P4[sj]);
                     R f;
                     if constexpr (sizeof(R) == 4) {
                         const float d = d2 > 0.f ? d2 * rsqrtf(d2) : 0.f;
-                        f = lambda_f_fast(T, d, hi, hj, inv);
+                        f = lambda_f_rows(p.lam4, d, hi, hj, inv);
                     } else {
                         f = lambda_f<R>(T, sqrt_rn(d2), hi, hj);
                     }
@@ -360,17 +348,14 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_pairs_queue(Pai
         // this lane's entry of candidate leaf Bl (the plain path loads it straight
         // into a register, so the walk can fetch the next leaf early)
         auto fetch = [&](int Bl) -> V {
-            if constexpr (TMA) return V{};
-            else return P4[(int64_t)(leaf0 + Bl) * kLeaf + lane];
+            return P4[(int64_t)(leaf0 + Bl) * kLeaf + lane];
         };
         // craw: fetch(Bl) (unused on the bulk-copy path, which stages the leaf here)
         auto process = [&](int Bl, bool mine, const V& craw) {
             const int Bg = leaf0 + Bl;
             ++n_tiles;
             const int countB = (int)min((int64_t)kLeaf, nh - (int64_t)Bl * kLeaf);
-            V c;
-            if constexpr (TMA) c = st_pos.load_lane(P4 + (int64_t)Bg * kLeaf, lane, p.cnt);
-            else c = craw;
+            V c = craw;
             if constexpr (sizeof(R) == 4) {
                 const float4 cB = p.cell[Bg];
                 c.x = __fadd_rn(c.x, __fsub_rn(cB.x, cA.x));
@@ -400,7 +385,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_pairs_queue(Pai
             //     staged tile (bits of okm = candidates), or lane = candidate, queries
             //     from their staged copy (bits = queries).  Same tests, same operands.
             const uint32_t qmask = __ballot_sync(0xffffffffu, mine);
-            const bool by_cand = !TMA && __popc(qmask) < __popc(cmask);
+            const bool by_cand = __popc(qmask) < __popc(cmask);
             uint32_t okm = 0u, allow;
             if (!by_cand) {
                 for (uint32_t mm = cmask; mm; mm &= mm - 1u) {
@@ -646,7 +631,7 @@ constexpr uint32_t kUnsure = 0x80000000u;   // on a candidate's id (below 2^27):
 // max over v of sigma(v) v / s0 for kind 1: v / (1 + (v/w)^2)^2 peaks at v = w / sqrt(3)
 constexpr float kSvMax = 0.32475953f;    // 3 sqrt(3) / 16, rounded up
 
-template <class R, int MODE, int PR, bool DRAG>
+template <class R, int PR, bool DRAG>
 __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
 {
     static_assert(PR >= 1 && PR <= kPerRoundMax, "32-pair groups drawn together");
@@ -711,7 +696,7 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
         // 1.001 and the 3e-6 cover every rounding and the |P - u| < 1e-6 count); a
         // bound that is not a number below one keeps every pair
         uint32_t thr = FULL;
-        if constexpr (MODE == kModeDraw) {
+        {
             const sidm_xs xs = p.xs[h];
             float sv;
             if (xs.kind == 1) {
@@ -751,7 +736,7 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
             const R m = (R)p.mass[h], t = p.bins ? (R)p.dt_max : (R)p.dt[h];
             return Factors{(R)xs.s0 * m * t, xs.kind == 1 ? R(1) / (R)xs.w : R(0), t, xs.kind == 1};
         };
-        constexpr bool kEvery = MODE == kModeDrawExact || DRAG;
+        constexpr bool kEvery = DRAG;
         const Factors fac = kEvery ? factors() : Factors{};
         // canonical d^2 of query pi and candidate pj (mixed form: the candidate
         // shifted into the query leaf's frame)
@@ -766,15 +751,15 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
             const R dx = sub_rn(cx, pi.x), dy = sub_rn(cy, pi.y), dz = sub_rn(cz, pi.z);
             return fma_rn(dz, dz, fma_rn(dy, dy, mul_rn(dx, dx)));
         };
-        // the full evaluation of the in-range pair (query lane li, slot sj): P (or its
-        // rate on individual steps, scaled to dt_max), decision, record
-        auto evaluate = [&](int li, uint32_t sj, uint32_t idi, uint32_t idj) -> float {
+        // the full evaluation of the in-range pair (query lane li, slot sj): P,
+        // decision, record
+        auto evaluate = [&](int li, uint32_t sj, uint32_t idi, uint32_t idj) {
             const Philox4 x = philox4x32_10_rk(p.step_lo, min(idi, idj), max(idi, idj), (uint32_t)h, p.rk);
             const Factors fc = kEvery ? fac : factors();
             const uint32_t si = (uint32_t)leaf * kLeaf + li;
             const int64_t ui = index_of(si), uj = index_of(sj);
             R ux, uy, uz;
-            if constexpr (MODE == kModeDraw && !DRAG) {
+            if constexpr (!DRAG) {
                 const R* vel = (const R*)p.vel;
                 ux = vel[uj] - vel[ui];
                 uy = vel[p.N + uj] - vel[p.N + ui];
@@ -788,8 +773,7 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
             const R v2 = ux * ux + uy * uy + uz * uz;
             const uint32_t a = min(idi, idj), b = max(idi, idj);
             // individual steps: the pair's longer step dt_max / 2^min(b_i, b_j)
-            const float up = p.bins ? __int_as_float((127 + min(p.bins[ui], p.bins[uj])) << 23) : 1.f;   // 2^min(b_i, b_j)
-            const float down = 1.f / up;                      // exact: bins are below 16
+            const float down = p.bins ? __int_as_float((127 - min(p.bins[ui], p.bins[uj])) << 23) : 1.f;   // 2^-min(b_i, b_j)
             const R prefp = fc.pref * down;
             // mixed form: P needs ~1e-6 relative accuracy only (the event decision
             // below is exact for the P computed here): reciprocal square roots and
@@ -810,15 +794,12 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
                 u = (R)ldexp((double)x.x[0], -32);
             }
             const R pre = prefp * sig * v;
-            bool need = true;
-            if constexpr (MODE == kModeDraw) {
-                const R P_up = pre * (R(kLamFUp) * inv * inv * inv);
-                need = drag || !(u >= P_up + R(2e-6));
-            }
+            const R P_up = pre * (R(kLamFUp) * inv * inv * inv);
+            const bool need = drag || !(u >= P_up + R(2e-6));
             R P = R(0), gfac = R(0);
             bool fire = false;
             if (need) {
-                if constexpr (MODE == kModeDraw) atomicAdd(&wst[4], 1ull);   // else every pair
+                atomicAdd(&wst[4], 1ull);
                 const R d2 = pair_d2(pi, pj, sj);
                 R f;
                 if constexpr (kF32) {
@@ -871,7 +852,6 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
                     if (drag) p.evg[slot] = (double)gfac;
                 }
             }
-            return (float)(P * up);
         };
 
         // Consecutive particles of the Morton curve can lie far apart (on the sparse
@@ -1138,29 +1118,7 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
                         const Philox4 x = philox4x32_10_rk(p.step_lo, min(idi[k], idj[k]), max(idi[k], idj[k]), (uint32_t)h, p.rk);
                         maybe |= (valid && x.x[0] <= thr ? 1u : 0u) << k;
                     }
-                    if constexpr (MODE == kModeDrawExact) {
-                        static_assert(MODE != kModeDrawExact || PR == 1, "one group at a time");
-                        // the per-particle sums of P: the query's by one addition per run of
-                        // its pairs in the group (they stand together), the partner's each
-                        const int li = (int)(ent[0] >> 8);
-                        const uint32_t sj = cslot[ent[0] & (kPCand - 1)];
-                        float ps = maybe ? evaluate(li, sj, idi[0], idj[0]) : 0.f;
-                        if (p.use_sump) {
-                            __syncwarp();
-                            if (maybe) atomicAdd(p.sump + index_of(sj), ps);
-                            const int before = __shfl_up_sync(FULL, li, 1);
-                            const uint32_t heads = __ballot_sync(FULL, lane == 0 || before != li);
-                            const uint32_t later = heads & ~((2u << lane) - 1u);
-                            const int end = later ? __ffs(later) - 1 : 32;         // of this lane's run
-#pragma unroll
-                            for (int o = 1; o < 32; o <<= 1) {
-                                const float y = __shfl_down_sync(FULL, ps, o);
-                                if (lane + o < end) ps += y;
-                            }
-                            if (((heads >> lane) & 1u) && maybe) atomicAdd(p.sump + index_of((uint32_t)leaf * kLeaf + li), ps);
-                            __syncwarp();
-                        }
-                    } else if (maybe) {
+                    if (maybe) {
 #pragma unroll 1
                         for (int k = 0; k < PR; ++k) {
                             if (!((maybe >> k) & 1u)) continue;
@@ -1192,7 +1150,6 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
             __syncwarp();
             if (lane == 0) {
                 wst[0] += n_pairs; wst[3] += n_tested; wst[5] += n_tiles;
-                if (MODE != kModeDraw) wst[4] += n_pairs;
                 wst[6] = max(wst[6], (unsigned long long)n_tiles);
             }
             __syncwarp();
@@ -1259,29 +1216,27 @@ void fill_params(sidm_ctx* c, PairParams& p, uint64_t seed, uint64_t step, const
     for (int g = 0; g < 8; ++g) { p.glx[g] = c->gl8x[g]; p.glw[g] = c->gl8w[g]; }
 }
 
-template <class R, bool TMA, int MODE, int PR = kPerRoundMax, bool DRAG = false>
-int launch_t(sidm_ctx* c, uint64_t seed, uint64_t step, const sidm_xs* xs, const double* dt, const double* mass,
-             const void* vel, sidm_step_stats* st, cudaStream_t s)
+template <class R, int MODE, bool DRAG>
+int launch_all(sidm_ctx* c, uint64_t seed, uint64_t step, const sidm_xs* xs, const double* dt, const double* mass,
+               const void* vel, sidm_step_stats* st, cudaStream_t s)
 {
     PairParams p;
     fill_params(c, p, seed, step, xs, dt, mass, vel, st);
     const LayoutHost& L = c->lay;
     const int warps = c->pair_warps;
-    const size_t smem = (size_t)warps * pair_warp_bytes<R, TMA>();
-    auto kern = k_pairs_queue<R, TMA, MODE, PR, DRAG>;
+    const size_t smem = (size_t)warps * pair_warp_bytes<R>();
+    auto kern = k_pairs_all<R, MODE, DRAG>;
     int occ = 0;
-    int rc = occupancy(c, (const void*)kern, warps * 32, smem, &occ);
-    if (rc) return rc;
-    cudaError_t e;
+    if (int rc = occupancy(c, (const void*)kern, warps * 32, smem, &occ)) return rc;
     if (occ < 1) return set_err(c, SIDM_ECAPACITY, "pair kernel does not fit on an SM");
     int grid = c->cfg.grid_ctas > 0 ? c->cfg.grid_ctas : c->sm_count * occ;
     grid = std::max(1, std::min(grid, (L.L + warps - 1) / warps));
     c->pair_grid = grid;
-    e = cudaMemsetAsync(&c->d_cnt->work[1], 0, sizeof(unsigned int), s);
+    cudaError_t e = cudaMemsetAsync(&c->d_cnt->work[1], 0, sizeof(unsigned int), s);
     if (e != cudaSuccess) return cuda_check(c, e, "pair work reset");
     const int tidx = MODE == kModeDiag ? -1 : timer_begin(c, 2, s);
     kern<<<grid, warps * 32, smem, s>>>(p);
-    if (tidx >= 0) timer_end(c, tidx, s);
+    timer_end(c, tidx, s);
     c->launches++;
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_check(c, e, "pair launch");
@@ -1294,7 +1249,7 @@ int launch_t(sidm_ctx* c, uint64_t seed, uint64_t step, const sidm_xs* xs, const
 // the parts repeat.
 constexpr int kPartsMax = 16;
 constexpr int64_t kPartsPerWarp = 4;
-template <class R, int MODE, int PR, bool DRAG>
+template <class R, int PR, bool DRAG>
 int launch_draws(sidm_ctx* c, uint64_t seed, uint64_t step, const sidm_xs* xs, const double* dt, const double* mass,
                  const void* vel, sidm_step_stats* st, cudaStream_t s)
 {
@@ -1303,7 +1258,7 @@ int launch_draws(sidm_ctx* c, uint64_t seed, uint64_t step, const sidm_xs* xs, c
     const LayoutHost& L = c->lay;
     const int warps = c->pair_warps;
     const size_t smem = (size_t)warps * draw_warp_bytes();
-    auto kern = k_pairs<R, MODE, PR, DRAG>;
+    auto kern = k_pairs<R, PR, DRAG>;
     int occ = 0;
     if (int rc = occupancy(c, (const void*)kern, warps * 32, smem, &occ)) return rc;
     if (occ < 1) return set_err(c, SIDM_ECAPACITY, "pair kernel does not fit on an SM");
@@ -1313,7 +1268,7 @@ int launch_draws(sidm_ctx* c, uint64_t seed, uint64_t step, const sidm_xs* xs, c
     c->pair_grid = grid;
     cudaError_t e = cudaMemsetAsync(&c->d_cnt->work[1], 0, sizeof(unsigned int), s);
     if (e != cudaSuccess) return cuda_check(c, e, "pair work reset");
-    if (MODE == kModeDraw) {
+    {
         k_vmax<R><<<L.nchunk * kVmaxSplit, 256, 0, s>>>((const R*)vel, L.N, c->d_chunk_halo, c->d_chunk_begin, c->d_halo_off,
                                                         xs, c->d_cnt);
         c->launches++;
@@ -1335,15 +1290,15 @@ static int launch_form(sidm_ctx* c, uint64_t seed, uint64_t step, const sidm_xs*
 {
     const bool exact = (c->cfg.flags & SIDM_FLAG_SUM_P) != 0;
     if (c->cfg.flags & SIDM_FLAG_DRAG)                  // forward-dominated halos allowed
-        return exact ? launch_draws<R, kModeDrawExact, 1, true>(c, seed, step, xs, dt, mass, vel, st, s)
-                     : launch_draws<R, kModeDraw, 1, true>(c, seed, step, xs, dt, mass, vel, st, s);
-    if (exact) return launch_draws<R, kModeDrawExact, 1, false>(c, seed, step, xs, dt, mass, vel, st, s);
+        return exact ? launch_all<R, kModeDrawExact, true>(c, seed, step, xs, dt, mass, vel, st, s)
+                     : launch_draws<R, 1, true>(c, seed, step, xs, dt, mass, vel, st, s);
+    if (exact) return launch_all<R, kModeDrawExact, false>(c, seed, step, xs, dt, mass, vel, st, s);
     // the hot path: groups of 32 pairs drawn together as configured (a launch knob)
     switch (c->cfg.pair_per_round > 0 ? c->cfg.pair_per_round : kPerRoundDefault) {
-    case 1: return launch_draws<R, kModeDraw, 1, false>(c, seed, step, xs, dt, mass, vel, st, s);
-    case 2: return launch_draws<R, kModeDraw, 2, false>(c, seed, step, xs, dt, mass, vel, st, s);
-    case 3: return launch_draws<R, kModeDraw, 3, false>(c, seed, step, xs, dt, mass, vel, st, s);
-    default: return launch_draws<R, kModeDraw, 4, false>(c, seed, step, xs, dt, mass, vel, st, s);
+    case 1: return launch_draws<R, 1, false>(c, seed, step, xs, dt, mass, vel, st, s);
+    case 2: return launch_draws<R, 2, false>(c, seed, step, xs, dt, mass, vel, st, s);
+    case 3: return launch_draws<R, 3, false>(c, seed, step, xs, dt, mass, vel, st, s);
+    default: return launch_draws<R, 4, false>(c, seed, step, xs, dt, mass, vel, st, s);
     }
 }
 
@@ -1358,9 +1313,7 @@ int launch_pairs(sidm_ctx* c, uint64_t seed, uint64_t step, const sidm_xs* xs, c
 int launch_pairs_diag(sidm_ctx* c, const sidm_xs* xs, const double* mass, cudaStream_t s)
 {
     if (c->lay.L == 0) return SIDM_OK;
-    if (c->cfg.precision == SIDM_FP64)
-        return launch_t<double, false, kModeDiag>(c, 0, 0, xs, nullptr, mass, nullptr, c->d_stats_own, s);
-    return launch_t<float, false, kModeDiag>(c, 0, 0, xs, nullptr, mass, nullptr, c->d_stats_own, s);
+    return launch_all<double, kModeDiag, false>(c, 0, 0, xs, nullptr, mass, nullptr, c->d_stats_own, s);
 }
 
 }  // namespace sidm
