@@ -1517,6 +1517,13 @@ static int radix_sort(sidm_ctx* c, unsigned long long*& ka, uint32_t*& va, unsig
     const int64_t tiles = cdiv(n, kTile);
     if (tiles > c->sort_tiles_cap || passes < 1 || passes > kMaxPasses || n >= ((int64_t)1 << 32))
         return set_err(c, SIDM_ECAPACITY, "radix sort scratch too small");
+    // up to kSmallKeys keys: every pass in one launch of one CTA
+    if (n <= kSmallKeys) {
+        SIDM_LAUNCH(c, k_sort_small<<<1, kSmallThreads, kSmallSmemBytes, s>>>(ka, va, (int)n, passes, kb, vb));
+        std::swap(ka, kb);
+        std::swap(va, vb);
+        return SIDM_OK;
+    }
     uint32_t* hist = c->d_sort_hist;
     uint32_t* tickets = hist + kMaxPasses * 256;
     if (!counted) {
@@ -1606,6 +1613,9 @@ extern "C" int sidm_create(sidm_ctx** out, const sidm_config* cfg)
     e = cudaFuncSetAttribute(sidm_sort::k_sort_pass, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)sidm_sort::kSmemBytes);
     if (e != cudaSuccess) return fail("cudaFuncSetAttribute k_sort_pass", e);
+    e = cudaFuncSetAttribute(sidm_sort::k_sort_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sidm_sort::kSmallSmemBytes);
+    if (e != cudaSuccess) return fail("cudaFuncSetAttribute k_sort_small", e);
 
     const int64_t N = cfg->n_max, H = cfg->halo_max;
     const int64_t Lmax = N / kLeaf + H + 1;

@@ -372,4 +372,104 @@ __global__ void __launch_bounds__(kThreads, kPassCtas) k_sort_pass(const unsigne
     }
 }
 
+// All passes of a small sort in one launch: one CTA keeps up to kSmallKeys keys in
+// shared memory and ranks them like a tile of k_sort_pass (warp w owns the keys
+// w * 32 m .. of m per lane), so the order is the same stable one.  Latency-bound:
+// a pass is a few barriers, against a launch, a cleared status and a look-back for
+// each digit: a cell build of 2048 particles takes 71 us instead of 118.
+constexpr int kSmallThreads = 1024, kSmallWarps = kSmallThreads / 32, kSmallItems = 8;
+constexpr int kSmallKeys = kSmallThreads * kSmallItems;
+struct SmallSmem {
+    unsigned long long key[kSmallKeys];
+    uint32_t val[kSmallKeys];
+    uint32_t wcnt[kSmallWarps][256];
+    uint32_t tstart[256];
+    uint32_t wsum[8];
+};
+constexpr size_t kSmallSmemBytes = sizeof(SmallSmem);
+
+__global__ void __launch_bounds__(kSmallThreads, 1) k_sort_small(const unsigned long long* __restrict__ kin,
+                                                                const uint32_t* __restrict__ vin, int n, int passes,
+                                                                unsigned long long* __restrict__ kout,
+                                                                uint32_t* __restrict__ vout)
+{
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    SmallSmem& S = *reinterpret_cast<SmallSmem*>(smem_raw);
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const uint32_t lt = (1u << lane) - 1u;
+    const int items = (n + kSmallThreads - 1) / kSmallThreads;
+    const int base = warp * 32 * items + lane;
+    unsigned long long k[kSmallItems];
+    uint32_t v[kSmallItems], rk[kSmallItems];
+#pragma unroll
+    for (int r = 0; r < kSmallItems; ++r) {
+        const int s = base + 32 * r;
+        const bool ok = r < items && s < n;
+        k[r] = ok ? kin[s] : 0ull;
+        v[r] = ok ? vin[s] : 0u;
+    }
+    for (int p = 0; p < passes; ++p) {
+        const int shift = 8 * p;
+        for (int i = lane; i < 256; i += 32) S.wcnt[warp][i] = 0u;
+        __syncwarp();
+#pragma unroll
+        for (int r = 0; r < kSmallItems; ++r) {
+            if (r >= items) break;                        // the same in every lane
+            const bool ok = base + 32 * r < n;
+            const uint32_t d = (uint32_t)(k[r] >> shift) & 255u;
+            const uint32_t peers = match_digit(d, ok);
+            const uint32_t before = ok ? S.wcnt[warp][d] : 0u;
+            rk[r] = before + (uint32_t)__popc(peers & lt);
+            __syncwarp();
+            if (ok && (peers & lt) == 0u) S.wcnt[warp][d] = before + (uint32_t)__popc(peers);
+            __syncwarp();
+        }
+        __syncthreads();
+        // thread t < 256 owns digit t: the warps' offsets inside its run, then the
+        // runs' starts
+        uint32_t run = 0u, inc = 0u;
+        if (t < 256) {
+#pragma unroll 8
+            for (int w = 0; w < kSmallWarps; ++w) {
+                const uint32_t c = S.wcnt[w][t];
+                S.wcnt[w][t] = run;
+                run += c;
+            }
+            inc = run;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += y;
+            }
+            if (lane == 31) S.wsum[warp] = inc;
+        }
+        __syncthreads();
+        if (t < 256) {
+            uint32_t before = 0u;
+#pragma unroll
+            for (int w = 0; w < 8; ++w) before += w < warp ? S.wsum[w] : 0u;
+            S.tstart[t] = before + inc - run;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < kSmallItems; ++r) {
+            if (r < items && base + 32 * r < n) {
+                const uint32_t d = (uint32_t)(k[r] >> shift) & 255u;
+                const uint32_t pos = S.tstart[d] + S.wcnt[warp][d] + rk[r];
+                S.key[pos] = k[r];
+                S.val[pos] = v[r];
+            }
+        }
+        __syncthreads();
+        if (p + 1 < passes) {
+#pragma unroll
+            for (int r = 0; r < kSmallItems; ++r) {
+                const int s = base + 32 * r;
+                if (r < items && s < n) { k[r] = S.key[s]; v[r] = S.val[s]; }
+            }
+        }
+    }
+    for (int s = t; s < n; s += kSmallThreads) { kout[s] = S.key[s]; vout[s] = S.val[s]; }
+}
+
 }  // namespace sidm_sort
