@@ -49,8 +49,8 @@ N_SM, LANES_PER_SM = 152, 128
 # algorithmic lane operations per unit of the two ALU-bound kernels: the operation
 # counts of the formulas as written, not counts of issued instructions
 OPS_PER_TEST = 10          # canonical d^2 (3 sub, 1 mul, 2 fma), sum, square, compare, ballot
-OPS_PER_PAIR = 121         # |v_ij| + sigma(v) + Philox4x32-10 + upper bound of P + draw decision + bookkeeping
-OPS_PER_LAMBDA = 50        # sqrt(d^2) + Lambda table (bicubic, 16 loads) + P + exact decision, when looked up
+OPS_PER_PAIR = 102         # Philox4x32-10 (90) + order of the ids, integer bound of the draw, queueing (12)
+OPS_PER_LAMBDA = 200       # |v_ij|, sigma(v), Philox again, sqrt(d^2), Lambda table (bicubic, 16 loads), P, exact decision
 OPS_PER_KNN_CAND = 8       # canonical d^2 (6) + key compare (2)
 # the kernel-size search as the scope table counts it: about 6 N_ngb candidate
 # distances of about 9 FP32 operations per particle
