@@ -1193,6 +1193,19 @@ __global__ void __launch_bounds__(sidm_sum::chunk_threads<R>()) k_energy_partial
     sidm_sum::chunk_sums(vel, N, b, e, part + 8 * (int64_t)c);
 }
 
+// FP64 velocities of few chunks: a cluster per chunk
+__global__ void __cluster_dims__(sidm_sum::kSplitF64, 1, 1) __launch_bounds__(32)
+    k_energy_partial_cluster(const double* __restrict__ vel, int64_t N, const int32_t* __restrict__ chunk_halo,
+                             const int64_t* __restrict__ chunk_begin, const int64_t* __restrict__ halo_off,
+                             double* __restrict__ part)
+{
+    const int c = (int)(blockIdx.x / sidm_sum::kSplitF64);
+    const int64_t b = chunk_begin[c];
+    int64_t e = b + kChunk;
+    if (e > halo_off[chunk_halo[c] + 1]) e = halo_off[chunk_halo[c] + 1];
+    sidm_sum::chunk_sums_cluster(vel, N, b, e, part + 8 * (int64_t)c);
+}
+
 // First merge level: one warp per group of up to kGroupChunks consecutive
 // chunks of a halo (groups numbered halo by halo).
 __global__ void k_energy_group(int H, int ngroup, const int32_t* __restrict__ group_off,
@@ -2353,7 +2366,13 @@ extern "C" int sidm_energy_momentum(sidm_ctx* c, const double* mass, const void*
     SIDM_CUDA(c, ensure_device(c));
     const LayoutHost& L = c->lay;
     if (L.nchunk > 0) {
-        if (c->cfg.precision == SIDM_FP64)
+        // FP64: a cluster per chunk while there are fewer chunks than SMs.  The whole call, a
+        // CTA per chunk against a cluster: 189 -> 99 us (1 chunk), 189 -> 113 (64), 191 -> 169
+        // (128, half of them short), but 1146 -> 1298 at 1024, where every SM has work anyway.
+        if (c->cfg.precision == SIDM_FP64 && L.nchunk < c->sm_count)
+            SIDM_LAUNCH(c, k_energy_partial_cluster<<<(unsigned)L.nchunk * sidm_sum::kSplitF64, 32, 0, s>>>(
+                (const double*)vel, L.N, c->d_chunk_halo, c->d_chunk_begin, c->d_halo_off, c->d_epart));
+        else if (c->cfg.precision == SIDM_FP64)
             SIDM_LAUNCH(c, k_energy_partial<double><<<L.nchunk, sidm_sum::chunk_threads<double>(), 0, s>>>(
                 (const double*)vel, L.N, c->d_chunk_halo, c->d_chunk_begin, c->d_halo_off, c->d_epart));
         else

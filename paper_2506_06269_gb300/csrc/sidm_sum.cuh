@@ -38,6 +38,8 @@
 // over the 256 threads.
 #pragma once
 
+#include <cooperative_groups.h>
+
 #include <cstdint>
 
 namespace sidm_sum {
@@ -239,6 +241,19 @@ __device__ __forceinline__ void chunk_sums(const float* __restrict__ vel, int64_
     }
 }
 
+// particle s added to the four FP64 sums of a thread
+__device__ __forceinline__ void add_particle(const double* __restrict__ vel, int64_t N, int64_t s, DD (&acc)[4])
+{
+    const double x = vel[s], y = vel[N + s], z = vel[2 * N + s];
+    double q = __dmul_rn(x, x);
+    q = __dadd_rn(q, __dmul_rn(y, y));
+    q = __dadd_rn(q, __dmul_rn(z, z));
+    dd_add(acc[0], q);
+    dd_add(acc[1], x);
+    dd_add(acc[2], y);
+    dd_add(acc[3], z);
+}
+
 // One chunk [b, e) of FP64 velocities: compensated sums in a fixed order.
 // Called by all kThreadsF64 threads of the CTA.
 __device__ __forceinline__ void chunk_sums(const double* __restrict__ vel, int64_t N, int64_t b, int64_t e,
@@ -247,16 +262,7 @@ __device__ __forceinline__ void chunk_sums(const double* __restrict__ vel, int64
     constexpr int kThreads = kThreadsF64;
     __shared__ DD sh[4][kThreads];
     DD acc[4] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
-    for (int64_t s = b + threadIdx.x; s < e; s += kThreads) {
-        const double x = vel[s], y = vel[N + s], z = vel[2 * N + s];
-        double q = __dmul_rn(x, x);
-        q = __dadd_rn(q, __dmul_rn(y, y));
-        q = __dadd_rn(q, __dmul_rn(z, z));
-        dd_add(acc[0], q);
-        dd_add(acc[1], x);
-        dd_add(acc[2], y);
-        dd_add(acc[3], z);
-    }
+    for (int64_t s = b + threadIdx.x; s < e; s += kThreads) add_particle(vel, N, s, acc);
 #pragma unroll
     for (int a = 0; a < 4; ++a) sh[a][threadIdx.x] = acc[a];
     __syncthreads();
@@ -275,6 +281,44 @@ __device__ __forceinline__ void chunk_sums(const double* __restrict__ vel, int64
 __device__ __forceinline__ DD shfl_down_dd(const DD& x, int o)
 {
     return DD{__shfl_down_sync(0xffffffffu, x.s, o), __shfl_down_sync(0xffffffffu, x.c, o)};
+}
+
+// The same sums of one chunk, in the same order, by a cluster of kSplitF64 CTAs of 32
+// threads: CTA r holds threads 32 r .. 32 r + 31; the tree's upper levels read the
+// accumulators of CTA r + w, the lower ones are shuffles.  The FP64 pipe (about 40
+// operations per particle at a sixteenth of the FP32 rate) is the bound, so fewer
+// chunks than SMs leave most of the chip idle with a CTA per chunk.
+constexpr int kSplitF64 = kThreadsF64 / 32;
+__device__ __forceinline__ void chunk_sums_cluster(const double* __restrict__ vel, int64_t N, int64_t b, int64_t e,
+                                                   double* __restrict__ out8)
+{
+    namespace cg = cooperative_groups;
+    __shared__ DD sh[4][32];
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank(), lane = (int)threadIdx.x;
+    DD acc[4] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
+#pragma unroll 4
+    for (int64_t s = b + rank * 32 + lane; s < e; s += kThreadsF64) add_particle(vel, N, s, acc);
+    for (int w = kSplitF64 / 2; w > 0; w >>= 1) {
+        if (rank >= w && rank < 2 * w)                     // written once: a CTA leaves the tree here
+#pragma unroll
+            for (int a = 0; a < 4; ++a) sh[a][lane] = acc[a];
+        cluster.sync();
+        if (rank < w) {
+            const DD* other = cluster.map_shared_rank(&sh[0][0], rank + w);
+#pragma unroll
+            for (int a = 0; a < 4; ++a) dd_merge(acc[a], other[a * 32 + lane]);
+        }
+    }
+    cluster.sync();                                        // no CTA ends while its memory is read
+    if (rank != 0) return;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int a = 0; a < 4; ++a) dd_merge(acc[a], shfl_down_dd(acc[a], o));
+    if (lane == 0)                                         // only lane 0 holds the whole tree
+#pragma unroll
+        for (int a = 0; a < 4; ++a) { out8[2 * a] = acc[a].s; out8[2 * a + 1] = acc[a].c; }
 }
 
 constexpr int kGroupChunks = 32;   // chunks per first-level group
