@@ -376,7 +376,8 @@ __global__ void __launch_bounds__(kThreads, kPassCtas) k_sort_pass(const unsigne
 // shared memory and ranks them like a tile of k_sort_pass (warp w owns the keys
 // w * 32 m .. of m per lane), so the order is the same stable one.  Latency-bound:
 // a pass is a few barriers, against a launch, a cleared status and a look-back for
-// each digit: a cell build of 2048 particles takes 71 us instead of 118.
+// each digit.  Cell build of 3000, 5000, 8192 particles: 71, 83, 99 us, with one
+// launch per pass 118, 120, 126; the line lies where the shared memory ends.
 constexpr int kSmallThreads = 1024, kSmallWarps = kSmallThreads / 32, kSmallItems = 8;
 constexpr int kSmallKeys = kSmallThreads * kSmallItems;
 struct SmallSmem {
