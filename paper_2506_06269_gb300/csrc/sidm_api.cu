@@ -1715,7 +1715,7 @@ extern "C" int sidm_create(sidm_ctx** out, const sidm_config* cfg)
         std::vector<float> Tf(T.begin(), T.end());
         e = cudaMalloc(&c->d_lam, Tf.size() * 4); if (e != cudaSuccess) return fail("cudaMalloc lam", e);
         e = cudaMemcpy(c->d_lam, Tf.data(), Tf.size() * 4, cudaMemcpyHostToDevice);
-        if (e == cudaSuccess && (cfg->flags & (SIDM_FLAG_SUM_P | SIDM_FLAG_DRAG))) {
+        if (e == cudaSuccess && (cfg->flags & SIDM_FLAG_DRAG) && !(cfg->flags & SIDM_FLAG_SUM_P)) {
             std::vector<float4> T4(Tf.size(), make_float4(0.f, 0.f, 0.f, 0.f));
             for (int r = 0; r < kLamNR; ++r)
                 for (int x = 0; x + 3 < kLamNX; ++x) {

@@ -173,7 +173,7 @@ struct sidm_ctx {
 
     // Lambda table (float or double [kLamNR][kLamNX])
     void* d_lam = nullptr;
-    float4* d_lam4 = nullptr;          // mixed form with per-pair lookups: (f[x], .., f[x + 3]) per entry
+    float4* d_lam4 = nullptr;          // mixed form, forward-dominated halos: (f[x], .., f[x + 3]) per entry
 
     int knn_grid = 0, pair_grid = 0, knn_warps = 4, pair_warps = 4;
 

@@ -36,7 +36,7 @@ struct PairParams {
     const void* vel;    // the caller's velocities [3][N] (unchanged until the resolve)
     int64_t N;
     const void* lam;
-    const float4* lam4; // the mixed form's table as groups of four along x (contexts that look up every pair)
+    const float4* lam4; // the mixed form's table as groups of four along x (forward-dominated halos, k_pairs)
     const sidm_xs* xs;
     const double* dt;
     const double* mass;
@@ -119,11 +119,15 @@ constexpr size_t pair_warp_bytes()
 // m W(d, h_i) and its velocity moments of j to particle i when d < h_i, and the
 // same for j; the mixed form gathers them per particle, k_knn_warm).  In-range
 // pairs are compacted into a per-warp queue of (slot i, slot j) that persists
-// across candidate leaves, filled in rounds of ballots.  The sums keep one FP32
-// addition per pair and particle, in this kernel's order of pairs: k_pairs with
-// the query's terms added up per run of its pairs took 31.5 ms where this takes
-// 38 for a satellite's big step of 2^22 particles (scalar table loads), but moved
-// the sums by their rounding (5e-7).
+// across candidate leaves, filled in rounds of ballots.  The sums take one FP32
+// addition per pair and particle, in this kernel's order of pairs within a warp
+// and in the order of arrival between warps, so their last bits differ from run
+// to run.  What would change them for good is left out: the query's terms added
+// up per run of its pairs in k_pairs (31.5 ms where this takes 38 of a satellite's
+// big step of 2^22 particles; 5e-7 off), and FP64 sums rounded once (89.2 against
+// 86.7 ms a big step; 1e-7 to 1e-6 off, the FP32 order's own rounding).  The table
+// is read by scalar loads: rows of four (lambda_f_rows) give the same bits and
+// 87.4 ms.
 template <class R, int MODE, bool DRAG>
 __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_pairs_all(PairParams p)
 {
@@ -286,7 +290,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_pairs_all(PairP
                     R f;
                     if constexpr (sizeof(R) == 4) {
                         const float d = d2 > 0.f ? d2 * rsqrtf(d2) : 0.f;
-                        f = lambda_f_rows(p.lam4, d, hi, hj, inv);
+                        f = lambda_f_fast(T, d, hi, hj, inv);
                     } else {
                         f = lambda_f<R>(T, sqrt_rn(d2), hi, hj);
                     }
