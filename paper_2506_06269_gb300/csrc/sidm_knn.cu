@@ -1125,6 +1125,7 @@ __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p,
         if constexpr (MODE == kMoments) {
             // the warps' moments, added in order by the first
             gather();
+            __syncwarp();                                      // the sums go where other lanes' queued slots were
             double* part_mom = (double*)(keys) + lane;         // [5][32], the queue is empty
             for (int i = 0; TEAM && i < 5; ++i) part_mom[32 * i] = mom[i];
             if constexpr (TEAM) {
