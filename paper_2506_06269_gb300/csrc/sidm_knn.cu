@@ -787,7 +787,7 @@ __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p,
     constexpr unsigned kRow = 32 * sizeof(K);          // bytes of one slot of all lanes
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int team_leaf;
-    __shared__ unsigned int team_bad, team_fail, team_err;
+    __shared__ unsigned int team_bad, team_stop, team_fail, team_err;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int nw = TEAM ? (int)(blockDim.x >> 5) : 1, part = TEAM ? wid : 0;   // nw: a power of two
     const size_t warp_bytes = warm_warp_bytes<R, MODE>(p.kcap);
@@ -1258,10 +1258,12 @@ __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p,
             if (attempt == 0) n_again += (unsigned long long)__popc(fail);
         }
         if constexpr (TEAM) {
-            if (wid == 0 && lane == 0) { team_fail = fail; if (bad) team_bad = 1u; }
+            // written between this attempt's two barriers only (team_bad may be set
+            // again by a warp that has begun the next attempt)
+            if (wid == 0 && lane == 0) { team_fail = fail; team_stop = bad ? 1u : 0u; }
             __syncthreads();
             fail = team_fail;
-            bad = team_bad != 0u;
+            bad = team_stop != 0u;
         }
         if (bad || fail == 0u) break;
         act = (fail >> lane) & 1u;
