@@ -490,15 +490,16 @@ __global__ void k_diag_final(int L, const int32_t* __restrict__ leaf_halo, const
     out[4 * N + u] = (R)(sqrt(4.0 * 3.14159265358979323846 * G / (rho * nu * nu)) / se);
 }
 
-// Largest kernel size of every leaf (into lo.w).  The FP64 form's FP32 search
-// takes w = h (1 + 2^-19) + e, e the offset's error (S4.w on entry), in place of h:
-// then an in-range pair has d < w_i + w_j in FP32 arithmetic, and a pair with
+// Largest kernel size of every leaf (into lo.w).  The FP64 form's FP32 search of
+// pairs takes the reach w = h (1 + 2^-19) + e, e the offset's error (S4.w), in place
+// of h: then an in-range pair has d < w_i + w_j in FP32 arithmetic, and a pair with
 // d^2 < (w_i + w_j)^2 (1 - 2^-11) is in range for certain, unless e exceeds
-// 2^-14 h for one of them (w stored with a minus sign).
+// 2^-14 h for one of them (w stored with a minus sign).  The reach has an array of
+// its own: kernel sizes may be found again on the same build, and need e then.
 template <class R>
 __global__ void k_leaf_hmax(int L, int H, const int32_t* __restrict__ leaf_halo, const int32_t* __restrict__ leaf_off,
                             const int64_t* __restrict__ halo_off, const typename Vec4<R>::T* __restrict__ P4,
-                            float4* __restrict__ S4, float4* __restrict__ nlo)
+                            const float4* __restrict__ S4, float* __restrict__ reach, float4* __restrict__ nlo)
 {
     const int lane = threadIdx.x & 31;
     const int leaf = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -510,10 +511,9 @@ __global__ void k_leaf_hmax(int L, int H, const int32_t* __restrict__ leaf_halo,
     if (lane < cntl) {
         const R hv = P4[(int64_t)leaf * kLeaf + lane].w;
         if constexpr (sizeof(R) == 8) {
-            float* w = &S4[(int64_t)leaf * kLeaf + lane].w;
-            const float e = *w;
+            const float e = S4[(int64_t)leaf * kLeaf + lane].w;
             m = __fadd_ru(__fmul_ru(__double2float_ru((double)hv), 1.0f + 0x1p-19f), e);
-            *w = e > 0x1p-14f * (float)hv ? -m : m;
+            reach[(int64_t)leaf * kLeaf + lane] = e > 0x1p-14f * (float)hv ? -m : m;
         } else {
             m = (float)hv;
         }
@@ -1562,7 +1562,7 @@ static void free_all(sidm_ctx* c)
 {
     void* ptrs[] = {c->d_halo_off, c->d_halo_pad, c->d_leaf_off, c->d_lvl_off, c->d_top, c->d_ngb, c->d_leaf_halo, c->d_knn_redo,
                     c->d_chunk_halo, c->d_chunk_begin, c->d_frame, c->d_key, c->d_key2, c->d_val, c->d_val2,
-                    c->d_sort_status, c->d_sort_hist, c->d_P4, c->d_S4, c->d_V4, c->d_ID, c->d_cell, c->d_cellb, c->d_nlo, c->d_nhi, c->d_perm, c->d_tmp_pos,
+                    c->d_sort_status, c->d_sort_hist, c->d_P4, c->d_S4, c->d_reach, c->d_V4, c->d_ID, c->d_cell, c->d_cellb, c->d_nlo, c->d_nhi, c->d_perm, c->d_tmp_pos,
                     c->d_tmp_vel, c->d_tmp_id, c->d_claim, c->d_hits, c->d_done, c->d_ev, c->d_sump,
                     c->d_stats_own, c->d_cnt, c->d_epart, c->d_chunk_off, c->d_group_off, c->d_gpart, c->d_lam, c->d_lam4, c->d_hprev, c->d_dacc, c->d_halo_ord,
                     c->d_evg, c->d_lkey, c->d_lval, c->d_lstart, c->d_llen, c->d_lptr, c->d_lact,
@@ -1660,7 +1660,7 @@ extern "C" int sidm_create(sidm_ctx** out, const sidm_config* cfg)
     ALLOC(c->d_sort_status, 256 * c->sort_tiles_cap);
     ALLOC(c->d_sort_hist, sidm_sort::kMaxPasses * 257);
     e = cudaMalloc(&c->d_P4, (size_t)Npad * 4 * rs); if (e != cudaSuccess) return fail("cudaMalloc P4", e);
-    if (fp64) ALLOC(c->d_S4, Npad);
+    if (fp64) { ALLOC(c->d_S4, Npad); ALLOC(c->d_reach, Npad); }
     e = cudaMalloc(&c->d_V4, (size_t)Npad * 4 * rs); if (e != cudaSuccess) return fail("cudaMalloc V4", e);
     ALLOC(c->d_ID, Npad);
     ALLOC(c->d_cell, Lmax);
@@ -1963,10 +1963,10 @@ extern "C" int sidm_kernel_sizes(sidm_ctx* c, const int32_t* n_ngb, void* h_dev,
     c->ngb_prev = c->ngb_host;
     if (c->cfg.precision == SIDM_FP64)
         SIDM_LAUNCH(c, k_leaf_hmax<double><<<(L.L * 32 + 255) / 256, 256, 0, s>>>(L.L, L.H, c->d_leaf_halo, c->d_leaf_off,
-                                                                                 c->d_halo_off, (const double4_16a*)c->d_P4, c->d_S4, c->d_nlo));
+                                                                                 c->d_halo_off, (const double4_16a*)c->d_P4, c->d_S4, c->d_reach, c->d_nlo));
     else
         SIDM_LAUNCH(c, k_leaf_hmax<float><<<(L.L * 32 + 255) / 256, 256, 0, s>>>(L.L, L.H, c->d_leaf_halo, c->d_leaf_off,
-                                                                               c->d_halo_off, (const float4*)c->d_P4, c->d_S4, c->d_nlo));
+                                                                               c->d_halo_off, (const float4*)c->d_P4, c->d_S4, c->d_reach, c->d_nlo));
     for (int l = 1; l < L.nlev; ++l) {
         const int cnt = L.lvl_off[(size_t)l * (L.H + 1) + L.H] - L.lvl_off[(size_t)l * (L.H + 1)];
         SIDM_LAUNCH(c, k_tree_level<<<std::max(1, (cnt * 32 + 255) / 256), 256, 0, s>>>(l, L.H, c->d_lvl_off, c->d_nlo, c->d_nhi));

@@ -117,7 +117,8 @@ struct sidm_ctx {
 
     // particles (padded per halo to multiples of 32 slots)
     void* d_P4 = nullptr;              // float4 (ox,oy,oz,h) | double4 (x,y,z,h)
-    float4* d_S4 = nullptr;            // FP64 form: FP32 offsets to the leaf's cell corner; w: see k_gather, k_leaf_hmax
+    float4* d_S4 = nullptr;            // FP64 form: FP32 offsets to the leaf's cell corner; w: bound of their error (k_gather)
+    float* d_reach = nullptr;          // FP64 form: reach of the FP32 pair search (k_leaf_hmax)
     void* d_V4 = nullptr;              // float4 (vx,vy,vz,id) | double4
     uint32_t* d_ID = nullptr;          // ids by slot
     float4* d_cell = nullptr;          // [Lmax] leaf frame origin relative to O

@@ -30,7 +30,8 @@ struct PairParams {
     const float4* nlo;
     const float4* nhi;
     const void* P4;
-    const void* S4;     // FP32 offsets and reach: mixed form P4, FP64 form see k_leaf_hmax
+    const void* S4;     // FP32 offsets (mixed form: P4, with the kernel size)
+    const float* reach; // FP64 form: reach in place of the kernel size (k_leaf_hmax)
     const void* V4;
     const uint32_t* ID;
     const void* vel;    // the caller's velocities [3][N] (unchanged until the resolve)
@@ -598,8 +599,8 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_pairs_all(PairP
 //  * one warp scan of the masks' bit counts per batch gives every lane its place
 //    in the warp's queue of (query lane, candidate) pairs, which is emptied 32
 //    pairs at a time, all lanes busy.
-// The FP64 form runs the same search on FP32 offsets (S4: reach w = h and the
-// rounding errors' bound, k_leaf_hmax), where a pair is out of range, in range
+// The FP64 form runs the same search on FP32 offsets (S4) with a reach w = h and
+// the rounding errors' bound (k_leaf_hmax), where a pair is out of range, in range
 // for certain, or (about 1 in 10^3) settled by its FP64 distance before its draw;
 // only pairs whose draw can fire take FP64 arithmetic.  2^20 NFW halo: 2.8 ms
 // per launch against 39 ms with every test and P on the FP64 pipe, 16384
@@ -693,6 +694,7 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
             continue;
         }
         float4 q = S4[slotA];
+        if constexpr (!kF32) q.w = p.reach[slotA];
         // FP64 form: a pair below this share of (w_i + w_j)^2 is in range for certain
         const float sure = kF32 ? 1.f : q.w < 0.f ? 0.f : 1.0f - 0x1p-11f;
         if constexpr (!kF32) q.w = fabsf(q.w);
@@ -978,6 +980,7 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
                 for (int u = 0; u < 2; ++u) {
                     const uint32_t s = (uint32_t)(leaf0 + Bl[u]) * kLeaf + lane;
                     c[u] = S4[s];
+                    if constexpr (!kF32) c[u].w = p.reach[s];
                     cB[u] = p.cell[leaf0 + Bl[u]];
                     id[u] = p.ID[s];
                     if constexpr (!kF32) {
@@ -1203,7 +1206,7 @@ void fill_params(sidm_ctx* c, PairParams& p, uint64_t seed, uint64_t step, const
     p.H = L.H; p.L = L.L;
     p.leaf_halo = c->d_leaf_halo; p.leaf_off = c->d_leaf_off; p.halo_off = c->d_halo_off;
     p.lvl_off = c->d_lvl_off; p.top = c->d_top; p.frame = c->d_frame; p.cell = c->d_cell;
-    p.nlo = c->d_nlo; p.nhi = c->d_nhi; p.P4 = c->d_P4; p.S4 = c->cfg.precision == SIDM_FP64 ? (const void*)c->d_S4 : c->d_P4; p.V4 = c->d_V4; p.ID = c->d_ID; p.lam = c->d_lam; p.lam4 = c->d_lam4;
+    p.nlo = c->d_nlo; p.nhi = c->d_nhi; p.P4 = c->d_P4; p.S4 = c->cfg.precision == SIDM_FP64 ? (const void*)c->d_S4 : c->d_P4; p.reach = c->d_reach; p.V4 = c->d_V4; p.ID = c->d_ID; p.lam = c->d_lam; p.lam4 = c->d_lam4;
     p.vel = vel; p.N = L.N; p.parts = 1;
     p.xs = xs; p.dt = dt; p.mass = mass;
     p.seed_lo = (uint32_t)seed; p.seed_hi = (uint32_t)(seed >> 32); p.step_lo = (uint32_t)step;
