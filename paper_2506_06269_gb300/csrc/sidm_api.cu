@@ -122,9 +122,10 @@ __global__ void __launch_bounds__(256) k_bbox(const double* __restrict__ pos, in
     }
 }
 
-// Halo frame: 2^E > largest extent, O = floor(min / 2^E) 2^E per axis.
+// Halo frame: 2^E > largest extent, O = floor(min / 2^E) 2^E per axis.  scaled: FP32
+// lengths in units of 2^E (the FP64 form).
 __global__ void k_frame(int H, const int64_t* __restrict__ halo_off, const unsigned long long* __restrict__ bb,
-                        HaloFrame* __restrict__ fr)
+                        HaloFrame* __restrict__ fr, int scaled)
 {
     int h = blockIdx.x * blockDim.x + threadIdx.x;
     if (h >= H) return;
@@ -141,9 +142,12 @@ __global__ void k_frame(int H, const int64_t* __restrict__ halo_off, const unsig
     for (int a = 0; a < 3; ++a) f.O[a] = ldexp(floor(ldexp(mn[a], -E)), E);
     f.E = E;
     f.qs = ldexp(1.0, kMortonBits - E - 1);
-    f.cube = (float)ldexp(1.0, E + 1);
-    f.margin = (float)ldexp(1.0, E + 1 - 20);
-    f.fine = (float)ldexp(1.0, E + 1 - kMortonBits);
+    const int sc = scaled ? min(max(E, -1000), 1000) : 0;    // both powers finite and normal
+    f.down = ldexp(1.0, -sc);
+    f.up = ldexp(1.0, sc);
+    f.cube = (float)ldexp(1.0, E + 1 - sc);
+    f.margin = (float)ldexp(1.0, E + 1 - 20 - sc);
+    f.fine = (float)ldexp(1.0, E + 1 - kMortonBits - sc);
     fr[h] = f;
 }
 
@@ -231,13 +235,13 @@ __global__ void k_leaf_fill(int L, int H, const int32_t* __restrict__ leaf_off, 
                                  (float)compact3(k >> 2) * fine, 0.f);
     cell[leaf] = c;
     const HaloFrame& f = fr[h];
-    cellb[leaf] = make_double4(__dadd_rn(f.O[0], (double)c.x), __dadd_rn(f.O[1], (double)c.y),
-                               __dadd_rn(f.O[2], (double)c.z), 0.0);
+    cellb[leaf] = make_double4(__dadd_rn(f.O[0], (double)c.x * f.up), __dadd_rn(f.O[1], (double)c.y * f.up),
+                               __dadd_rn(f.O[2], (double)c.z * f.up), 0.0);
 }
 
 // Gather into Morton order (the FP64 form): sorted user arrays (scratch),
 // internal padded tracks, permutation.  S4 gets the FP32 offset to the leaf's
-// cell corner and, in w, a bound of its error: 2^-24 per axis of the largest
+// cell corner (in the halo's FP32 unit) and, in w, a bound of its error: 2^-24 per axis of the largest
 // offset and twice the rounding of the corner's FP64 position, with room.
 template <class R>
 __global__ void k_gather(int64_t N, int H, const int64_t* __restrict__ halo_off, const int64_t* __restrict__ halo_pad,
@@ -273,11 +277,11 @@ __global__ void k_gather(int64_t N, int H, const int64_t* __restrict__ halo_off,
         P4[slot] = p;
         const double4 b = cellb[slot / kLeaf];
         float4 o;
-        o.x = __double2float_rn(__dsub_rn(x[0], b.x));
-        o.y = __double2float_rn(__dsub_rn(x[1], b.y));
-        o.z = __double2float_rn(__dsub_rn(x[2], b.z));
         const HaloFrame& f = fr[h];
-        const float far = __double2float_ru(fmax(fmax(fabs(f.O[0]), fabs(f.O[1])), fabs(f.O[2])));
+        o.x = __double2float_rn(__dsub_rn(x[0], b.x) * f.down);
+        o.y = __double2float_rn(__dsub_rn(x[1], b.y) * f.down);
+        o.z = __double2float_rn(__dsub_rn(x[2], b.z) * f.down);
+        const float far = __double2float_ru(fmax(fmax(fabs(f.O[0]), fabs(f.O[1])), fabs(f.O[2])) * f.down);
         o.w = __fadd_ru(__fmul_ru(0x1p-22f, fmaxf(fmaxf(fabsf(o.x), fabsf(o.y)), fabsf(o.z))),
                         __fmul_ru(0x1p-50f, __fadd_ru(far, f.cube)));
         S4[slot] = o;
@@ -369,7 +373,7 @@ __global__ void k_leaf_bbox(int L, int64_t N, const int32_t* __restrict__ leaf_h
     float mn[3], mx[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        const double y = __dsub_rn(pos[a * N + s], f.O[a]);
+        const double y = __dsub_rn(pos[a * N + s], f.O[a]) * f.down;
         mn[a] = __double2float_rd(y);
         mx[a] = __double2float_ru(y);
     }
@@ -499,7 +503,8 @@ __global__ void k_diag_final(int L, const int32_t* __restrict__ leaf_halo, const
 template <class R>
 __global__ void k_leaf_hmax(int L, int H, const int32_t* __restrict__ leaf_halo, const int32_t* __restrict__ leaf_off,
                             const int64_t* __restrict__ halo_off, const typename Vec4<R>::T* __restrict__ P4,
-                            const float4* __restrict__ S4, float* __restrict__ reach, float4* __restrict__ nlo)
+                            const HaloFrame* __restrict__ fr, const float4* __restrict__ S4, float* __restrict__ reach,
+                            float4* __restrict__ nlo)
 {
     const int lane = threadIdx.x & 31;
     const int leaf = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -512,8 +517,9 @@ __global__ void k_leaf_hmax(int L, int H, const int32_t* __restrict__ leaf_halo,
         const R hv = P4[(int64_t)leaf * kLeaf + lane].w;
         if constexpr (sizeof(R) == 8) {
             const float e = S4[(int64_t)leaf * kLeaf + lane].w;
-            m = __fadd_ru(__fmul_ru(__double2float_ru((double)hv), 1.0f + 0x1p-19f), e);
-            reach[(int64_t)leaf * kLeaf + lane] = e > 0x1p-14f * (float)hv ? -m : m;
+            const double hs = (double)hv * fr[h].down;
+            m = __fadd_ru(__fmul_ru(__double2float_ru(hs), 1.0f + 0x1p-19f), e);
+            reach[(int64_t)leaf * kLeaf + lane] = e > 0x1p-14f * (float)hs ? -m : m;
         } else {
             m = (float)hv;
         }
@@ -1855,7 +1861,8 @@ static int build_impl(sidm_ctx* c, double* pos, R* vel, uint32_t* id, cudaStream
     SIDM_CUDA(c, cudaMemsetAsync(c->d_cnt->bbox, 0xFF, sizeof(unsigned long long) * 3 * H, s));
     SIDM_CUDA(c, cudaMemsetAsync(c->d_cnt->bbox + 3 * H, 0x00, sizeof(unsigned long long) * 3 * H, s));
     SIDM_LAUNCH(c, k_bbox<<<L.nchunk * kBboxSplit, 256, 0, s>>>(pos, N, c->d_chunk_halo, c->d_chunk_begin, c->d_halo_off, H, c->d_cnt->bbox));
-    SIDM_LAUNCH(c, k_frame<<<(H + 127) / 128, 128, 0, s>>>(H, c->d_halo_off, c->d_cnt->bbox, c->d_frame));
+    SIDM_LAUNCH(c, k_frame<<<(H + 127) / 128, 128, 0, s>>>(H, c->d_halo_off, c->d_cnt->bbox, c->d_frame,
+                                                        c->cfg.precision == SIDM_FP64 ? 1 : 0));
     if (int rc = sort_prepare(c, s)) return rc;
     SIDM_LAUNCH(c, k_keys<<<grid_for(c, N, 256), 256, 0, s>>>(pos, N, c->d_halo_off, H, c->d_frame, c->d_key, c->d_val,
                                                                L.sort_passes, c->d_sort_hist));
@@ -1963,10 +1970,10 @@ extern "C" int sidm_kernel_sizes(sidm_ctx* c, const int32_t* n_ngb, void* h_dev,
     c->ngb_prev = c->ngb_host;
     if (c->cfg.precision == SIDM_FP64)
         SIDM_LAUNCH(c, k_leaf_hmax<double><<<(L.L * 32 + 255) / 256, 256, 0, s>>>(L.L, L.H, c->d_leaf_halo, c->d_leaf_off,
-                                                                                 c->d_halo_off, (const double4_16a*)c->d_P4, c->d_S4, c->d_reach, c->d_nlo));
+                                                                                 c->d_halo_off, (const double4_16a*)c->d_P4, c->d_frame, c->d_S4, c->d_reach, c->d_nlo));
     else
         SIDM_LAUNCH(c, k_leaf_hmax<float><<<(L.L * 32 + 255) / 256, 256, 0, s>>>(L.L, L.H, c->d_leaf_halo, c->d_leaf_off,
-                                                                               c->d_halo_off, (const float4*)c->d_P4, c->d_S4, c->d_reach, c->d_nlo));
+                                                                               c->d_halo_off, (const float4*)c->d_P4, c->d_frame, c->d_S4, c->d_reach, c->d_nlo));
     for (int l = 1; l < L.nlev; ++l) {
         const int cnt = L.lvl_off[(size_t)l * (L.H + 1) + L.H] - L.lvl_off[(size_t)l * (L.H + 1)];
         SIDM_LAUNCH(c, k_tree_level<<<std::max(1, (cnt * 32 + 255) / 256), 256, 0, s>>>(l, L.H, c->d_lvl_off, c->d_nlo, c->d_nhi));

@@ -32,6 +32,11 @@ constexpr uint32_t kIdLimit = 1u << 27;
 struct HaloFrame {
     double O[3];
     double qs;         // Morton quantisation scale 2^(17-E-1) (a power of two)
+    // the halo's FP32 lengths (leaf corners and boxes, the FP64 form's offsets and
+    // reaches, and the three below) are the caller's times 2^-s, s = 0 in the mixed
+    // form, E in the FP64 form: there only FP32 helpers of FP64 results are scaled, so
+    // that their squares stay in FP32's range in any unit of length
+    double down, up;   // 2^-s, 2^s
     int E;
     float cube;        // 2^(E+1)
     float margin;      // pruning margin: 2^(E+1) * 2^-20 (canonical vs exact distance)

@@ -304,8 +304,9 @@ __global__ void k_knn(KnnParams p)
         if constexpr (sizeof(R) == 4) {
             pq = make_float3(__fadd_rn(cA.x, (float)q.x), __fadd_rn(cA.y, (float)q.y), __fadd_rn(cA.z, (float)q.z));
         } else {
-            pq = make_float3(__double2float_rn((double)q.x - fr.O[0]), __double2float_rn((double)q.y - fr.O[1]),
-                             __double2float_rn((double)q.z - fr.O[2]));
+            pq = make_float3(__double2float_rn(((double)q.x - fr.O[0]) * fr.down),
+                             __double2float_rn(((double)q.y - fr.O[1]) * fr.down),
+                             __double2float_rn(((double)q.z - fr.O[2]) * fr.down));
         }
         // boxes of the query points of each group of 32 / G consecutive
         // lanes (shared memory): a candidate is kept if it lies within the
@@ -332,7 +333,9 @@ __global__ void k_knn(KnnParams p)
         }
         auto my_r2 = [&]() -> float {
             if (!act) return -1.0f;
-            float r = to_float_ru<R>(sqrt_ru(key_d2<R, NBR>(root)));
+            R rr = sqrt_ru(key_d2<R, NBR>(root));
+            if constexpr (sizeof(R) == 8) rr *= fr.down;   // to the halo's FP32 unit
+            float r = to_float_ru<R>(rr);
             r = __fadd_ru(__fmul_ru(r, 1.0f + 0x1p-20f), fr.margin);
             return __fmul_ru(r, r);
         };
@@ -434,8 +437,9 @@ __global__ void k_knn(KnnParams p)
                 if constexpr (sizeof(R) == 4) {
                     pc = make_float3(__fadd_rn(cA.x, c.x), __fadd_rn(cA.y, c.y), __fadd_rn(cA.z, c.z));
                 } else {
-                    pc = make_float3(__double2float_rn((double)c.x - fr.O[0]), __double2float_rn((double)c.y - fr.O[1]),
-                                     __double2float_rn((double)c.z - fr.O[2]));
+                    pc = make_float3(__double2float_rn(((double)c.x - fr.O[0]) * fr.down),
+                                     __double2float_rn(((double)c.y - fr.O[1]) * fr.down),
+                                     __double2float_rn(((double)c.z - fr.O[2]) * fr.down));
                 }
                 bool reach = false;
 #pragma unroll
@@ -717,8 +721,8 @@ __global__ void k_knn(KnnParams p)
 // a 4-ary max-heap once it is ordered, up to kWPend further ones waiting behind.
 //
 // The mixed form's keys are the canonical distances and kk = N_ngb.  The FP64
-// form searches with FP32 offsets too (S4: offset to the leaf's cell corner, w =
-// a bound of the offset's error) and keeps kk = N_ngb + kWExtra keys with their
+// form searches with FP32 offsets too (S4: offset to the leaf's cell corner, in
+// units of 2^HaloFrame::E, w = a bound of the offset's error) and keeps kk = N_ngb + kWExtra keys with their
 // slots; distances in FP64 are formed only for the candidates whose FP32 distance
 // lies so near the N_ngb-th that rounding could change their order (one or two).
 //
@@ -839,7 +843,7 @@ __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p,
         if (active) {
             if constexpr (MODE == kMoments) rad = (float)hp;
             else if constexpr (kF32) rad = __fmul_ru((float)hp, p.slack);
-            else rad = __double2float_ru(__dmul_ru((double)hp, (double)p.slack));
+            else rad = __double2float_ru(__dmul_ru((double)hp * p.frame[h].down, (double)p.slack));
         }
         uint32_t todo = bad ? 0u : __ballot_sync(FULL, active);
         while (todo) {
@@ -1438,8 +1442,8 @@ constexpr float kGuessWide = 1.0f;
 template <class R>
 __global__ void __launch_bounds__(256) k_knn_guess(int L, const int32_t* __restrict__ leaf_halo, const int32_t* __restrict__ leaf_off,
                                                    const int64_t* __restrict__ halo_off, const int32_t* __restrict__ ngb,
-                                                   const float4* __restrict__ S4, const float4* __restrict__ cell,
-                                                   typename Vec4<R>::T* __restrict__ P4)
+                                                   const HaloFrame* __restrict__ frame, const float4* __restrict__ S4,
+                                                   const float4* __restrict__ cell, typename Vec4<R>::T* __restrict__ P4)
 {
     constexpr unsigned FULL = 0xffffffffu;
     __shared__ float4 window[8][(2 * kGuessSpan + 1) * kLeaf];
@@ -1520,7 +1524,7 @@ __global__ void __launch_bounds__(256) k_knn_guess(int L, const int32_t* __restr
         }
         if (more) g = sqrtf(high) * 1.001f;
     }
-    if (lane < n) P4[(int64_t)leaf * kLeaf + lane].w = (R)g;
+    if (lane < n) P4[(int64_t)leaf * kLeaf + lane].w = sizeof(R) == 8 ? (R)((double)g * frame[h].up) : (R)g;
 }
 
 template <class R>
@@ -1529,7 +1533,7 @@ int launch_guess(sidm_ctx* c, cudaStream_t s)
     using V = typename Vec4<R>::T;
     const float4* S4 = c->cfg.precision == SIDM_FP64 ? c->d_S4 : (const float4*)c->d_P4;
     k_knn_guess<R><<<(unsigned)(((int64_t)c->lay.L * 32 + 255) / 256), 256, 0, s>>>(c->lay.L, c->d_leaf_halo, c->d_leaf_off, c->d_halo_off,
-                                                                                  c->d_ngb, S4, c->d_cell, (V*)c->d_P4);
+                                                                                  c->d_ngb, c->d_frame, S4, c->d_cell, (V*)c->d_P4);
     c->launches++;
     return cuda_check(c, cudaGetLastError(), "knn guess launch");
 }

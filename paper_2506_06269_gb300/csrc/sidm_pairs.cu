@@ -98,10 +98,11 @@ __device__ __forceinline__ bool step_opens(int b, int n_bins, int s)
     return (s & ((1 << (n_bins - 1 - b)) - 1)) == 0;
 }
 
+// a length in the halo's FP32 unit, rounded up
 template <class R>
-__device__ __forceinline__ float to_float_ru_p(R v)
+__device__ __forceinline__ float to_float_ru_p(R v, double down)
 {
-    if constexpr (sizeof(R) == 8) return __double2float_ru((double)v);
+    if constexpr (sizeof(R) == 8) return __double2float_ru((double)v * down);
     else return (float)v;
 }
 
@@ -377,10 +378,11 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_pairs_all(PairP
             if constexpr (sizeof(R) == 4) {
                 pc = make_float3(__fadd_rn(cA.x, c.x), __fadd_rn(cA.y, c.y), __fadd_rn(cA.z, c.z));
             } else {
-                pc = make_float3(__double2float_rn((double)c.x - fr.O[0]), __double2float_rn((double)c.y - fr.O[1]),
-                                 __double2float_rn((double)c.z - fr.O[2]));
+                pc = make_float3(__double2float_rn(((double)c.x - fr.O[0]) * fr.down),
+                                 __double2float_rn(((double)c.y - fr.O[1]) * fr.down),
+                                 __double2float_rn(((double)c.z - fr.O[2]) * fr.down));
             }
-            const float rc = __fadd_ru(__fmul_ru(__fadd_ru(to_float_ru_p<R>(c.w), hmaxA), 1.0f + 0x1p-20f), fr.margin);
+            const float rc = __fadd_ru(__fmul_ru(__fadd_ru(to_float_ru_p<R>(c.w, fr.down), hmaxA), 1.0f + 0x1p-20f), fr.margin);
             const uint32_t cmask = __ballot_sync(
                 0xffffffffu, lane < countB && point_gap2_rd(pc, qlo, qhi) <= __fmul_ru(rc, rc) &&
                                  (!p.bins || step_opens(p.bins[hb + (int64_t)Bl * kLeaf + lane], p.n_bins, p.substep)));
@@ -452,10 +454,11 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_pairs_all(PairP
         if constexpr (sizeof(R) == 4) {
             pq = make_float3(__fadd_rn(cA.x, (float)q.x), __fadd_rn(cA.y, (float)q.y), __fadd_rn(cA.z, (float)q.z));
         } else {
-            pq = make_float3(__double2float_rn((double)q.x - fr.O[0]), __double2float_rn((double)q.y - fr.O[1]),
-                             __double2float_rn((double)q.z - fr.O[2]));
+            pq = make_float3(__double2float_rn(((double)q.x - fr.O[0]) * fr.down),
+                             __double2float_rn(((double)q.y - fr.O[1]) * fr.down),
+                             __double2float_rn(((double)q.z - fr.O[2]) * fr.down));
         }
-        const float hq = active ? to_float_ru_p<R>(q.w) : -INFINITY;
+        const float hq = active ? to_float_ru_p<R>(q.w, fr.down) : -INFINITY;
         // this lane's query reaches box c: within (h_i + hmax_node)(1 + 2^-20) + margin
         auto near_box = [&](int c) -> bool {
             const float4 lo = blo[c], hi = bhi[c];
@@ -599,7 +602,8 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_pairs_all(PairP
 //  * one warp scan of the masks' bit counts per batch gives every lane its place
 //    in the warp's queue of (query lane, candidate) pairs, which is emptied 32
 //    pairs at a time, all lanes busy.
-// The FP64 form runs the same search on FP32 offsets (S4) with a reach w = h and
+// The FP64 form runs the same search on FP32 offsets (S4, in units of
+// 2^HaloFrame::E) with a reach w = h and
 // the rounding errors' bound (k_leaf_hmax), where a pair is out of range, in range
 // for certain, or (about 1 in 10^3) settled by its FP64 distance before its draw;
 // only pairs whose draw can fire take FP64 arithmetic.  2^20 NFW halo: 2.8 ms
