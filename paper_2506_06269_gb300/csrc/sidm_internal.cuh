@@ -48,7 +48,7 @@ struct DevCounters {
     unsigned long long ev_count;     // events drawn this step
     unsigned long long de_lo;        // 128-bit fixed-point sum of pair dE (2^-80 units)
     unsigned long long de_hi;
-    unsigned int vmax[kMaxHalos];    // bits of the largest speed per halo (FP32, >= 0; halos of constant cross-section)
+    unsigned long long vmax2[kMaxHalos];   // bits of the largest squared speed per halo (FP64, >= 0; halos of constant cross-section)
     unsigned int work[4];            // persistent work-queue counters; [2], [3]: grid barrier
     unsigned int status;             // sticky SIDM_DEV_* bits (cleared by sidm_status)
     unsigned int pad;

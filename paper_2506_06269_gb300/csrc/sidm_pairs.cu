@@ -640,6 +640,14 @@ constexpr uint32_t kUnsure = 0x80000000u;   // on a candidate's id (below 2^27):
 // max over v of sigma(v) v / s0 for kind 1: v / (1 + (v/w)^2)^2 peaks at v = w / sqrt(3)
 constexpr float kSvMax = 0.32475953f;    // 3 sqrt(3) / 16, rounded up
 
+// speed from its square, to a few FP32 units in the last place, with room for what
+// squares below the form's normal numbers lose
+__device__ __forceinline__ double speed_of(float v2) { return (double)(sqrtf(v2) + 4e-19f); }
+__device__ __forceinline__ double speed_of(double v2)
+{
+    return (v2 > 1e-30 && v2 < 1e30 ? (double)sqrtf((float)v2) : sqrt(v2)) + 4e-154;
+}
+
 template <class R, int PR, bool DRAG>
 __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
 {
@@ -708,30 +716,40 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
         uint32_t thr = FULL;
         {
             const sidm_xs xs = p.xs[h];
-            float sv;
+            // Lengths, speeds and cross-sections may lie anywhere in the form's range, so
+            // the factors meet in FP64 (a few operations per leaf); what the mixed form's
+            // FP32 products of P can gain by rounding below the normal numbers is added
+            double sv;
             if (xs.kind == 1) {
-                sv = kSvMax * fabsf((float)xs.w);
+                sv = (double)kSvMax * fabs((double)(R)xs.w);
             } else {
-                float vi = 0.f;
+                R vi2 = R(0);
                 if (active) {
                     const R* vel = (const R*)p.vel;
                     const int64_t uA = index_of(slotA);
-                    const float vx = (float)vel[uA], vy = (float)vel[p.N + uA], vz = (float)vel[2 * p.N + uA];
-                    vi = sqrtf(vx * vx + vy * vy + vz * vz);
+                    const R vx = vel[uA], vy = vel[p.N + uA], vz = vel[2 * p.N + uA];
+                    vi2 = vx * vx + vy * vy + vz * vz;
                 }
-                sv = vi + __uint_as_float(p.cnt->vmax[h]);
+                sv = speed_of(vi2) + speed_of((R)__longlong_as_double((long long)p.cnt->vmax2[h]));
             }
-            double dtl;
+            R X = (R)xs.s0 * (R)p.mass[h] * (p.bins ? (R)p.dt_max : (R)p.dt[h]);
             if (p.bins) {                                     // the longest step that opens now
                 const int tz = p.substep ? __ffs(p.substep) - 1 : 31;
-                dtl = ldexp(p.dt_max, -max(0, p.n_bins - 1 - tz));
-            } else {
-                dtl = p.dt[h];
+                X *= (R)__int_as_float((127 - max(0, p.n_bins - 1 - tz)) << 23);
             }
-            const float inv = 1.f / (kF32 ? q.w : (1.0f - 0x1p-20f) * (float)P4[slotA].w);
-            const float b = (float)(xs.s0 * p.mass[h] * dtl) * sv * (kLamFUp * inv * inv * inv) * 1.001f + 3e-6f;
+            double b;
+            if constexpr (kF32) {
+                const float inv = 1.f / q.w;
+                b = (double)X * sv * (1.001 * kLamFUp * ((double)inv * inv * inv) + 0x1p-146);
+                if (X > 0.f && X < 0x1p-100f) b = 1.0;
+            } else {
+                const double down = p.frame[h].down;
+                const float inv = 1.f / ((1.0f - 0x1p-20f) * (float)((double)P4[slotA].w * down));
+                b = (double)X * down * down * down * sv * (1.001 * kLamFUp * ((double)inv * inv * inv));
+            }
+            const float bf = __double2float_ru(b + 3e-6);
             uint32_t t = FULL;
-            if (b < 1.f) t = (uint32_t)(fmaxf(b, 3e-6f) * 4294967296.f) + 1u;
+            if (bf < 1.f) t = (uint32_t)(fmaxf(bf, 3e-6f) * 4294967296.f) + 1u;
             thr = __reduce_max_sync(FULL, active ? t : 0u);
             if (drag) thr = FULL;
         }
@@ -1178,9 +1196,9 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
     }
 }
 
-// Largest speed of every halo whose cross-section does not depend on the speed
-// (kind 0), for the bound of P: kSplit CTAs per reduction chunk, one atomic each.
-// A NaN speed drops out of the maximum: its pairs have P = NaN and never fire.
+// Largest squared speed of every halo whose cross-section does not depend on the
+// speed (kind 0), for the bound of P: kSplit CTAs per reduction chunk, one atomic
+// each.  A NaN drops out of the maximum: its pairs have P = NaN and never fire.
 constexpr int kVmaxSplit = 4, kVmaxChunk = 16384;
 template <class R>
 __global__ void __launch_bounds__(256) k_vmax(const R* __restrict__ vel, int64_t N, const int32_t* __restrict__ chunk_halo,
@@ -1192,14 +1210,15 @@ __global__ void __launch_bounds__(256) k_vmax(const R* __restrict__ vel, int64_t
     if (xs[h].kind == 1) return;
     const int64_t b = chunk_begin[c] + (int64_t)part * (kVmaxChunk / kVmaxSplit);
     const int64_t e = min(min(chunk_begin[c] + kVmaxChunk, halo_off[h + 1]), b + kVmaxChunk / kVmaxSplit);
-    float m = 0.f;
+    R m = R(0);
 #pragma unroll 4
     for (int64_t s = b + threadIdx.x; s < e; s += blockDim.x) {
-        const float x = (float)vel[s], y = (float)vel[N + s], z = (float)vel[2 * N + s];
-        m = fmaxf(m, x * x + y * y + z * z);
+        const R x = vel[s], y = vel[N + s], z = vel[2 * N + s];
+        const R v2 = x * x + y * y + z * z;
+        m = v2 > m ? v2 : m;
     }
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0 && m > 0.f) atomicMax(&cnt->vmax[h], __float_as_uint(sqrtf(m)));
+    for (int o = 16; o > 0; o >>= 1) { const R y = __shfl_xor_sync(0xffffffffu, m, o); m = y > m ? y : m; }
+    if ((threadIdx.x & 31) == 0 && m > R(0)) atomicMax(&cnt->vmax2[h], (unsigned long long)__double_as_longlong((double)m));
 }
 
 void fill_params(sidm_ctx* c, PairParams& p, uint64_t seed, uint64_t step, const sidm_xs* xs, const double* dt,
