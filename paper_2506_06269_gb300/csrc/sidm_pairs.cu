@@ -1023,7 +1023,11 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
                     const float r = (c[u].w + fw.w) * (1.0f + 0x1p-18f);
                     const bool keep = open[u] && gx * gx + gy * gy + gz * gz <= r * r;
                     const uint32_t m = __ballot_sync(FULL, keep);
-                    if (u == 0 && Bl[0] == A) { nself = __popc(m); rank = __popc(m & lt); }   // A is the first of its walk
+                    if (u == 0 && Bl[0] == A) {                           // A is the first of its walk
+                        nself = __popc(m);
+                        rank = __popc(m & lt);
+                        n_tested -= __reduce_add_sync(FULL, act ? (unsigned)rank + 1u : 0u);   // each of its pairs once
+                    }
                     if (keep) {
                         const uint32_t e = cnum + navail + __popc(m & lt);
                         float* at = ring + (e & (kPRing - 1));
@@ -1033,7 +1037,7 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
                         ca[kPCand] = (uint32_t)(leaf0 + Bl[u]) * kLeaf + lane;
                     }
                     navail += __popc(m);
-                    n_tested += (uint32_t)(n_act * __popc(m));       // an upper bound inside the query leaf
+                    n_tested += (uint32_t)(n_act * __popc(m));
                 }
                 n_tiles += min(2, nl - li);
                 li += 2;
