@@ -63,8 +63,10 @@ extern "C" {
 #define SIDM_FLAG_TIMING  0x2  /* time hot kernels with CUDA events (sidm_kernel_times) */
 #define SIDM_FLAG_LOCAL_DIAG 0x4 /* keep scratch for sidm_local_diagnostics (40 B/particle) */
 #define SIDM_FLAG_DRAG    0x8  /* keep scratch for forward-dominated halos (sidm_xs.angular = 1):
-                                  per-particle interaction lists, 64 B per event_cap, and
-                                  40 (FP64: 72) more up to 1024 particles per SM */
+                                  per-particle interaction lists, 64 B per event_cap; with
+                                  n_max up to 1024 particles per SM and 40 B (FP64: 72) more
+                                  per event_cap to be had, rounds with a thread per particle
+                                  (fixed at creation; the results are the same) */
 
 typedef struct sidm_ctx sidm_ctx;
 

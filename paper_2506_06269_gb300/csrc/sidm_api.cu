@@ -1702,9 +1702,16 @@ extern "C" int sidm_create(sidm_ctx** out, const sidm_config* cfg)
         ALLOC(c->d_lact, 2 * N);
         ALLOC(c->d_lcnt, 8);
         if (cdiv(N, kRoundThreads) <= c->sm_count) {                // rounds with a thread per particle
-            e = cudaMalloc(&c->d_lent, (size_t)m * 4 * rs); if (e != cudaSuccess) return fail("cudaMalloc lent", e);
-            ALLOC(c->d_lpart, m);
-            e = cudaMalloc(&c->d_lpub, (size_t)3 * N * 4 * rs); if (e != cudaSuccess) return fail("cudaMalloc lpub", e);
+            e = cudaMalloc(&c->d_lent, (size_t)m * 4 * rs);
+            if (e == cudaSuccess) e = dev_alloc(&c->d_lpart, (size_t)m);
+            if (e == cudaSuccess) e = cudaMalloc(&c->d_lpub, (size_t)3 * N * 4 * rs);
+            if (e == cudaErrorMemoryAllocation) {                   // the rounds over lists need none of the three
+                cudaGetLastError();
+                cudaFree(c->d_lent); cudaFree(c->d_lpart); cudaFree(c->d_lpub);
+                c->d_lent = nullptr; c->d_lpart = nullptr; c->d_lpub = nullptr;
+            } else if (e != cudaSuccess) {
+                return fail("cudaMalloc lent", e);
+            }
         }
     }
 #undef ALLOC
