@@ -8,12 +8,13 @@ leaf size that defines the canonical FP32 distance is not a knob):
                                  the candidate mask), knn_chains (independent
                                  distance chains), knn_batch (loop per staged leaf,
                                  over compacted batches, or those plus the
-                                 fixed-bound warm-start kernel), knn_flush (merge
+                                 fixed-bound kernel), knn_flush (merge
                                  threshold before node tests), knn_slack
                                  (warm-start bound)
-  pair kernel (k_pairs)          pair_warps, pair_per_round (pairs a lane queues
-                                 per round)
-  candidate staging              use_tma (plain loads or bulk async copies)
+  pair kernel (k_pairs)          pair_warps, pair_per_round (groups of 32 pairs
+                                 drawn together)
+  candidate staging              use_tma (plain loads, or bulk async copies in the
+                                 per-lane kernel-size search)
 
 The search is coordinate descent from the defaults: one knob at a time over
 its values, keeping the fastest, two sweeps.  A trial builds a context with the
@@ -36,10 +37,10 @@ KNN_KNOBS = {
 }
 PAIR_KNOBS = {
     "pair_warps": (4, 8),
-    "pair_per_round": (3, 4),
+    "pair_per_round": (1, 2, 3),
 }
 DEFAULTS = {"knn_warps": 8, "knn_batch": 3, "knn_groups": 2, "knn_chains": 4, "knn_flush": 32, "knn_slack": 1.07,
-            "pair_warps": 8, "pair_per_round": 4, "use_tma": 0}
+            "pair_warps": 8, "pair_per_round": 2, "use_tma": 0}
 
 
 def _trial(make_inputs, ks, xs_list, dts, masses, halo_off, precision, kw, reps, settle=2):
