@@ -53,10 +53,12 @@ struct KnnParams {
     unsigned int* work;          // persistent work counter (zeroed before the launch)
     const int32_t* leaf_list;    // NULL: every leaf; else the leaves listed here ...
     const unsigned int* list_len;  // ... of which there are *list_len
+    int32_t* long_list;          // k_knn_warm without teams: where leaves of more than tiles_max candidate leaves go
+    unsigned tiles_max;
+    unsigned int* long_len;
     void* hprev;        // out: h per particle (next call's guess), NULL for neighbour lists
     int use_guess;      // P4.w holds each particle's previous kernel size
     float slack;        // guess bound = previous h * slack
-    float grow;         // factor of the bound between attempts
     const void* V4;     // moments: velocities, particle mass, sums [5][nacc]
     const double* mass;
     double* dacc;
@@ -728,11 +730,14 @@ __global__ void k_knn(KnnParams p)
 //
 // A lane that admits fewer than N_ngb keys (its guess was too small) tries again
 // with a wider bound.  A leaf goes to a list that the per-lane search (k_knn,
-// warm-started, failing lanes cold) then redoes when its particles have no
-// previous kernel size, when kWAttempts bounds did not do, when the tree walk's
-// stack overflows, or when the FP32 order of the FP64 form does not settle it
-// (more than kWBand candidates within the error, or one that was not kept); so
-// the result is the same exact k-th distance as a cold search.
+// warm-started after a warm start, failing lanes cold) then redoes when its
+// particles have no previous kernel size, when they would take more than kWRuns
+// runs, when kWAttempts bounds did not do, when the tree walk's stack overflows, or
+// when the FP32 order of the FP64 form does not settle it (more than kWBand
+// candidates within the error, or one that was not kept); so the result is the same
+// exact k-th distance as a cold search.  A leaf that has streamed tiles_max candidate
+// leaves (an outlier whose kernel reaches the centre: thousands, on one warp, while
+// the SMs idle) is started anew by a team, in a launch of its own.
 //
 // Issue-bound and, with 10 to 15 warps per SM (their keys fill the shared memory),
 // latency-bound.  Per search, this launch and the redo's together: 2^20 NFW halo,
@@ -741,11 +746,12 @@ __global__ void k_knn(KnnParams p)
 // 0.37 ms); FP64 form 2.2 ms (11.6 ms with every distance in FP64).  Eight halos of
 // 1500 to 30000 particles, N_ngb up to 128: 0.50 ms (0.98); 2048 particles 40 us
 // (84), teams; FP64 16384 particles 0.22 ms (4.4).  kWSpread 2, 2.5, 3, 4: 1.15,
-// 1.11, 1.12, 1.20 ms at 2^20 and 0.47, 0.58, 0.60, 0.64 ms for the eight halos;
-// A first search, 300,007 NFW particles, N_ngb = 48: 0.85 ms with the guess
-// against 2.5 ms in the per-lane kernel (whose heaps fill from the Morton window,
-// 20 of 32 lanes active); 100,003 Hernquist particles 1.2 against 1.5 ms (its
-// longest leaf).  Neighbour lists there 0.45 ms (1.87 in the per-lane kernel);
+// 1.11, 1.12, 1.20 ms at 2^20 and 0.47, 0.58, 0.60, 0.64 ms for the eight halos.
+// A first search, 300,007 NFW particles, N_ngb = 48: 0.62 ms with the guess
+// (0.78 before long leaves went to teams) against 2.5 ms in the per-lane kernel
+// (whose heaps fill from the Morton window, 20 of 32 lanes active); 100,003
+// Hernquist particles with their lists 1.36 ms (1.55).  Neighbour lists there
+// 0.45 ms (1.87 in the per-lane kernel);
 // moments of the 300,007 particles 0.57 ms (1.74 ms over in-range pairs, with ten
 // FP64 atomics each).
 // Boxes of four lane groups in wide runs: 1.36 ms; runs of a leaf dealt out to the
@@ -760,7 +766,19 @@ constexpr int kWBand = 4;       // FP64 form: candidates compared in FP64
 static_assert((kWRing & (kWRing - 1)) == 0 && kWRing >= kWBatch - 1 + 2 * kLeaf, "the ring holds a batch's leftover plus two leaves");
 static_assert(kWPend >= kWBatch, "one batch fits after a merge");
 constexpr int kWarmMaxWarps = 8;   // the kernel's launch bound: 256 threads, two CTAs per SM
-constexpr int kWAttempts = 10;     // bounds tried, each KnnParams::grow times the one before, before the redo
+constexpr int kWAttempts = 8;      // bounds tried, each 1.1 to 3 times the one before, before the redo
+// Runs of a leaf at most; a leaf of more goes to the redo.  Leaves of NFW and Hernquist
+// halos take three at most with sizes near theirs; with guesses ten times too small
+// each lane is a run: 100,000 Hernquist particles 2.76 ms with runs and attempts
+// without limit, 0.95 through the redo.  4 instead of 8: 45.3 against 44.1 ms for the
+// 64-halo batch, whose halos of few, far particles have leaves of five.
+constexpr int kWRuns = 8;
+// Candidate leaves one warp streams for a leaf; one that wants more goes to a team.
+// 200,003 Hernquist particles, N_ngb = 128: 3.64 ms with one warp throughout, 1.43
+// with 512, but the eight halos above 0.58 ms with 512 against 0.54 with 1024.  A first
+// search has more of them: neighbours of the 100,003 particles 1.28, 1.36, 1.62,
+// 1.97 ms with 192, 384, 768, 1024, first sizes of the 300,007 0.74, 0.62, 0.62, 0.62.
+constexpr unsigned kWTiles = 1024, kWTilesGuess = 384;   // (from a density guess)
 // widest box of a run of queries / its largest bound: a run costs a walk, a wide
 // box reaches dense regions that none of its queries does; a team shares both
 constexpr float kWSpread = 2.25f, kWSpreadTeam = 3.0f;
@@ -792,6 +810,7 @@ __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p,
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int team_leaf;
     __shared__ unsigned int team_bad, team_stop, team_fail, team_err;
+    __shared__ float team_rad[32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int nw = TEAM ? (int)(blockDim.x >> 5) : 1, part = TEAM ? wid : 0;   // nw: a power of two
     const size_t warp_bytes = warm_warp_bytes<R, MODE>(p.kcap);
@@ -814,7 +833,12 @@ __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p,
         int leaf = 0;
         if constexpr (TEAM) {
             __syncthreads();
-            if (threadIdx.x == 0) { team_leaf = (int)atomicAdd(p.work, 1u); team_bad = team_fail = team_err = 0u; }
+            if (threadIdx.x == 0) {
+                int next = (int)atomicAdd(p.work, 1u);
+                if (p.leaf_list) next = (unsigned)next < *p.list_len ? p.leaf_list[next] : p.L;
+                team_leaf = next;
+                team_bad = team_fail = team_err = 0u;
+            }
             __syncthreads();
             leaf = team_leaf;
         } else {
@@ -835,7 +859,7 @@ __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p,
         const unsigned long long tiles0 = n_tiles;
         // a particle without a previous kernel size sends its leaf to the redo
         // (moments: a particle without an extent has no neighbours inside it)
-        bool bad = MODE != kMoments && __any_sync(FULL, active && !(hp > R(0)));
+        bool bad = MODE != kMoments && __any_sync(FULL, active && !(hp > R(0))), too_long = false;
         const float margin = p.frame[h].margin;
         const float4 cA = p.cell[leaf];
         // the lane's bound: slack h_prev rounded up
@@ -846,9 +870,8 @@ __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p,
             else rad = __double2float_ru(__dmul_ru((double)hp * p.frame[h].down, (double)p.slack));
         }
         uint32_t todo = bad ? 0u : __ballot_sync(FULL, active);
-        while (todo) {
-        bool act = (todo >> lane) & 1u;
         const float px = __fadd_rn(cA.x, q.x), py = __fadd_rn(cA.y, q.y), pz = __fadd_rn(cA.z, q.z);
+        bool act = false;
         float w[7];
         auto box = [&]() {                                   // of the act lanes: lo, -hi, -largest bound
             w[0] = act ? px : INFINITY;  w[1] = act ? py : INFINITY;  w[2] = act ? pz : INFINITY;
@@ -865,9 +888,12 @@ __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p,
         auto wide = [&]() {
             return fmaxf(fmaxf(-w[3] - w[0], -w[4] - w[1]), -w[5] - w[2]) > (TEAM ? kWSpreadTeam : kWSpread) * -w[6];
         };
-        box();
-        widest();
-        if (wide()) {                                        // the same in every lane
+        // act: the next run of the lanes left
+        auto next_run = [&](uint32_t left) {
+            act = (left >> lane) & 1u;
+            box();
+            widest();
+            if (!wide()) return;                             // the same in every lane
             // boxes of the lanes up to this one: the run ends before the first that is too wide
             box();
             for (int o = 1; o < 32; o <<= 1) {
@@ -879,9 +905,29 @@ __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p,
             }
             const uint32_t over = __ballot_sync(FULL, act && wide());
             if (over) act = act && lane < __ffs(over) - 1;
+        };
+        // a leaf no wider than two of the cells that order it is taken whole (in a core
+        // denser than the cells, leaves lie on one another, and each run would load them
+        // all), another of more than kWRuns runs goes to the redo, which takes all its
+        // lanes through one walk
+        act = (todo >> lane) & 1u;
+        box();
+        widest();
+        bool whole = !wide() || fmaxf(fmaxf(-w[3] - w[0], -w[4] - w[1]), -w[5] - w[2]) <= 2.f * p.frame[h].fine;
+        if (!whole && MODE != kMoments) {
+            uint32_t left = todo;
+            for (int r = 0; r < kWRuns && left; ++r) {
+                next_run(left);
+                left &= ~__ballot_sync(FULL, act);
+            }
+            if (left) { bad = true; todo = 0u; }
         }
+        while (todo) {
+        if (whole) act = (todo >> lane) & 1u;
+        else next_run(todo);
         todo &= ~__ballot_sync(FULL, act);
         // a lane that admits fewer than N_ngb keys tries again with a wider bound
+        int found = 0;                                 // keys of the last attempt
         for (int attempt = 0;; ++attempt) {
         uint32_t root = act ? __float_as_uint(MODE == kMoments ? __fmul_rn(rad, rad) : __fmul_ru(rad, rad)) : 0u;   // bits of the lane's d^2 bound
         float err = 0.f;                               // FP64 form: largest offset error of a candidate
@@ -1066,6 +1112,7 @@ __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p,
                 __syncwarp();
             } else if (!started || sp > 0) {
                 // walk until the list may not hold another node's leaves, or the tree is done
+                if (!TEAM && (unsigned)(n_tiles - tiles0) > p.tiles_max) { bad = too_long = true; break; }
                 nl = li = 0;
                 if (!started) {
                     const int nb = p.lvl_off[top * Hp + h];
@@ -1126,6 +1173,7 @@ __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p,
             }
             if (fin) break;
         }
+        if (too_long) break;
         if constexpr (MODE == kMoments) {
             // the warps' moments, added in order by the first
             gather();
@@ -1233,6 +1281,11 @@ __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p,
                 }
             }
             fail = __ballot_sync(FULL, again);
+            // the next bound: what holds N_ngb and two standard deviations of its Poisson
+            // count at the density that the keys found suggest
+            // (three times as far where the last step found nothing more)
+            if (again) rad *= attempt > 0 && n == found ? 3.f : fminf(fmaxf(cbrtf(((float)k + 2.f * sqrtf((float)k) + 1.f) / ((float)n + 1.f)), 1.1f), 3.f);
+            found = n;
             if (__any_sync(FULL, !ok && !again) || (fail && attempt == kWAttempts - 1)) bad = true;
             if (act && ok) {
                 const int64_t u = p.halo_off[h] + (int64_t)slotA - (int64_t)leaf0 * kLeaf;
@@ -1264,18 +1317,24 @@ __global__ void __launch_bounds__(kWarmMaxWarps * 32, 2) k_knn_warm(KnnParams p,
         if constexpr (TEAM) {
             // written between this attempt's two barriers only (team_bad may be set
             // again by a warp that has begun the next attempt)
-            if (wid == 0 && lane == 0) { team_fail = fail; team_stop = bad ? 1u : 0u; }
+            if (wid == 0) {
+                team_rad[lane] = rad;
+                if (lane == 0) { team_fail = fail; team_stop = bad ? 1u : 0u; }
+            }
             __syncthreads();
             fail = team_fail;
             bad = team_stop != 0u;
+            rad = team_rad[lane];
         }
         if (bad || fail == 0u) break;
         act = (fail >> lane) & 1u;
-        if (act) rad *= p.grow;
         }   // attempts
         if (bad) break;
         }   // runs of queries
-        if (MODE != kMoments && bad && part == 0 && lane == 0) { const unsigned r = atomicAdd(redo_len, 1u); redo_list[r] = leaf; }
+        if ((MODE != kMoments || too_long) && bad && part == 0 && lane == 0) {
+            const unsigned r = atomicAdd(too_long ? p.long_len : redo_len, 1u);
+            (too_long ? p.long_list : redo_list)[r] = leaf;
+        }
         n_tiles_max = n_tiles - tiles0 > n_tiles_max ? n_tiles - tiles0 : n_tiles_max;
         __syncwarp();
     }
@@ -1302,11 +1361,10 @@ void fill_params(sidm_ctx* c, KnnParams& p, void* h_out, uint32_t* nbr, int k_st
     p.S4 = c->cfg.precision == SIDM_FP64 ? (const void*)c->d_S4 : c->d_P4;
     p.h_out = h_out; p.nbr = nbr; p.k_stride = k_stride; p.kcap = c->kmax_cur; p.cnt = c->d_cnt;
     p.work = &c->d_cnt->work[0];
-    p.leaf_list = nullptr; p.list_len = nullptr;
+    p.leaf_list = nullptr; p.list_len = nullptr; p.long_list = nullptr; p.long_len = nullptr; p.tiles_max = ~0u;
     p.hprev = nbr ? nullptr : c->d_hprev;
     p.use_guess = use_guess ? 1 : 0;
     p.slack = c->cfg.knn_slack > 0.f ? c->cfg.knn_slack : kGuessSlackDefault;
-    p.grow = 1.5f;
     p.flush_node = c->cfg.knn_flush > 0 ? c->cfg.knn_flush : kFlushNodeDefault;
 }
 
@@ -1393,38 +1451,44 @@ int launch_warm(sidm_ctx* c, void* h_out, cudaStream_t s, uint32_t* nbr = nullpt
     KnnParams p;
     fill_params(c, p, h_out, nbr, k_stride, true);
     p.V4 = c->d_V4; p.mass = mass; p.dacc = c->d_dacc; p.nacc = c->lay.N;
-    if (guessed) { p.slack = 1.0f; p.grow = 2.0f; }   // a density guess (k_knn_guess)
+    if (guessed) p.slack = 1.0f;                   // a density guess (k_knn_guess)
     if (NBR) p.slack = 1.0f + 0x1p-20f;            // the kernel size itself is the bound
     const size_t per_warp = warm_warp_bytes<R, MODE>(p.kcap);
     int warps = 0, grid = 0;
     if (int rc = pick_shape(c, (const void*)k_knn_warm<R, false, MODE>, per_warp, &warps, &grid, kWarmMaxWarps)) return rc;
-    bool team = false;
-    if (c->lay.L < kTeamItems * grid * warps) {
-        int w = kWarmMaxWarps;
-        while (w > 1 && (w > c->knn_warps || (size_t)w * per_warp > (size_t)226 * 1024)) w /= 2;
-        int occ = 0;
-        if (int rc = occupancy(c, (const void*)k_knn_warm<R, true, MODE>, w * 32, (size_t)w * per_warp, &occ)) return rc;
-        if (occ >= 1 && w > 1) {
-            team = true;
-            warps = w;
-            grid = c->cfg.grid_ctas > 0 ? c->cfg.grid_ctas : c->sm_count * occ;
-            grid = std::max(1, std::min(grid, c->lay.L));
-        }
-    }
+    int tw = kWarmMaxWarps, occ = 0;                // a team's warps
+    while (tw > 1 && (tw > c->knn_warps || (size_t)tw * per_warp > (size_t)226 * 1024)) tw /= 2;
+    if (int rc = occupancy(c, (const void*)k_knn_warm<R, true, MODE>, tw * 32, (size_t)tw * per_warp, &occ)) return rc;
+    const bool can_team = occ >= 1 && tw > 1;
+    const int team_grid = std::max(1, std::min(c->cfg.grid_ctas > 0 ? c->cfg.grid_ctas : c->sm_count * occ, c->lay.L));
+    const bool team = can_team && c->lay.L < kTeamItems * grid * warps;
+    const unsigned tiles_max = guessed ? kWTilesGuess : kWTiles;
+    // a halo of few leaves has none that streams so many of them
+    const bool longs = can_team && !team && c->lay.L > (int)tiles_max;
+    if (team) { warps = tw; grid = team_grid; }
     c->knn_grid = grid;
     cudaError_t e = cudaMemsetAsync(&c->d_cnt->work[0], 0, sizeof(unsigned int), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(&c->d_cnt->knn_redo[0], 0, 2 * sizeof(unsigned int), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(&c->d_cnt->knn_redo[0], 0, 4 * sizeof(unsigned int), s);
     if (e != cudaSuccess) return cuda_check(c, e, "knn work reset");
     const int tidx = MODE == kMoments ? -1 : timer_begin(c, 1, s);
+    p.tiles_max = longs ? tiles_max : ~0u;
+    if (longs) { p.long_list = c->d_knn_long; p.long_len = &c->d_cnt->knn_redo[2]; }
     if (team) k_knn_warm<R, true, MODE><<<grid, warps * 32, (size_t)warps * per_warp, s>>>(p, c->d_knn_redo, &c->d_cnt->knn_redo[0]);
     else k_knn_warm<R, false, MODE><<<grid, warps * 32, (size_t)warps * per_warp, s>>>(p, c->d_knn_redo, &c->d_cnt->knn_redo[0]);
-    timer_end(c, tidx, s);
     c->launches++;
+    if (longs) {
+        p.leaf_list = c->d_knn_long;
+        p.list_len = &c->d_cnt->knn_redo[2];
+        p.work = &c->d_cnt->knn_redo[3];
+        k_knn_warm<R, true, MODE><<<team_grid, tw * 32, (size_t)tw * per_warp, s>>>(p, c->d_knn_redo, &c->d_cnt->knn_redo[0]);
+        c->launches++;
+    }
+    timer_end(c, tidx, s);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_check(c, e, "knn launch");
     if constexpr (MODE == kMoments) return SIDM_OK;
     else if constexpr (NBR) return launch_t<float, true, false, kGroupsDefault, kChainsDefault>(c, nullptr, nbr, k_stride, false, s, true);
-    else return launch_tuned<R>(c, h_out, true, s, true);
+    else return launch_tuned<R>(c, h_out, !guessed, s, true);
 }
 
 // A guess for every particle of a search that has no earlier kernel sizes, into
@@ -1436,9 +1500,13 @@ int launch_warm(sidm_ctx* c, void* h_out, cudaStream_t s, uint32_t* nbr = nullpt
 // leaf; a wrong guess costs time, never accuracy.
 // A guess that holds more than N_ngb particles of the kGuessSpan leaves on either
 // side in Morton order is lowered to the radius that holds N_ngb of them: on the
-// sparse shell even the quartile can reach across the halo.
+// sparse shell even the quartile can reach across the halo.  In a leaf wider than
+// kGuessMixed times the quartile's guess (dense and sparse particles side by side,
+// where the quartile is far too small for some) every particle takes that radius, which
+// cannot fail: first sizes of 2003 Hernquist particles, N_ngb = 128, 0.56 ms (0.93).
 constexpr int kGuessRank = 10, kGuessNear = 4, kGuessSpan = 4;
 constexpr float kGuessWide = 1.0f;
+constexpr float kGuessMixed = 9.0f;   // about four runs of kWSpread
 template <class R>
 __global__ void __launch_bounds__(256) k_knn_guess(int L, const int32_t* __restrict__ leaf_halo, const int32_t* __restrict__ leaf_off,
                                                    const int64_t* __restrict__ halo_off, const int32_t* __restrict__ ngb,
@@ -1480,6 +1548,14 @@ __global__ void __launch_bounds__(256) k_knn_guess(int L, const int32_t* __restr
     const float rf = radius2(far), rn = radius2(near);
     const float vf = rf * sqrtf(rf) / (float)far, vn = rn * sqrtf(rn) / (float)near;
     const float v = lane < n ? (vf > 6.f * vn ? 1.5f * vn : vf) : INFINITY;
+    float ext = 0.f;                                           // the leaf's width
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const float x = a == 0 ? q.x : a == 1 ? q.y : q.z;
+        float lo = lane < n ? x : INFINITY, up = lane < n ? x : -INFINITY;
+        for (int o = 16; o > 0; o >>= 1) { lo = fminf(lo, __shfl_xor_sync(FULL, lo, o)); up = fmaxf(up, __shfl_xor_sync(FULL, up, o)); }
+        ext = fmaxf(ext, up - lo);
+    }
     int rank = 0;
     for (int t = 0; t < kLeaf; ++t) {
         const float y = __shfl_sync(FULL, v, t);
@@ -1517,7 +1593,17 @@ __global__ void __launch_bounds__(256) k_knn_guess(int L, const int32_t* __restr
     const int want = ngb[h] + 1;                               // the particle itself among them
     float low = 0.f, high = g2;
     const bool more = lane < n && within(g2) > want;
-    if (__any_sync(FULL, more)) {
+    const float gq = cbrtf(wide * quart * (k + 2.f * sqrtf(k) + 1.f));
+    if (ext > kGuessMixed * gq) {                              // the same in every lane
+        // dense and sparse particles in one leaf: the radius that holds N_ngb of the window
+        uint32_t a = 0u, b = __float_as_uint(3.f * ext * ext);
+        while (within(__uint_as_float(b)) < want && b < 0x7f000000u) b += 0x1000000u;      // four times the square
+        for (int it = 0; it < 12; ++it) {
+            const uint32_t mid = a + (b - a) / 2u;
+            if (within(__uint_as_float(mid)) >= want) b = mid; else a = mid;
+        }
+        g = sqrtf(__uint_as_float(b)) * 1.001f;
+    } else if (__any_sync(FULL, more)) {
         for (int it = 0; it < 8; ++it) {
             const float mid = 0.5f * (low + high);
             if (within(mid) >= want) high = mid; else low = mid;
