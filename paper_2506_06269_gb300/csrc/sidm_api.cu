@@ -1566,7 +1566,7 @@ static int radix_sort(sidm_ctx* c, unsigned long long*& ka, uint32_t*& va, unsig
 
 static void free_all(sidm_ctx* c)
 {
-    void* ptrs[] = {c->d_halo_off, c->d_halo_pad, c->d_leaf_off, c->d_lvl_off, c->d_top, c->d_ngb, c->d_leaf_halo, c->d_knn_redo, c->d_knn_long,
+    void* ptrs[] = {c->d_halo_off, c->d_halo_pad, c->d_leaf_off, c->d_lvl_off, c->d_top, c->d_ngb, c->d_leaf_halo, c->d_knn_redo, c->d_knn_long, c->d_pair_rest,
                     c->d_chunk_halo, c->d_chunk_begin, c->d_frame, c->d_key, c->d_key2, c->d_val, c->d_val2,
                     c->d_sort_status, c->d_sort_hist, c->d_P4, c->d_S4, c->d_reach, c->d_V4, c->d_ID, c->d_cell, c->d_cellb, c->d_nlo, c->d_nhi, c->d_perm, c->d_tmp_pos,
                     c->d_tmp_vel, c->d_tmp_id, c->d_claim, c->d_hits, c->d_done, c->d_ev, c->d_sump,
@@ -1657,6 +1657,9 @@ extern "C" int sidm_create(sidm_ctx** out, const sidm_config* cfg)
     ALLOC(c->d_leaf_halo, Lmax);
     ALLOC(c->d_knn_redo, Lmax);
     ALLOC(c->d_knn_long, Lmax);
+    // one rest per item at most: a leaf each, or up to twice four items per resident warp
+    c->pair_rest_cap = (int)std::min<int64_t>(Lmax + 8 * 64 * (int64_t)c->sm_count, INT32_MAX);
+    ALLOC(c->d_pair_rest, c->pair_rest_cap);
     ALLOC(c->d_chunk_halo, c->chunk_cap);
     ALLOC(c->d_chunk_begin, c->chunk_cap);
     ALLOC(c->d_frame, H);

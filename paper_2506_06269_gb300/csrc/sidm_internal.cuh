@@ -49,6 +49,7 @@ struct DevCounters {
     unsigned long long de_lo;        // 128-bit fixed-point sum of pair dE (2^-80 units)
     unsigned long long de_hi;
     unsigned long long vmax2[kMaxHalos];   // bits of the largest squared speed per halo (FP64, >= 0; halos of constant cross-section)
+    unsigned int pair_rest[2];       // rests that the pair kernel's warps left; the work counter of their launch
     unsigned int work[4];            // persistent work-queue counters; [2], [3]: grid barrier
     unsigned int status;             // sticky SIDM_DEV_* bits (cleared by sidm_status)
     unsigned int pad;
@@ -141,6 +142,8 @@ struct sidm_ctx {
     unsigned long long* d_claim = nullptr;  // [N] resolve claims (all ones at rest)
     uint32_t* d_hits = nullptr;             // [N] events per particle (zero at rest)
     uint8_t* d_done = nullptr;              // [event_cap]
+    int4* d_pair_rest = nullptr;            // [pair_rest_cap] rests of the pair kernel's items
+    int pair_rest_cap = 0;
     sidm_event* d_ev = nullptr;             // [event_cap]
     float* d_sump = nullptr;                // [N] (SIDM_FLAG_SUM_P)
     double* d_dacc = nullptr;               // [5][N] kernel-weighted moments (SIDM_FLAG_LOCAL_DIAG)

@@ -51,6 +51,11 @@ struct PairParams {
     float* sump;
     int use_sump;
     int parts;          // warps that share a query leaf's candidate leaves (a power of two)
+    int parts_log;
+    // what a warp leaves after kPTiles candidate leaves, (leaf, part | run << 8, first
+    // candidate leaf, accepted leaves before it), and the second launch that takes it
+    int4* rest;
+    int rest_cap;       // 0: a warp leaves nothing
     double* dacc;       // local diagnostics: [5][nacc] kernel-weighted moments
     int64_t nacc;
     DevCounters* cnt;
@@ -595,17 +600,17 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_pairs_all(PairP
 //    test per child, a lane each); accepted leaves are listed and loaded two at
 //    a time;
 //  * a listed leaf's candidates are kept if they come within h_j + the largest
-//    h of the queries' box (tested in the query leaf's own frame, where the gap
-//    rounded down bounds the canonical distance from below) and go to a ring;
+//    h of the queries' box (tested in the query leaf's own frame, with room for
+//    the rounding of the gap) and go to a ring;
 //  * batches of kPBatch ring entries are tested against all 32 queries, two
 //    candidates per packed FP32 operation, into one bit mask per lane;
 //  * one warp scan of the masks' bit counts per batch gives every lane its place
 //    in the warp's queue of (query lane, candidate) pairs, which is emptied 32
 //    pairs at a time, all lanes busy.
 // The FP64 form runs the same search on FP32 offsets (S4, in units of
-// 2^HaloFrame::E) with a reach w = h and
-// the rounding errors' bound (k_leaf_hmax), where a pair is out of range, in range
-// for certain, or (about 1 in 10^3) settled by its FP64 distance before its draw;
+// 2^HaloFrame::E) with a reach w = h and the rounding errors' bound (k_leaf_hmax),
+// where a pair is out of range, in range for certain, or (about 1 in 10^3) settled
+// by its FP64 distance before its draw;
 // only pairs whose draw can fire take FP64 arithmetic.  2^20 NFW halo: 2.8 ms
 // per launch against 39 ms with every test and P on the FP64 pipe, 16384
 // particles 0.13 against 1.30 ms.
@@ -625,6 +630,13 @@ constexpr int kPCand = 256;     // candidates whose ids and slots are kept for q
 constexpr int kPQueue = 32 * (kPBatch + kPerRoundMax);   // queued pairs: a batch behind less than one draw's
 constexpr int kPList = 64;      // accepted leaves listed before they are streamed
 constexpr float kPSpread = 3.0f;   // widest box of a run of queries / its largest h
+// Candidate leaves after which a warp leaves the rest of its item to a second launch,
+// whose warps share it: the kernel of an outlier reaches the centre, and one warp would
+// test the whole halo while the SMs idle.  Hernquist halos, N_ngb = 128: 200,000
+// particles 1.39 ms (2.08 without; 1.87 with 1024), 400,000 1.92 (5.66; 2.05).  256
+// leaves rests to ordinary warps of the 64-halo batch (72 against 50 ms).
+constexpr uint32_t kPTiles = 512;
+constexpr int kPRest = 32;         // warps that share such a rest at most (a power of two)
 static_assert((kPRing & (kPRing - 1)) == 0 && kPRing >= kPBatch - 1 + 2 * kLeaf, "the ring holds a batch's leftover plus two leaves");
 static_assert(kPCand == 256, "a queued pair is (query lane << 8 | candidate mod 256)");
 
@@ -648,7 +660,8 @@ __device__ __forceinline__ double speed_of(double v2)
     return (v2 > 1e-30 && v2 < 1e30 ? (double)sqrtf((float)v2) : sqrt(v2)) + 4e-154;
 }
 
-template <class R, int PR, bool DRAG>
+// REST: the launch that takes up the rests that the warps of the first one left
+template <class R, int PR, bool DRAG, bool REST>
 __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
 {
     static_assert(PR >= 1 && PR <= kPerRoundMax, "32-pair groups drawn together");
@@ -674,15 +687,26 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
     const V* __restrict__ V4 = (const V*)p.V4;
     const uint32_t lt = (1u << lane) - 1u;
     const int Hp = p.H + 1;
-    const int64_t items = (int64_t)p.L * p.parts;
+    int64_t items = (int64_t)p.L * p.parts;
+    int share = 1;                                         // warps that share a rest while some would have none
+    if constexpr (REST) {
+        items = min(p.cnt->pair_rest[0], (unsigned)p.rest_cap);
+        while (share < kPRest && items * share < (int64_t)gridDim.x * blockDim.x / 32) share *= 2;
+        items *= share;
+    }
 
     while (true) {
         unsigned int item = 0u;
-        if (lane == 0) item = atomicAdd(&p.cnt->work[1], 1u);
+        if (lane == 0) item = atomicAdd(REST ? &p.cnt->pair_rest[1] : &p.cnt->work[1], 1u);
         item = __shfl_sync(FULL, item, 0);
         if ((int64_t)item >= items) break;
-        const int leaf = (int)(item / (unsigned)p.parts);
-        const int part = (int)(item & (unsigned)(p.parts - 1));
+        // (leaf, part | runs before << 8, first candidate leaf, accepted leaves before it)
+        int4 it = make_int4(0, 0, 0, 0);
+        if constexpr (REST) it = p.rest[item / (unsigned)share];
+        const int leaf = REST ? it.x : (int)(item / (unsigned)p.parts);
+        const int part = REST ? it.y & 255 : (int)(item & (unsigned)(p.parts - 1));
+        int run = REST ? -(it.y >> 8) : 0;                 // below 0: a run before the rest's
+        bool whole = false;
         const int h = p.leaf_halo[leaf];
         const int leaf0 = p.leaf_off[h];
         const int A = leaf - leaf0;
@@ -885,7 +909,9 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
         // Consecutive particles of the Morton curve can lie far apart (on the sparse
         // outer shell on opposite sides of the halo), and boxes around them would
         // reach most of it: the queries are taken in runs of lanes whose box is at
-        // most kPSpread times their largest h wide (nearly always one run)
+        // most kPSpread times their largest h wide (nearly always one run).  A leaf no
+        // wider than two of the cells that order it is taken whole: in a core denser
+        // than the cells, leaves lie on one another, and each run would load them all
         uint32_t todo = __ballot_sync(FULL, active);
         while (todo) {
         bool act = (todo >> lane) & 1u;
@@ -907,7 +933,8 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
                 return fmaxf(fmaxf(-w[3] - w[0], -w[4] - w[1]), -w[5] - w[2]) > kPSpread * -w[6];
             };
             box();
-            if (wide()) {                                    // the same in every lane
+            if (run == 0) whole = fmaxf(fmaxf(-w[3] - w[0], -w[4] - w[1]), -w[5] - w[2]) <= 2.f * p.frame[h].fine;
+            if (!whole && wide()) {                          // the same in every lane
                 // boxes of the lanes up to this one: the run ends before the first that is too wide
 #pragma unroll
                 for (int i = 0; i < 7; ++i) w[i] = v[i];
@@ -923,6 +950,7 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
                 box();
             }
             todo &= ~__ballot_sync(FULL, act);
+            if (REST && run < 0) { ++run; continue; }
             float f[6] = {act ? q.x : INFINITY,  act ? q.y : INFINITY,  act ? q.z : INFINITY,
                           act ? -q.x : INFINITY, act ? -q.y : INFINITY, act ? -q.z : INFINITY};
 #pragma unroll
@@ -954,18 +982,22 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
         // visited iff the queries' box comes within (h + hmax_child)(1 + 2^-20) +
         // margin of the child's box, h the queries' largest, and its subtree holds a
         // leaf >= A
-        int nl = 0, seen = 0, sp = 0;
+        int nl = 0, seen = REST ? it.w : 0, sp = 0;
+        const int from = REST ? max(A, it.z) : A;          // the first leaf of this walk
+        it.z = it.w = 0;                                   // later runs start anew
         bool failed = false;
         auto visit = [&](int lev, int first, int base, int n) {
             float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
-            const bool in = lane < n && ((int64_t)(first + lane + 1) << (kArityLog * lev)) > (int64_t)A;
+            const bool in = lane < n && ((int64_t)(first + lane + 1) << (kArityLog * lev)) > (int64_t)from;
             if (in) { lo = p.nlo[base + first + lane]; hi = p.nhi[base + first + lane]; }
             const float4 qhi = wbox[1];
             const float r = __fadd_ru(__fmul_ru(__fadd_ru(qhi.w, lo.w), 1.0f + 0x1p-20f), margin);
             const bool ok = box_gap2_rd(wbox[0], qhi, lo, hi) <= __fmul_ru(r, r);
             uint32_t acc = __ballot_sync(FULL, in && ok);
             if (lev == 0) {
-                const bool mine = ((acc >> lane) & 1u) && ((seen + __popc(acc & lt)) & (p.parts - 1)) == part;
+                const int no = seen + __popc(acc & lt);
+                const bool mine = ((acc >> lane) & 1u) && (no & (p.parts - 1)) == part &&
+                                  (!REST || ((unsigned)(no >> p.parts_log) & (share - 1)) == (item & (share - 1)));
                 seen += __popc(acc);
                 acc = __ballot_sync(FULL, mine);
                 if (mine) list[nl + __popc(acc & lt)] = first + lane;
@@ -1042,6 +1074,17 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
                 n_tiles += min(2, nl - li);
                 li += 2;
                 __syncwarp();
+            } else if (!REST && sp > 0 && n_tiles > kPTiles && p.rest_cap > 0 && !failed) {
+                // the rest of this walk (the unvisited leaves are those from the stack's
+                // top node on) and the later runs go to the second launch
+                const int e = stack[sp - 1];
+                unsigned int slot = 0u;
+                if (lane == 0) slot = atomicAdd(&p.cnt->pair_rest[0], 1u);
+                slot = __shfl_sync(FULL, slot, 0);
+                if (slot >= (unsigned)p.rest_cap) { raise_status(p.cnt, SIDM_DEV_STACK); break; }   // cannot happen: one per item
+                if (lane == 0) p.rest[slot] = make_int4(leaf, part | (run << 8), (e & 0xFFFFFF) << (kArityLog * (e >> 24)), seen);
+                sp = 0;
+                todo = 0u;
             } else if (sp > 0 && !failed) {
                 // walk until the list may not hold another node's leaves, or the tree is done
                 nl = li = 0;
@@ -1177,6 +1220,7 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
             if (fin) break;
         }
         if (failed && lane == 0) raise_status(p.cnt, SIDM_DEV_STACK);
+        ++run;
         }   // runs of queries
         // this leaf's counts into the warp's 64-bit statistics
         {
@@ -1279,10 +1323,10 @@ int launch_all(sidm_ctx* c, uint64_t seed, uint64_t step, const sidm_xs* xs, con
 
 // With few query leaves each is shared by several warps (a
 // power of two, at most kPartsMax), so that every resident warp has about
-// kPartsPerWarp items: the last wave stays short, at the price of the walk that
-// the parts repeat.
+// N_ngb / 16 items, 2 to 4: the last wave stays short, at the price of the walk that
+// the parts repeat, which weighs more the fewer neighbours there are (N_ngb = 16,
+// 100,000 uniform particles: 147 us with 4 parts, 181 with 8; Hernquist 179, 230).
 constexpr int kPartsMax = 16;
-constexpr int64_t kPartsPerWarp = 4;
 template <class R, int PR, bool DRAG>
 int launch_draws(sidm_ctx* c, uint64_t seed, uint64_t step, const sidm_xs* xs, const double* dt, const double* mass,
                  const void* vel, sidm_step_stats* st, cudaStream_t s)
@@ -1292,12 +1336,22 @@ int launch_draws(sidm_ctx* c, uint64_t seed, uint64_t step, const sidm_xs* xs, c
     const LayoutHost& L = c->lay;
     const int warps = c->pair_warps;
     const size_t smem = (size_t)warps * draw_warp_bytes();
-    auto kern = k_pairs<R, PR, DRAG>;
+    auto kern = k_pairs<R, PR, DRAG, false>;
+    auto kern_rest = k_pairs<R, DRAG ? 1 : kPerRoundDefault, DRAG, true>;   // the groups drawn together change no result
     int occ = 0;
     if (int rc = occupancy(c, (const void*)kern, warps * 32, smem, &occ)) return rc;
     if (occ < 1) return set_err(c, SIDM_ECAPACITY, "pair kernel does not fit on an SM");
     int grid = c->cfg.grid_ctas > 0 ? c->cfg.grid_ctas : c->sm_count * occ;
-    while (p.parts < kPartsMax && (int64_t)L.L * p.parts < kPartsPerWarp * grid * warps) p.parts *= 2;
+    // (four, too, where a warp's kPTiles leaves are much of the halo)
+    const int64_t want = (int64_t)(L.L < 2 * (int)kPTiles ? 4 : std::max(2, std::min(4, c->kmax_cur / 16))) * grid * warps;
+    while (p.parts < kPartsMax && (int64_t)L.L * p.parts < want) { p.parts *= 2; ++p.parts_log; }
+    int rest_occ = 0;
+    if (int rc = occupancy(c, (const void*)kern_rest, warps * 32, smem, &rest_occ)) return rc;
+    if (rest_occ < 1) return set_err(c, SIDM_ECAPACITY, "pair kernel does not fit on an SM");
+    const int rest_grid = std::max(1, c->cfg.grid_ctas > 0 ? c->cfg.grid_ctas : c->sm_count * rest_occ);
+    p.rest = c->d_pair_rest;
+    // a halo of few leaves has no warp that wants so many; every item may leave one rest
+    p.rest_cap = L.L > (int)kPTiles && (int64_t)L.L * p.parts <= c->pair_rest_cap ? c->pair_rest_cap : 0;
     grid = (int)std::max<int64_t>(1, std::min<int64_t>(grid, ((int64_t)L.L * p.parts + warps - 1) / warps));
     c->pair_grid = grid;
     cudaError_t e = cudaMemsetAsync(&c->d_cnt->work[1], 0, sizeof(unsigned int), s);
@@ -1309,8 +1363,12 @@ int launch_draws(sidm_ctx* c, uint64_t seed, uint64_t step, const sidm_xs* xs, c
     }
     const int tidx = timer_begin(c, 2, s);
     kern<<<grid, warps * 32, smem, s>>>(p);
-    timer_end(c, tidx, s);
     c->launches++;
+    if (p.rest_cap > 0) {
+        kern_rest<<<rest_grid, warps * 32, smem, s>>>(p);
+        c->launches++;
+    }
+    timer_end(c, tidx, s);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_check(c, e, "pair launch");
     return SIDM_OK;
