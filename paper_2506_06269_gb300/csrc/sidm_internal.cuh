@@ -333,12 +333,24 @@ __device__ __forceinline__ bool lambda_stencil(float d, float hi, float hj, floa
     return true;
 }
 
-// FP32 interpolated f, from the table
+// FP32 interpolated f, from the table (written out: through lambda_stencil the
+// compiler spills 80 bytes instead of 4 in the kernel that forms every P)
 __device__ __forceinline__ float lambda_f_fast(const float* __restrict__ T, float d, float hi, float hj, float inv)
 {
-    int ix, ir;
+    const float hmin = fminf(hi, hj);
+    float x = __fdividef(d, hi + hj);
+    if (!(x < 1.f)) return 0.f;
+    x = fmaxf(x, 0.f);
+    const float rho = hmin * inv;
+    const float gx = x * (float)(kLamNX - 1);
+    int ix = (int)floorf(gx) - 1;
+    ix = ix < 0 ? 0 : (ix > kLamNX - 4 ? kLamNX - 4 : ix);
+    const float gr = rho * (float)(kLamNR - 1);
+    int ir = (int)floorf(gr) - 1;
+    ir = ir < 0 ? 0 : (ir > kLamNR - 4 ? kLamNR - 4 : ir);
     float wx[4], wr[4];
-    if (!lambda_stencil(d, hi, hj, inv, ix, ir, wx, wr)) return 0.f;
+    lagrange4<float>(gx - (float)ix, wx);
+    lagrange4<float>(gr - (float)ir, wr);
     float f = 0.f;
 #pragma unroll
     for (int a = 0; a < 4; ++a) {
