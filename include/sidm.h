@@ -93,9 +93,9 @@ typedef struct {
     float   knn_slack;   /*   warm-start bound / previous kernel size, 1..2 (1.07)   */
     int32_t pair_per_round; /* pair kernel: groups of 32 pairs drawn together, 1..4 (2; plain draws) */
     int32_t knn_batch;   /* kernel-size search: 1 loops over each staged leaf's      */
-                         /*   candidates, 2 over compacted batches of them, 3 as 2    */
-                         /*   with warm-started searches in the fixed-bound kernel    */
-                         /*   (default 3; bulk copies and neighbour lists take 1)     */
+                         /*   candidates, 2 over compacted batches of them, 3 takes   */
+                         /*   the fixed-bound kernel, lists too, and 2 for what it    */
+                         /*   hands on (default 3; bulk copies take 1)                */
 } sidm_config;
 
 /* Cross-section per unit mass of one halo (Sect. 3.8, Eq. vel_dep), given as
@@ -162,7 +162,7 @@ typedef struct {
                                   /* (FP64, exact fixed-point accumulation)       */
     float max_sum_p;              /* max_i sum_j P_ij (SIDM_FLAG_SUM_P only)      */
     float pad_;
-    unsigned long long n_tested;  /* candidate pairs given the in-range test      */
+    unsigned long long n_tested;  /* candidate pairs given the in-range test, each once */
 } sidm_step_stats;
 
 /* One accepted scatter event, as kept for the current step. */
@@ -302,8 +302,9 @@ int sidm_get_sum_p(sidm_ctx* ctx, float* out_dev, cudaStream_t stream);
 int64_t sidm_launch_count(const sidm_ctx* ctx);
 
 /* Device time of the hot kernels, measured with CUDA events recorded on the
- * launching stream around each launch (contexts created with
- * SIDM_FLAG_TIMING; at most 4096 launches are recorded between resets).
+ * launching stream around each launch, or a launch and the one that takes up
+ * what it leaves (contexts created with SIDM_FLAG_TIMING; at most 4096 are
+ * recorded between resets).
  *   ms_out[4]    : milliseconds of {cell build (whole a0 sequence), kernel-size
  *                  kernel, pair kernel, resolve kernel} since the last reset
  *   count_out[4] : launches recorded per slot (may be NULL)
@@ -325,9 +326,9 @@ int sidm_kernel_times(sidm_ctx* ctx, double* ms_out, int64_t* count_out, int32_t
 int sidm_diagnostics(sidm_ctx* ctx, uint64_t* out, int32_t reset);
 
 /* Local diagnostics of every particle (Sect. 3.5 Eq. hDl, Sect. 3.6
- * Eq. knudsen_number, App. C Eq. effective_cross_section), from one traversal
- * of the in-range pairs fused with the kernel sums (no draws, no velocity
- * change):
+ * Eq. knudsen_number, App. C Eq. effective_cross_section), from one search per
+ * particle inside its kernel (FP64 form: one traversal of the in-range pairs);
+ * no draws, no velocity change:
  *   rho_i = sum over j with d_ij < h_i, i itself included, of m W(d_ij, h_i)
  *           (SPH density over the particle's own kernel);
  *   nu_i  = 1-D velocity dispersion of the same kernel-weighted moments,
@@ -344,9 +345,9 @@ int sidm_diagnostics(sidm_ctx* ctx, uint64_t* out, int32_t reset);
  *   out_dev  : out, f32 (SIDM_MIXED) or f64 (SIDM_FP64) [5][N]: rho, nu,
  *              sigma_eff/m, h/l, Kn, in the order left by sidm_build_cells
  * Requires SIDM_FLAG_LOCAL_DIAG at creation and a preceding
- * sidm_kernel_sizes; uses the kernel sizes and N_ngb of that call.  The
- * moments are summed with FP64 atomics, so the last bits of rho and nu may
- * differ between runs. */
+ * sidm_kernel_sizes; uses the kernel sizes and N_ngb of that call.  In the
+ * FP64 form the moments are summed with FP64 atomics, so the last bits of rho
+ * and nu may differ between runs there. */
 int sidm_local_diagnostics(sidm_ctx* ctx, const sidm_xs* xs_dev, const double* mass_dev, const void* vel_dev,
                            double G, void* out_dev, cudaStream_t stream);
 
@@ -424,7 +425,7 @@ int sidm_timestep_criterion(sidm_ctx* ctx, double tau, double dt_min, double dt_
  * every case -- a stale or wrong guess costs time, never accuracy -- so this
  * is the usual SPH practice of starting from the previous smoothing length
  * (Sect. 2: h follows the N_ngb nearest neighbours as particles move).
- *   enable : 0 disables it (every search starts cold), non-zero enables it
+ *   enable : 0 disables it (every search starts without them), non-zero enables it
  * Host-only; takes effect at the next sidm_build_cells. */
 int sidm_warm_start(sidm_ctx* ctx, int32_t enable);
 

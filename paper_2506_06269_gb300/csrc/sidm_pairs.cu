@@ -614,8 +614,8 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_pairs_all(PairP
 // only pairs whose draw can fire take FP64 arithmetic.  2^20 NFW halo: 2.8 ms
 // per launch against 39 ms with every test and P on the FP64 pipe, 16384
 // particles 0.13 against 1.30 ms.
-// Issue-bound (2.8 of 4 instructions per cycle): mixed form 1.94 ms per launch for the 2^20
-// NFW halo at N_ngb = 64 (3.28 ms before), 2.65e8 in-range pairs, 1.24e9 tests.
+// Issue-bound (2.9 of 4 instructions per cycle): mixed form 1.95 ms for the 2^20
+// NFW halo at N_ngb = 64 (3.28 ms before), 2.65e8 in-range pairs, 1.16e9 tests.
 // Filling the queue in rounds of ballots and forming sigma(v) and
 // a bound of P for every pair, with masked tests, took 331 lane instructions
 // per in-range pair (52 % of them queueing and masks); a queue per lane, without
