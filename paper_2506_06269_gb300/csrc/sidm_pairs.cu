@@ -706,7 +706,6 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
         const int leaf = REST ? it.x : (int)(item / (unsigned)p.parts);
         const int part = REST ? it.y & 255 : (int)(item & (unsigned)(p.parts - 1));
         int run = REST ? -(it.y >> 8) : 0;                 // below 0: a run before the rest's
-        bool whole = false;
         const int h = p.leaf_halo[leaf];
         const int leaf0 = p.leaf_off[h];
         const int A = leaf - leaf0;
@@ -909,9 +908,11 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
         // Consecutive particles of the Morton curve can lie far apart (on the sparse
         // outer shell on opposite sides of the halo), and boxes around them would
         // reach most of it: the queries are taken in runs of lanes whose box is at
-        // most kPSpread times their largest h wide (nearly always one run).  A leaf no
-        // wider than two of the cells that order it is taken whole: in a core denser
-        // than the cells, leaves lie on one another, and each run would load them all
+        // most kPSpread times their largest h wide (nearly always one run).  Lanes no
+        // wider apart than two of the cells that order them are not split: in a core
+        // denser than the cells, leaves lie on one another, and each run would load them
+        // all.  The runs follow from the lanes left alone, so that both launches cut
+        // them alike
         uint32_t todo = __ballot_sync(FULL, active);
         while (todo) {
         bool act = (todo >> lane) & 1u;
@@ -933,7 +934,7 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
                 return fmaxf(fmaxf(-w[3] - w[0], -w[4] - w[1]), -w[5] - w[2]) > kPSpread * -w[6];
             };
             box();
-            if (run == 0) whole = fmaxf(fmaxf(-w[3] - w[0], -w[4] - w[1]), -w[5] - w[2]) <= 2.f * p.frame[h].fine;
+            const bool whole = fmaxf(fmaxf(-w[3] - w[0], -w[4] - w[1]), -w[5] - w[2]) <= 2.f * p.frame[h].fine;
             if (!whole && wide()) {                          // the same in every lane
                 // boxes of the lanes up to this one: the run ends before the first that is too wide
 #pragma unroll

@@ -47,7 +47,7 @@ def _positions(kind, n):
     return ics.hernquist(n, 3).pos
 
 
-CASES = [("core", 60000, 16), ("core", 40000, 100), ("cusp", 50000, 24), ("two", 60000, 32), ("clumps", 40000, 48),
+CASES = [("core", 60000, 16), ("core", 40000, 100), ("core", 200000, 16), ("cusp", 300000, 16), ("two", 400000, 32), ("cusp", 50000, 24), ("two", 60000, 32), ("clumps", 40000, 48),
          ("hernquist", 120000, 128)]
 
 
