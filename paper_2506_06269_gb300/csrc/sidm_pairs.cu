@@ -636,7 +636,11 @@ constexpr float kPSpread = 3.0f;   // widest box of a run of queries / its large
 // particles 1.39 ms (2.08 without; 1.87 with 1024), 400,000 1.92 (5.66; 2.05).  256
 // leaves rests to ordinary warps of the 64-halo batch (72 against 50 ms).
 constexpr uint32_t kPTiles = 512;
-constexpr int kPRest = 32;         // warps that share such a rest at most (a power of two)
+// Warps that share such a rest, at least and at most (powers of two): beside many short
+// rests there can be a long one, so every rest is cut.  At least 1, 4, 8, 16: a core of
+// 400,000 particles within six cells, with outliers, N_ngb = 16, 11.7, 6.9, 4.6, 3.5 ms,
+// a dense halo beside a wide one 18.8, 8.1, 6.3, 6.4; ordinary halos alike.
+constexpr int kPRestMin = 16, kPRest = 32;
 static_assert((kPRing & (kPRing - 1)) == 0 && kPRing >= kPBatch - 1 + 2 * kLeaf, "the ring holds a batch's leftover plus two leaves");
 static_assert(kPCand == 256, "a queued pair is (query lane << 8 | candidate mod 256)");
 
@@ -688,7 +692,7 @@ __global__ void __launch_bounds__(256, 3) k_pairs(PairParams p)
     const uint32_t lt = (1u << lane) - 1u;
     const int Hp = p.H + 1;
     int64_t items = (int64_t)p.L * p.parts;
-    int share = 1;                                         // warps that share a rest while some would have none
+    int share = kPRestMin;                                 // warps that share a rest: more while some would have none
     if constexpr (REST) {
         items = min(p.cnt->pair_rest[0], (unsigned)p.rest_cap);
         while (share < kPRest && items * share < (int64_t)gridDim.x * blockDim.x / 32) share *= 2;
